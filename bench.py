@@ -251,7 +251,7 @@ def kernel_source_hash() -> str:
 
 
 # Sources that define the compute-bound legs' kernels and their launch shapes.
-PIPE_SOURCES = ("ci_device.cuh", "ci_gen.cuh", "ci_gen_bbs.cu", "ci_gen_bbs16.cu", "ci_gen_xor128.cu",
+PIPE_SOURCES = ("ci_device.cuh", "ci_crt.cuh", "ci_gen.cuh", "ci_gen_bbs.cu", "ci_gen_bbs16.cu", "ci_gen_xor128.cu",
                 "ci_gen_xor64.cu", "ci_gen_xs32.cu", "ci_split.cu", "ci_split.h", "ci_bg.cu", "ci_modarith.cuh",
                 "ci_naive.cu", "ci_internal.h", "ci_kernels.cu", "ci_tune.cu", "ci_tune.h")
 

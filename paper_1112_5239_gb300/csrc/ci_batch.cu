@@ -42,8 +42,13 @@ __device__ __forceinline__ void run_sink(const BatchTask &T, uint64_t g, uint4 *
 // Persistent: every warp loops claiming one unit at a time from the cursor
 // until the queue is empty.  Units are handed out in queue order, and the
 // host orders tasks longest-first, so long serial chains start early.
+// Resident warps per SM asked of the register allocator: 128 registers.  (The
+// 300 requests of mixed sizes: 4.52 ms; 24 warps and 85 registers 5.29, 32 and
+// 64 registers 5.77, spilling in the generators' loops.)
+constexpr int kBatchWarps = 16;
+
 template <int WARPS>
-__global__ void __launch_bounds__(WARPS * 32) k_batched(BatchHeader *hdr, const BatchTask *tasks) {
+__global__ void __launch_bounds__(WARPS * 32, kBatchWarps / WARPS) k_batched(BatchHeader *hdr, const BatchTask *tasks) {
     __shared__ uint4 tiles[WARPS][256];
     const int lane = threadIdx.x & 31;
     uint4 *tile = tiles[threadIdx.x >> 5];

@@ -18,26 +18,30 @@
 // row.  The squarings use the Barrett reduction of the BBS strategy source
 // (modulus odd, below 2^62), which keeps x_i canonical so its low bits are
 // read directly; a warp whose moduli all have at least 34 bits takes its
-// limb form.
+// limb form.  Decryption knows the factors: a warp whose factors all lie in
+// (2^30, 2^31) squares their residues instead (ci_crt.cuh), starting from the
+// two square roots, and never forms x_0 (2^18 x 1024: 390 us against 578 in
+// the 62-bit form).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <mutex>
 
+#include "ci_crt.cuh"
 #include "ci_device.cuh"
 #include "ci_internal.h"
-#include "ci_trace.h"
 #include "ci_modarith.cuh"
+#include "ci_trace.h"
 
 namespace ci {
 namespace {
 
 using namespace dev;
 
-#ifndef CI_BG_MIN_BLOCKS
-#define CI_BG_MIN_BLOCKS 6  // resident blocks per SM asked of the register allocator: 40 registers,
-                            // no spills (measured: 6 and 8 equal, 4 slower for decryption)
-#endif
+// Resident blocks per SM asked of the register allocator: 64 registers, no
+// spills (2^18 x 1024: decryption 390 us, 398 with 5 blocks, 422 with 6;
+// encryption 437, 446 and 454).
+constexpr int kBgMinBlocks = 4;
 
 constexpr int kBgWarps = 8;    // warps per block
 constexpr int kBgTile = 32;    // chunks per staged row
@@ -49,54 +53,71 @@ __device__ __forceinline__ uint32_t bg_w(uint64_t N) {
     return lg ? 31u - (uint32_t)__clz((int)lg) : 0u;             // floor(log2 lg)
 }
 
-// One chunk: b = x_i & mask (x_i canonical), key ^= b, x_{i+1} = x_i^2.
-// kLimb: the limb-form square (every modulus of the warp has 34..62 bits).
-struct BgLane {
+// The keystream of one message: draw() returns b = x_i & mask (x_i canonical)
+// and takes x_{i+1} = x_i^2.  One form per way of squaring.
+template <bool kLimb>  // 62-bit Barrett; kLimb: every modulus of the warp has 34..62 bits
+struct BgBarrett {
     Barrett62 B;
     uint64_t x;
     uint32_t mask, key;
-    template <bool kLimb>
-    __device__ __forceinline__ uint64_t sqr(uint64_t v) const {
-        return kLimb ? B.sqr_limb(v) : B.sqr(v);
+    __device__ __forceinline__ uint32_t draw() {
+        const uint32_t b = (uint32_t)x & mask;
+        x = kLimb ? B.sqr_limb(x) : B.sqr(x);
+        return b;
     }
-    template <bool kLimb>
-    __device__ __forceinline__ uint32_t chunk(uint32_t v) {
-        key ^= (uint32_t)x & mask;
-        x = sqr<kLimb>(x);
-        return (v ^ key) & 0xFFu;
-    }
-    // Four chunks, one per byte of w: the keystream bytes are gathered into
-    // one word and XORed in once (key < 2^8: S^0 is a byte, the b_i have at
-    // most 5 bits).
-    template <bool kLimb>
-    __device__ __forceinline__ uint32_t word(uint32_t w) {
-        uint32_t ks = 0;
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            key ^= (uint32_t)x & mask;
-            x = sqr<kLimb>(x);
-            ks |= key << (8 * b);
-        }
-        return w ^ ks;
+};
+struct BgCrt {  // both factors known, in (2^30, 2^31)
+    CrtModulus C;
+    uint32_t rp, rq, mask, key;
+    __device__ __forceinline__ uint32_t draw() {
+        const uint32_t b = C.low(rp, rq) & mask;
+        rp = C.P.sqr(rp);
+        rq = C.Q.sqr(rq);
+        return b;
     }
 };
 
+// One chunk: key ^= b, c = m ^ key.
+template <class Lane>
+__device__ __forceinline__ uint32_t bg_chunk(Lane &s, uint32_t v) {
+    s.key ^= s.draw();
+    return (v ^ s.key) & 0xFFu;
+}
+// Four chunks, one per byte of w: the keystream bytes are gathered into one
+// word and XORed in once (key < 2^8: S^0 is a byte, the b_i have at most 5
+// bits).
+template <class Lane>
+__device__ __forceinline__ uint32_t bg_word(Lane &s, uint32_t w) {
+    uint32_t ks = 0;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        s.key ^= s.draw();
+        ks |= s.key << (8 * b);
+    }
+    return w ^ ks;
+}
+
 // Encryption key check: N odd, 3 <= N < 2^62 (the range of Barrett62).
-__device__ __forceinline__ bool bg_setup_encrypt(uint64_t N, uint64_t r, BgLane &s) {
+__device__ __forceinline__ bool bg_setup_encrypt(uint64_t N, uint64_t r, Barrett62 &B, uint64_t &x) {
     const bool ok = (N & 1ull) && N >= 3 && N < (1ull << 62);
     if (!ok) N = 3;
-    s.B.set(N, barrett_mu(N));
-    s.x = s.B.sqr(r % N);  // x_0 = r^2 mod N
+    B.set(N, barrett_mu(N));
+    x = B.sqr(r % N);  // x_0 = r^2 mod N
     return ok;
 }
 
 // Decryption key check: p != q, both prime, = 3 mod 4, below 2^32, p q < 2^62.
-// x_0 = the square root of y taken L times mod p and mod q, joined by
-// Garner's formula x_0 = r_p + p ((r_q - r_p) p^-1 mod q).
-__device__ __forceinline__ bool bg_setup_decrypt(uint64_t p, uint64_t q, uint64_t y, uint64_t L, BgLane &s) {
-    const bool ok = p < (1ull << 32) && q < (1ull << 32) && (p & 3ull) == 3 && (q & 3ull) == 3 && p != q &&
-                    p * q < (1ull << 62) && is_prime_u32(p) && is_prime_u32(q);
-    uint64_t x0 = 0, N = 3;
+// The residues of x_0, the square root of y taken L times mod p and mod q,
+// and p^-1 mod q for joining them (Garner: x_0 = r_p + p ((r_q - r_p) p^-1
+// mod q)); p < q on return.  A rejected key becomes a valid dummy pair.
+struct BgRoots {
+    uint32_t p, q, rp, rq, pinv;
+};
+__device__ __forceinline__ bool bg_setup_decrypt(uint64_t a, uint64_t b, uint64_t y, uint64_t L, BgRoots &s) {
+    const uint64_t p = a < b ? a : b, q = a < b ? b : a;
+    const bool ok = q < (1ull << 32) && (p & 3ull) == 3 && (q & 3ull) == 3 && p != q && p * q < (1ull << 62) &&
+                    is_prime_u32(p) && is_prime_u32(q);
+    s = BgRoots{(1u << 30) + 3u, (1u << 31) - 1u, 0u, 0u, 1u};
     if (ok) {
         const Barrett32 Bp1(p - 1), Bq1(q - 1);      // even moduli: Barrett
         const Mont32 Mp((uint32_t)p), Mq((uint32_t)q);  // odd primes: Montgomery
@@ -104,23 +125,18 @@ __device__ __forceinline__ bool bg_setup_decrypt(uint64_t p, uint64_t q, uint64_
         const uint64_t eq = Bq1.pow((q + 1) / 4, L);
         // y mod N < p q, below p 2^32 and q 2^32: taken to Montgomery form by REDC
         const uint64_t yN = y < p * q ? y : y % (p * q);
-        const uint32_t rp = Mp.from(Mp.pow_m(Mp.to_wide(yN), ep));
-        const uint32_t rq_m = Mq.pow_m(Mq.to_wide(yN), eq);  // Montgomery forms mod q from here
-        const uint32_t pinv_m = Mq.pow_m(Mq.to_any((uint32_t)p), q - 2);  // Fermat: p^(q-2) = p^-1 mod q
-        const uint32_t rp_m = Mq.to_any(rp);
-        const uint32_t diff_m = rq_m >= rp_m ? rq_m - rp_m : (uint32_t)((uint64_t)rq_m + q - rp_m);
-        const uint64_t t = Mq.from(Mq.mul(diff_m, pinv_m));  // (r_q - r_p) p^-1 mod q
-        x0 = rp + p * t;                              // < p + p (q - 1) = N
-        N = p * q;
+        s.p = (uint32_t)p;
+        s.q = (uint32_t)q;
+        s.rp = Mp.from(Mp.pow_m(Mp.to_wide(yN), ep));
+        s.rq = Mq.from(Mq.pow_m(Mq.to_wide(yN), eq));
+        s.pinv = Mq.from(Mq.pow_m(Mq.to((uint32_t)p), q - 2));  // Fermat: p^(q-2) = p^-1 mod q
     }
-    s.B.set(N, barrett_mu(N));
-    s.x = x0;
     return ok;
 }
 
 // The chunks of one warp's 32 messages (lane = message), after key setup.
-template <bool kVec, bool kLimb>
-__device__ __forceinline__ void bg_rows(BgLane &s, uint32_t keep, bool live, uint64_t msg, uint64_t m0,
+template <bool kVec, class Lane>
+__device__ __forceinline__ void bg_rows(Lane &s, uint32_t keep, bool live, uint64_t msg, uint64_t m0,
                                         uint32_t rows, uint64_t L, const uint8_t *in, uint8_t *out, uint8_t *tile,
                                         uint8_t *row, uint32_t lane) {
     if constexpr (kVec) {  // L a multiple of 32, rows 16-byte aligned
@@ -130,14 +146,14 @@ __device__ __forceinline__ void bg_rows(BgLane &s, uint32_t keep, bool live, uin
             const uint64_t steps = L / kBgTile;
             for (uint64_t t = 0; t < steps; ++t) {  // each step reads its 32 bytes before writing them
                 uint4 a = src[2 * t], b = src[2 * t + 1];
-                a.x = s.word<kLimb>(a.x) & keep;
-                a.y = s.word<kLimb>(a.y) & keep;
-                a.z = s.word<kLimb>(a.z) & keep;
-                a.w = s.word<kLimb>(a.w) & keep;
-                b.x = s.word<kLimb>(b.x) & keep;
-                b.y = s.word<kLimb>(b.y) & keep;
-                b.z = s.word<kLimb>(b.z) & keep;
-                b.w = s.word<kLimb>(b.w) & keep;
+                a.x = bg_word(s, a.x) & keep;
+                a.y = bg_word(s, a.y) & keep;
+                a.z = bg_word(s, a.z) & keep;
+                a.w = bg_word(s, a.w) & keep;
+                b.x = bg_word(s, b.x) & keep;
+                b.y = bg_word(s, b.y) & keep;
+                b.z = bg_word(s, b.z) & keep;
+                b.w = bg_word(s, b.w) & keep;
                 dst[2 * t] = a;
                 dst[2 * t + 1] = b;
             }
@@ -154,9 +170,9 @@ __device__ __forceinline__ void bg_rows(BgLane &s, uint32_t keep, bool live, uin
                 uint32_t *w = reinterpret_cast<uint32_t *>(row);
                 if (width == kBgTile) {
 #pragma unroll
-                    for (int j = 0; j < kBgTile / 4; ++j) w[j] = s.word<kLimb>(w[j]) & keep;
+                    for (int j = 0; j < kBgTile / 4; ++j) w[j] = bg_word(s, w[j]) & keep;
                 } else {
-                    for (uint32_t j = 0; j < width; ++j) row[j] = (uint8_t)(s.chunk<kLimb>(row[j]) & keep);
+                    for (uint32_t j = 0; j < width; ++j) row[j] = (uint8_t)(bg_chunk(s, row[j]) & keep);
                 }
             }
             __syncwarp();
@@ -168,7 +184,7 @@ __device__ __forceinline__ void bg_rows(BgLane &s, uint32_t keep, bool live, uin
 }
 
 template <bool kDecrypt, bool kVec>
-__global__ void __launch_bounds__(kBgWarps * 32, CI_BG_MIN_BLOCKS)
+__global__ void __launch_bounds__(kBgWarps * 32, kBgMinBlocks)
     k_bg(uint64_t n_msgs, uint64_t L, const uint64_t *__restrict__ key_a, const uint64_t *__restrict__ key_b,
          const uint8_t *__restrict__ S0, const uint64_t *__restrict__ y_in, const uint8_t *in, uint8_t *out,
          uint64_t *__restrict__ y_out, uint32_t *__restrict__ n_rejected) {
@@ -185,22 +201,53 @@ __global__ void __launch_bounds__(kBgWarps * 32, CI_BG_MIN_BLOCKS)
         const uint64_t msg = m0 + lane;
         const bool live = msg < n_msgs;
         const uint32_t rows = n_msgs - m0 < 32 ? (uint32_t)(n_msgs - m0) : 32u;
-        BgLane s;
+        uint32_t key = 0, mask = 0;
+        Barrett62 B;
+        uint64_t x = 0;
         bool ok = false;
-        if (live) {
-            ok = kDecrypt ? bg_setup_decrypt(key_a[msg], key_b[msg], y_in[msg], L, s)
-                          : bg_setup_encrypt(key_a[msg], key_b[msg], s);
-            s.mask = ok ? (1u << bg_w(s.B.M)) - 1u : 0u;
-            s.key = S0[msg];
-            if (!ok && n_rejected) atomicAdd(n_rejected, 1u);
+        if constexpr (kDecrypt) {
+            BgRoots k{(1u << 30) + 3u, (1u << 31) - 1u, 0u, 0u, 1u};  // dead lanes: the dummy pair
+            if (live) ok = bg_setup_decrypt(key_a[msg], key_b[msg], y_in[msg], L, k);
+            if (live) key = S0[msg];
+            if (live && !ok && n_rejected) atomicAdd(n_rejected, 1u);
+            const uint32_t keep = ok ? 0xFFFFFFFFu : 0u;  // a rejected key's row is written as zeros
+            mask = ok ? (1u << bg_w((uint64_t)k.p * k.q)) - 1u : 0u;
+            // the same in every lane: the branches never diverge
+            if (__all_sync(0xFFFFFFFFu, k.p > (1u << 30) && k.q < (1u << 31))) {
+                BgCrt s;
+                s.C.set_inverse(k.p, k.q, k.pinv);
+                s.rp = k.rp;
+                s.rq = k.rq;
+                s.mask = mask;
+                s.key = key;
+                bg_rows<kVec>(s, keep, live, msg, m0, rows, L, in, out, tile, row, lane);
+                continue;
+            }
+            // x_0 by Garner; p < q, so r_p < q
+            const Mont32 Mq(k.q);
+            const uint32_t diff = k.rq >= k.rp ? k.rq - k.rp : k.rq + (k.q - k.rp);
+            x = k.rp + (uint64_t)k.p * Mq.mul(Mq.to(diff), k.pinv);  // < p + p (q - 1) = N
+            B.set((uint64_t)k.p * k.q, barrett_mu((uint64_t)k.p * k.q));
+        } else {
+            B.set(3, barrett_mu(3));
+            if (live) {
+                ok = bg_setup_encrypt(key_a[msg], key_b[msg], B, x);
+                mask = ok ? (1u << bg_w(B.M)) - 1u : 0u;
+                key = S0[msg];
+                if (!ok && n_rejected) atomicAdd(n_rejected, 1u);
+            }
         }
-        const uint32_t keep = ok ? 0xFFFFFFFFu : 0u;  // a rejected key's row is written as zeros
-        // the same in every lane: the branch never diverges
-        if (__all_sync(0xFFFFFFFFu, !live || s.B.M >= (1ull << 33)))
-            bg_rows<kVec, true>(s, keep, live, msg, m0, rows, L, in, out, tile, row, lane);
-        else
-            bg_rows<kVec, false>(s, keep, live, msg, m0, rows, L, in, out, tile, row, lane);
-        if (!kDecrypt && live) y_out[msg] = ok ? s.x : 0ull;
+        const uint32_t keep = ok ? 0xFFFFFFFFu : 0u;
+        if (__all_sync(0xFFFFFFFFu, !live || B.M >= (1ull << 33))) {
+            BgBarrett<true> s{B, x, mask, key};
+            bg_rows<kVec>(s, keep, live, msg, m0, rows, L, in, out, tile, row, lane);
+            x = s.x;
+        } else {
+            BgBarrett<false> s{B, x, mask, key};
+            bg_rows<kVec>(s, keep, live, msg, m0, rows, L, in, out, tile, row, lane);
+            x = s.x;
+        }
+        if (!kDecrypt && live) y_out[msg] = ok ? x : 0ull;
     }
 }
 

@@ -16,7 +16,9 @@
 #include <cuda.h>  // CUtensorMap (TMA descriptor type only)
 
 #include <cstdint>
+#include <type_traits>
 
+#include "ci_crt.cuh"
 #include "ci_internal.h"
 
 namespace ci {
@@ -58,10 +60,13 @@ __device__ __forceinline__ uint64_t lane_draw(uint64_t seed, uint64_t lane, uint
 // ------------------------------------------------------- strategy sources
 // Each source: load/store of its words for lane l, the pair of combination
 // arrays the lane uses, and next() returning the lane's own strategy word.
+// kHeavy: next() is long, the output loops are not unrolled; kOneStep: nor
+// are four steps written per turn (eleven squarings each would leave the
+// instruction cache).
 
 // 32-bit xor128 (Marsaglia), the xor-like the paper uses for Algorithm 4.
 struct SrcXor128 {
-    static constexpr bool kHeavy = false;
+    static constexpr bool kHeavy = false, kOneStep = false;
     uint32_t a, b, c, d;
     __device__ __forceinline__ void load(const DevState &s, uint64_t l) {
         a = s.u32[F_A * s.P + l];
@@ -91,7 +96,7 @@ struct SrcXor128 {
 
 // Algorithm 2: z ^= z << 13; z ^= z >> 17; z ^= z << 5.
 struct SrcXorshift32 {
-    static constexpr bool kHeavy = false;
+    static constexpr bool kHeavy = false, kOneStep = false;
     uint32_t z;
     __device__ __forceinline__ void load(const DevState &s, uint64_t l) { z = s.u32[F_A * s.P + l]; }
     __device__ __forceinline__ void store(const DevState &s, uint64_t l) const { s.u32[F_A * s.P + l] = z; }
@@ -110,7 +115,7 @@ struct SrcXorshift32 {
 // xor64, the 64-bit xorshift of the paper's Sec. 7 measurements; the lane's
 // strategy word is the low 32 bits of each step.
 struct SrcXor64 {
-    static constexpr bool kHeavy = false;
+    static constexpr bool kHeavy = false, kOneStep = false;
     uint64_t z;
     __device__ __forceinline__ void load(const DevState &s, uint64_t l) {
         z = (uint64_t)s.u32[F_A * s.P + l] | ((uint64_t)s.u32[F_B * s.P + l] << 32);
@@ -285,7 +290,7 @@ struct Barrett62 {
 // Blum Blum Shub strategy source (Algorithm 5 generalised to w = 5 bits per
 // squaring for 62-bit moduli): 7 chunks of 5 bits, then two shift steps.
 struct SrcBbs {
-    static constexpr bool kHeavy = true;
+    static constexpr bool kHeavy = true, kOneStep = true;
     Barrett62 B;
     uint64_t y;  // BBS state, canonical in [0, M)
     uint32_t sel;
@@ -325,6 +330,82 @@ struct SrcBbs {
     __device__ __forceinline__ uint32_t next() { return limb ? assemble<true>() : assemble<false>(); }
 };
 
+// The same source on the residues of the two factors (ci_crt.cuh), bound by
+// the FMA-heavy pipe as the 62-bit form is, but with 30 instead of 51 cycles
+// of it per squaring of a warp: 2^16 x 4096 outputs in 3.28 instead of 5.38
+// ms, 300 uneven requests in one launch 4.52 instead of 6.88 ms.  Its constants are computed from
+// the state's p and q when a warp's work starts, or read from `crt` (kCrtWords
+// fields of P words, written by crt_store) where a call prepares them once for
+// many units.  load() is false in every lane unless all lanes of the warp hold
+// factors the residue form takes (all seeded ones do; imported moduli may have
+// shorter factors, which keep the 62-bit form).
+constexpr int kCrtWords = 4;  // mu_p, mu_q, beta (0: not usable), beta_s
+
+struct SrcBbsCrt {
+    static constexpr bool kHeavy = true, kOneStep = true;
+    CrtModulus C;
+    uint32_t rp, rq, sel;
+    __device__ __forceinline__ bool load(const DevState &s, uint64_t l, const uint32_t *crt) {
+        const uint32_t a = s.u32[F_P * s.P + l], b = s.u32[F_Q * s.P + l];
+        bool ok;
+        if (crt) {
+            C.P.set(min(a, b), crt[l]);
+            C.Q.set(max(a, b), crt[s.P + l]);
+            C.beta = crt[2 * s.P + l];
+            C.beta_s = crt[3 * s.P + l];
+            ok = C.beta != 0u;
+        } else {
+            ok = C.set(a, b);
+        }
+        if (!__all_sync(kFull, ok)) return false;
+        const uint64_t y = s.u64[G_Y * s.P + l];
+        rp = (uint32_t)(y % C.P.p);
+        rq = (uint32_t)(y % C.Q.p);
+        sel = s.u32[F_SEL * s.P + l];
+        return true;
+    }
+    __device__ __forceinline__ void store(const DevState &s, uint64_t l) const {
+        s.u64[G_Y * s.P + l] = C.value(rp, rq);
+    }
+    __device__ __forceinline__ void arrays(const DevState &, uint64_t, int &a1, int &a2) const {
+        a1 = (int)(sel & 7u);
+        a2 = 8 + (int)((sel >> 8) & 7u);
+    }
+    // One BBS output: x <- x^2 mod M; the low word of x (its low bits are the secure ones).
+    __device__ __forceinline__ uint32_t bbs() {
+        rp = C.P.sqr(rp);
+        rq = C.Q.sqr(rq);
+        return C.low(rp, rq);
+    }
+    __device__ __forceinline__ uint32_t next() {
+        uint32_t t = 0;
+#pragma unroll
+        for (int c = 0; c < 7; ++c) t = (t << 5) | (bbs() & 31u);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const uint32_t shift = bbs() & 3u;
+            t <<= shift;
+            t |= bbs() & ((1u << shift) - 1u);  // array_shift = {0, 1, 3, 7}
+        }
+        return t;
+    }
+};
+
+// Lane l's residue constants, for SrcBbsCrt::load.
+__device__ __forceinline__ void crt_store(const DevState &s, uint64_t l, uint32_t *crt) {
+    CrtModulus C{};
+    const bool ok = C.set(s.u32[F_P * s.P + l], s.u32[F_Q * s.P + l]);
+    crt[l] = C.P.mu;
+    crt[s.P + l] = C.Q.mu;
+    crt[2 * s.P + l] = ok ? C.beta : 0u;
+    crt[3 * s.P + l] = C.beta_s;
+}
+
+// Shortest unit that takes the residue form when its constants have to be
+// computed first (2^16 streams, written: 12 outputs 21.3 us against 23.1 in
+// the 62-bit form, 16 outputs 25.2 against 29.2; 8 outputs 18.8 against 17.6).
+constexpr uint64_t kCrtMinLength = 12;
+
 // Algorithm 5 as printed: eight BBS generators per lane with moduli below
 // 2^16, so x^2 fits 32 bits.  x^2 mod M by Barrett reduction with
 // mu = floor(2^32 / M): q = mulhi(x^2, mu) is floor(x^2 / M) or one less, so a
@@ -333,7 +414,7 @@ struct SrcBbs {
 // arrays are read from BBS1 and BBS2 when the call starts; at the end of the
 // call generator k (state and modulus) is stored in place k + 1.
 struct SrcBbs16 {
-    static constexpr bool kHeavy = true;
+    static constexpr bool kHeavy = true, kOneStep = false;
     uint32_t y[8], M[8], mu[8];
     uint32_t sel1, sel2;
     __device__ __forceinline__ void load(const DevState &s, uint64_t l) {
@@ -464,19 +545,13 @@ __device__ __forceinline__ void store4(uint32_t *p, uint32_t v) {
 // D = sum_i x_i K^(n-1-i) mod 2^64, to counts[r].  `tile` is this warp's
 // 32 x TC::KT words of shared memory (written sinks).  SINK_V4 needs out, ld
 // and col0 aligned to 4 words.
-template <class Src, int SINK, class TC = TileDefault>
-__device__ __forceinline__ void warp_task(const DevState &st, uint64_t g, uint64_t n, uint32_t *out,
-                                          uint64_t ld, uint64_t col0, uint64_t *counts,
-                                          uint4 *tile) {
+template <class Src, int SINK, class TC>
+__device__ __forceinline__ void warp_loop(Src &src, const DevState &st, uint64_t g, uint64_t n, uint32_t *out,
+                                          uint64_t ld, uint64_t col0, uint64_t *counts, uint4 *tile) {
     constexpr int KT = (SINK == SINK_V4 || SINK == SINK_SCALAR) ? TC::KT : 32;
     constexpr int CH = KT / 4;
-    CI_WARP_CHECK(st, g < st.P / 32, CHK_GROUP, g);
-    if (SINK == SINK_V4 || SINK == SINK_SCALAR) CI_WARP_CHECK(st, col0 + n <= ld, CHK_COLS, col0 + n);
-    if (SINK == SINK_V4) CI_WARP_CHECK(st, (col0 | ld) % 4 == 0, CHK_V4_ALIGN, col0);
     const int lane = threadIdx.x & 31;
     const uint64_t l = g * 32 + lane;
-    Src src;
-    src.load(st, l);
     uint32_t x = st.u32[F_X * st.P + l];
     uint32_t slot = st.u32[F_SLOT * st.P + l];
     int a1, a2;
@@ -502,19 +577,24 @@ __device__ __forceinline__ void warp_task(const DevState &st, uint64_t g, uint64
             }
             hits += 16u - m;
         } else {
+            if (Src::kOneStep) {
+#pragma unroll 1
+                for (int k = 0; k < KT; ++k) tw[tile_word<KT>(lane, k)] = ci_step(src, x, slot, p1, p2);
+            } else {
 #pragma unroll(Src::kHeavy ? 1 : CH)
-            for (int q = 0; q < CH; ++q) {
-                uint4 v;
-                v.x = ci_step(src, x, slot, p1, p2);
-                v.y = ci_step(src, x, slot, p1, p2);
-                v.z = ci_step(src, x, slot, p1, p2);
-                v.w = ci_step(src, x, slot, p1, p2);
-                tile[lane * CH + (q ^ (lane & 7))] = v;
+                for (int q = 0; q < CH; ++q) {
+                    uint4 v;
+                    v.x = ci_step(src, x, slot, p1, p2);
+                    v.y = ci_step(src, x, slot, p1, p2);
+                    v.z = ci_step(src, x, slot, p1, p2);
+                    v.w = ci_step(src, x, slot, p1, p2);
+                    tile[lane * CH + (q ^ (lane & 7))] = v;
+                }
             }
             __syncwarp();
             if (SINK == SINK_V4) {
                 constexpr int RPI = 32 / CH;  // tile rows per warp-wide store
-#pragma unroll
+#pragma unroll(Src::kOneStep ? 2 : CH)
                 for (int k = 0; k < CH; ++k) {
                     const int r = RPI * k + lane / CH, c = lane % CH;
                     const uint4 v = tile[r * CH + (c ^ (r & 7))];
@@ -563,6 +643,28 @@ __device__ __forceinline__ void warp_task(const DevState &st, uint64_t g, uint64
     st.u32[F_SLOT * st.P + l] = slot;
     if (SINK == SINK_QC && l < st.S) counts[l] += hits;
     if (SINK == SINK_DIGEST && l < st.S) counts[l] = hits;
+}
+
+template <class Src, int SINK, class TC = TileDefault>
+__device__ __forceinline__ void warp_task(const DevState &st, uint64_t g, uint64_t n, uint32_t *out,
+                                          uint64_t ld, uint64_t col0, uint64_t *counts,
+                                          uint4 *tile, const uint32_t *crt = nullptr) {
+    CI_WARP_CHECK(st, g < st.P / 32, CHK_GROUP, g);
+    if (SINK == SINK_V4 || SINK == SINK_SCALAR) CI_WARP_CHECK(st, col0 + n <= ld, CHK_COLS, col0 + n);
+    if (SINK == SINK_V4) CI_WARP_CHECK(st, (col0 | ld) % 4 == 0, CHK_V4_ALIGN, col0);
+    const uint64_t l = g * 32 + (threadIdx.x & 31);
+    if constexpr (std::is_same<Src, SrcBbs>::value) {
+        if (crt || n >= kCrtMinLength) {
+            SrcBbsCrt c;
+            if (c.load(st, l, crt)) {  // the same in every lane
+                warp_loop<SrcBbsCrt, SINK, TC>(c, st, g, n, out, ld, col0, counts, tile);
+                return;
+            }
+        }
+    }
+    Src src;
+    src.load(st, l);
+    warp_loop<Src, SINK, TC>(src, st, g, n, out, ld, col0, counts, tile);
 }
 
 // ------------------------------------------------ TMA bulk tensor stores

@@ -244,14 +244,16 @@ __constant__ uint32_t c_bbs16_squarings[8] = {2, 2, 2, 1, 1, 1, 2, 1};
 
 // lambda(M) = lcm(p - 1, q - 1) of each lane's BBS modulus and its Barrett
 // reciprocal, once per lane (every segment's jump uses them):
-// lam[l] = lambda, lam[P + l] = barrett_mu(lambda).
-__global__ void __launch_bounds__(256) k_split_lambda(DevState src, uint64_t *lam) {
+// lam[l] = lambda, lam[P + l] = barrett_mu(lambda); likewise the constants of
+// the residue form (every segment's run uses them).
+__global__ void __launch_bounds__(256) k_split_lambda(DevState src, uint64_t *lam, uint32_t *crt) {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < src.P; l += stride) {
         const uint64_t p = src.u32[F_P * src.P + l], q = src.u32[F_Q * src.P + l];
         const uint64_t v = (p - 1) / gcd64(p - 1, q - 1) * (q - 1);
         lam[l] = v;
         lam[src.P + l] = barrett_mu(v);
+        crt_store(src, l, crt);
     }
 }
 
@@ -688,21 +690,23 @@ constexpr uint64_t kOneLaunchGroupsPerSm = CI_ONE_LAUNCH_GROUPS_PER_SM;
 // segment state with that index.
 // Instantiated per source and sink, with at most 64 registers (4 blocks of 8
 // warps per SM): the all-source batched kernel needs 128, which held the
-// BBS segments to 16 resident warps per SM.  BBS segments (one serial
-// squaring chain per lane) ask for 5 blocks, i.e. 48 registers; segments of
-// Algorithm 5 as printed (eight generators per lane, 118 registers in the
-// single-call kernel) for 2 blocks, 128 registers, so that their loop does
-// not spill.
+// BBS segments to 16 resident warps per SM.  BBS segments ask for 3 blocks, 80
+// registers: the residue form's constants fit without spills, and its two
+// independent chains per lane fill the pipes from 24 warps per SM on
+// (2^16 x 4096: 3.28 ms; 3.50 with 4 blocks, 3.95 with 5, 3.39 with 2;
+// 5.38 in the 62-bit form with 5).  Segments of Algorithm 5 as printed (eight
+// generators per lane, 118 registers in the single-call kernel) ask for 2
+// blocks, 128 registers, so that their loop does not spill.
 template <class Src>
 constexpr int split_min_blocks() {
-    return std::is_same<Src, SrcBbs>::value ? 5 : std::is_same<Src, SrcBbs16Seg>::value ? 2 : 4;
+    return std::is_same<Src, SrcBbs>::value ? 3 : std::is_same<Src, SrcBbs16Seg>::value ? 2 : 4;
 }
 
 template <class Src, int SINK>
 __global__ void __launch_bounds__(256, split_min_blocks<Src>()) k_split_run(SegSpace seg, DevState caller, int zero, uint32_t k_begin,
                                                    uint32_t k_end, uint32_t K, uint64_t len, uint64_t len_last,
                                                    uint64_t groups, uint32_t *out, uint64_t ld, uint64_t col0,
-                                                   uint64_t *aux) {
+                                                   uint64_t *aux, const uint32_t *crt) {
     __shared__ uint4 tiles[8][256];
     uint4 *tile = tiles[threadIdx.x >> 5];
     const uint64_t units = (uint64_t)(k_end - k_begin) * groups;
@@ -714,16 +718,16 @@ __global__ void __launch_bounds__(256, split_min_blocks<Src>()) k_split_run(SegS
         const DevState st = k != 0 ? seg.at(k) : zero < 0 ? caller : seg.at((uint64_t)zero);
         const uint64_t n = k + 1 == K ? len_last : len;
         if (SINK == SINK_V4 || SINK == SINK_SCALAR)
-            warp_task<Src, SINK>(st, g, n, out, ld, col0 + k * len, nullptr, tile);
+            warp_task<Src, SINK>(st, g, n, out, ld, col0 + k * len, nullptr, tile, crt);
         else
-            warp_task<Src, SINK>(st, g, n, nullptr, 0, 0, aux + k * caller.P, tile);
+            warp_task<Src, SINK>(st, g, n, nullptr, 0, 0, aux + k * caller.P, tile, crt);
     }
 }
 
 template <class Src, int SINK>
 cudaError_t launch_split_run(const SegSpace &sp, const DevState &caller, int zero, uint32_t kb, uint32_t ke,
                              uint32_t K, uint64_t len, uint64_t len_last, uint32_t *out, uint64_t ld, uint64_t col0,
-                             uint64_t *aux, cudaStream_t stream) {
+                             uint64_t *aux, const uint32_t *crt, cudaStream_t stream) {
     static int per_sm = 0;
     static std::once_flag once;
     std::call_once(once, [] {
@@ -734,7 +738,7 @@ cudaError_t launch_split_run(const SegSpace &sp, const DevState &caller, int zer
     if (units == 0) return cudaSuccess;
     const int blocks = (int)std::min<uint64_t>(units, (uint64_t)sm_count() * per_sm);  // a block per unit at most
     k_split_run<Src, SINK><<<blocks, 256, 0, stream>>>(sp, caller, zero, kb, ke, K, len, len_last, groups, out, ld,
-                                                       col0, aux);
+                                                       col0, aux, crt);
     return cudaGetLastError();
 }
 
@@ -769,7 +773,7 @@ template <class Src, int SINK>
 __global__ void __launch_bounds__(256, split_min_blocks<Src>()) k_split_run_fix(SegSpace seg, uint32_t K, uint64_t len,
                                                        uint64_t len_last, uint64_t groups, uint32_t *out, uint64_t ld,
                                                        uint64_t col0, uint2 *starts, uint32_t *events,
-                                                       unsigned long long *next_unit) {
+                                                       unsigned long long *next_unit, const uint32_t *crt) {
     __shared__ uint4 tiles[8][256];
     uint4 *tile = tiles[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
@@ -783,7 +787,7 @@ __global__ void __launch_bounds__(256, split_min_blocks<Src>()) k_split_run_fix(
         uint64_t k = u / groups;
         const uint64_t g = u % groups, l = g * 32 + lane;
         const DevState st = seg.at(k);
-        warp_task<Src, SINK>(st, g, k + 1 == K ? len_last : len, out, ld, col0 + k * len, nullptr, tile);
+        warp_task<Src, SINK>(st, g, k + 1 == K ? len_last : len, out, ld, col0 + k * len, nullptr, tile, crt);
         if (k == 0) {  // the same threads stored segment 0's end: c_1
             starts[P + l] = make_uint2(st.u32[F_SLOT * P + l], st.u32[F_X * P + l]);
             k = 1;
@@ -820,7 +824,7 @@ __global__ void __launch_bounds__(256, split_min_blocks<Src>()) k_split_run_fix(
 template <class Src, int SINK>
 cudaError_t launch_split_run_fix(const SegSpace &sp, uint32_t K, uint64_t len, uint64_t len_last, uint64_t groups,
                                  uint32_t *out, uint64_t ld, uint64_t col0, uint2 *starts, uint32_t *events,
-                                 unsigned long long *next_unit, cudaStream_t stream) {
+                                 unsigned long long *next_unit, const uint32_t *crt, cudaStream_t stream) {
     static int per_sm = 0;
     static std::once_flag once;
     std::call_once(once, [] {
@@ -830,27 +834,27 @@ cudaError_t launch_split_run_fix(const SegSpace &sp, uint32_t K, uint64_t len, u
     const uint64_t units = (uint64_t)K * groups;
     const int blocks = (int)std::min<uint64_t>((units + 7) / 8, (uint64_t)sm_count() * per_sm);
     k_split_run_fix<Src, SINK><<<blocks, 256, 0, stream>>>(sp, K, len, len_last, groups, out, ld, col0, starts, events,
-                                                           next_unit);
+                                                           next_unit, crt);
     return cudaGetLastError();
 }
 
 template <int SINK>
 cudaError_t split_run_sink(int variant, int xl, const SegSpace &sp, const DevState &caller, int caller0, uint32_t kb,
                            uint32_t ke, uint32_t K, uint64_t len, uint64_t len_last, uint32_t *out, uint64_t ld,
-                           uint64_t col0, uint64_t *aux, cudaStream_t stream) {
+                           uint64_t col0, uint64_t *aux, const uint32_t *crt, cudaStream_t stream) {
     if (variant == CI_VAR_BBS)
-        return launch_split_run<SrcBbs, SINK>(sp, caller, caller0, kb, ke, K, len, len_last, out, ld, col0, aux, stream);
+        return launch_split_run<SrcBbs, SINK>(sp, caller, caller0, kb, ke, K, len, len_last, out, ld, col0, aux, crt, stream);
     if (variant == CI_VAR_BBS16)
         return launch_split_run<SrcBbs16Seg, SINK>(sp, caller, caller0, kb, ke, K, len, len_last, out, ld, col0, aux,
-                                                   stream);
+                                                   crt, stream);
     if (xl == CI_XL_XORSHIFT32)
         return launch_split_run<SrcXorshift32, SINK>(sp, caller, caller0, kb, ke, K, len, len_last, out, ld, col0, aux,
-                                                     stream);
+                                                     crt, stream);
     if (xl == CI_XL_XOR64)
         return launch_split_run<SrcXor64, SINK>(sp, caller, caller0, kb, ke, K, len, len_last, out, ld, col0, aux,
-                                                stream);
+                                                crt, stream);
     return launch_split_run<SrcXor128, SINK>(sp, caller, caller0, kb, ke, K, len, len_last, out, ld, col0, aux,
-                                             stream);
+                                             crt, stream);
 }
 
 // Runs segments [kb, ke) into the caller's sink (CI_SINK_*); written outputs
@@ -858,20 +862,20 @@ cudaError_t split_run_sink(int variant, int xl, const SegSpace &sp, const DevSta
 // state (zero < 0) or segment state `zero`.
 cudaError_t split_run(const ci_states_s &h, int sink, const SegSpace &sp, int caller0, uint32_t kb, uint32_t ke,
                       uint32_t K, uint64_t len, uint64_t len_last, uint32_t *out, uint64_t ld, uint64_t col0,
-                      uint64_t *aux, cudaStream_t stream) {
+                      uint64_t *aux, const uint32_t *crt, cudaStream_t stream) {
     const DevState caller = h.view();
     if (sink == CI_SINK_QC)
         return split_run_sink<SINK_QC>(h.variant, h.xl, sp, caller, caller0, kb, ke, K, len, len_last, out, ld, col0,
-                                       aux, stream);
+                                       aux, crt, stream);
     if (sink == CI_SINK_DIGEST)
         return split_run_sink<SINK_DIGEST>(h.variant, h.xl, sp, caller, caller0, kb, ke, K, len, len_last, out, ld,
-                                           col0, aux, stream);
+                                           col0, aux, crt, stream);
     const bool v4 = (reinterpret_cast<uintptr_t>(out) & 15u) == 0 && ld % 4 == 0 && col0 % 4 == 0 && len % 4 == 0;
     if (v4)
         return split_run_sink<SINK_V4>(h.variant, h.xl, sp, caller, caller0, kb, ke, K, len, len_last, out, ld, col0,
-                                       aux, stream);
+                                       aux, crt, stream);
     return split_run_sink<SINK_SCALAR>(h.variant, h.xl, sp, caller, caller0, kb, ke, K, len, len_last, out, ld, col0,
-                                       aux, stream);
+                                       aux, crt, stream);
 }
 
 int split_block_count(uint64_t items) {
@@ -967,7 +971,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
             else return fail(CI_E_INVAL, "unsplit CI_VAR_BBS16 output needs ld == n and col0 == 0");
         } else {
             SegSpace none{};
-            e = split_run(*h, sink, none, -1, 0, 1, 1, n, n, out, ld, col0, aux, stream);
+            e = split_run(*h, sink, none, -1, 0, 1, 1, n, n, out, ld, col0, aux, nullptr, stream);
         }
         return e == cudaSuccess ? CI_OK : cuda_fail(e, "split run");
     }
@@ -1013,7 +1017,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
     const int own_first = b16 ? (int)F_Y16 : (int)F_A, own_count = b16 ? 8 : kOwnWords;
     const uint64_t res_bytes = 8ull * K * h->P;  // per-segment consumer results
     const uint64_t own_bytes = fixup ? 0 : (4ull * own_count + (bbs ? 8ull : 0ull)) * K * h->P;
-    const uint64_t lam_bytes = b16 ? 4ull * 8 * h->P : bbs ? 16ull * h->P : 0;
+    const uint64_t lam_bytes = b16 ? 4ull * 8 * h->P : bbs ? (16ull + 4ull * kCrtWords) * h->P : 0;
     uint8_t *ws = nullptr;
     if ((e = cudaMallocAsync(reinterpret_cast<void **>(&ws), stride * slots + 2 * res_bytes + own_bytes + lam_bytes,
                              stream)) != cudaSuccess)
@@ -1028,6 +1032,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
     }
     uint32_t *lam16 = b16 ? reinterpret_cast<uint32_t *>(after + own_bytes) : nullptr;
     uint64_t *lam64 = bbs ? reinterpret_cast<uint64_t *>(after + own_bytes) : nullptr;
+    uint32_t *crt = bbs ? reinterpret_cast<uint32_t *>(lam64 + 2 * h->P) : nullptr;  // residue-form constants
 
     // Handles over the segment states (host copies of the caller's, moved).
     std::vector<ci_states_s> segs(slots, *h);
@@ -1042,7 +1047,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
 
     ci_status st = CI_OK;
     if (b16) k_split_lambda16<<<split_block_count(h->P), 256, 0, stream>>>(src, lam16);
-    if (bbs) k_split_lambda<<<split_block_count(h->P), 256, 0, stream>>>(src, lam64);
+    if (bbs) k_split_lambda<<<split_block_count(h->P), 256, 0, stream>>>(src, lam64, crt);
     k_split_setup<<<split_block_count(slots * h->P), 256, 0, stream>>>(src, sp, (uint32_t)K, len, h->variant, h->xl,
                                                                        own, lam16, lam64);
     if ((e = cudaGetLastError()) != cudaSuccess) st = cuda_fail(e, "split setup");
@@ -1057,14 +1062,14 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
         if ((e = cudaMemsetAsync(res3, 0, 8 + 4 * K * groups, stream)) == cudaSuccess) {
             if (bbs)
                 e = v4 ? launch_split_run_fix<SrcBbs, SINK_V4>(sp, k32, len, len_last, groups, out, ld, col0, starts,
-                                                               events, next_unit, stream)
+                                                               events, next_unit, crt, stream)
                        : launch_split_run_fix<SrcBbs, SINK_SCALAR>(sp, k32, len, len_last, groups, out, ld, col0,
-                                                                   starts, events, next_unit, stream);
+                                                                   starts, events, next_unit, crt, stream);
             else
                 e = v4 ? launch_split_run_fix<SrcBbs16Seg, SINK_V4>(sp, k32, len, len_last, groups, out, ld, col0,
-                                                                    starts, events, next_unit, stream)
+                                                                    starts, events, next_unit, crt, stream)
                        : launch_split_run_fix<SrcBbs16Seg, SINK_SCALAR>(sp, k32, len, len_last, groups, out, ld, col0,
-                                                                        starts, events, next_unit, stream);
+                                                                        starts, events, next_unit, crt, stream);
         }
         if (e == cudaSuccess) {
             k_split_copy_back<<<split_block_count(h->P), 256, 0, stream>>>(src, segs[K - 1].view(), h->variant);
@@ -1078,9 +1083,9 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
     // otherwise segments 0 .. K-2, of which only the end states are needed)
     if (st == CI_OK) {
         e = fixup ? split_run(*h, sink, sp, 0, 0, (uint32_t)K, (uint32_t)K, len, len_last, out, ld, col0, nullptr,
-                              stream)
+                              crt, stream)
                   : split_run(*h, CI_SINK_DIGEST, sp, 0, 0, (uint32_t)K - 1, (uint32_t)K, len, len_last, nullptr, 0,
-                              0, res1, stream);
+                              0, res1, crt, stream);
         if (e != cudaSuccess) st = cuda_fail(e, "split pass 1");
     }
     uint2 *starts = reinterpret_cast<uint2 *>(res1);  // K * P (slot, x) pairs, after pass 1
@@ -1117,7 +1122,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
         st = cuda_fail(e, "clearing counts");
     if (st == CI_OK) {  // pass 2: every segment from its true start into the sink
         e = split_run(*h, sink, sp, b16 ? (int)K : -1, 0, (uint32_t)K, (uint32_t)K, len, len_last, out, ld, col0,
-                      res3, stream);
+                      res3, crt, stream);
         if (e != cudaSuccess) st = cuda_fail(e, "split pass 2");
     }
     if (st == CI_OK) {

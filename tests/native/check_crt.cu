@@ -1,0 +1,92 @@
+// Host check of the residue form of the modular square (ci_crt.cuh) against
+// 128-bit arithmetic, over the whole range of factors it accepts: random
+// and consecutive odd factors, the ends of (2^30, 2^31), and residues 0, 1,
+// p / 2 on both sides, p - 1 and where the quotient is nearly exact.  Prints
+// "ok" when nothing differs.
+#include <cstdint>
+#include <cstdio>
+#include <random>
+
+#include "ci_crt.cuh"
+
+using namespace ci::dev;
+typedef unsigned __int128 u128;
+
+static uint64_t gcd(uint64_t a, uint64_t b) {
+    while (b) {
+        const uint64_t t = a % b;
+        a = b;
+        b = t;
+    }
+    return a;
+}
+
+int main() {
+    std::mt19937_64 g(11125239);
+    long bad = 0, n = 0;
+    const uint32_t lo = (1u << 30) + 1, hi = (1u << 31) - 1;
+
+    // CrtPrime::sqr
+    for (int k = 0; k < 400000; ++k) {
+        uint32_t p;
+        if (k < 4000) p = lo + (uint32_t)k;
+        else if (k < 8000) p = hi - (uint32_t)(k - 4000);
+        else p = lo + (uint32_t)(g() % (hi - lo + 1));
+        p |= 1u;
+        CrtPrime c;
+        c.set(p);
+        for (int j = 0; j < 24; ++j) {
+            uint32_t r;
+            switch (j) {
+                case 0: r = 0; break;
+                case 1: r = 1; break;
+                case 2: r = p - 1; break;
+                case 3: r = p - 2; break;
+                case 4: r = p / 2; break;
+                case 5: r = p / 2 + 1; break;
+                default: r = (uint32_t)(g() % p);
+            }
+            if (j >= 12) {  // r^2 just above or below a multiple of p near the top of the range
+                const uint64_t m = (uint64_t)p * (p / 4 - (uint64_t)(g() % 1000));
+                uint64_t s = (uint64_t)__builtin_sqrtl((long double)m);
+                r = (uint32_t)(s + (g() & 1));
+                if (r >= p) r = p - 1;
+            }
+            bad += c.sqr(r) != (uint32_t)((uint64_t)r * r % p), ++n;
+        }
+    }
+    printf("square modulo a factor: %ld of %ld differ\n", bad, n);
+    long all = bad;
+
+    // CrtModulus: acceptance, value, chains of squarings
+    bad = n = 0;
+    CrtModulus m;
+    bad += m.set(1u << 30, hi) || m.set(lo, lo) || m.set(lo, 1u << 31) || m.set(lo + 1, hi) || m.set(3, hi);
+    long taken = 0;
+    for (int k = 0; k < 60000; ++k) {
+        uint32_t a = (k & 1) ? lo + 2 * (uint32_t)(g() % 5000) : lo + (uint32_t)(g() % (hi - lo + 1));
+        uint32_t b = (k & 2) ? hi - 2 * (uint32_t)(g() % 5000) : lo + (uint32_t)(g() % (hi - lo + 1));
+        a |= 1u;
+        b |= 1u;
+        if (!m.set(a, b)) continue;  // not coprime, or a composite q without Fermat's inverse
+        ++taken;
+        bad += gcd(a, b) != 1, ++n;
+        const uint32_t p = m.P.p, q = m.Q.p;
+        const uint64_t M = (uint64_t)p * q;
+        uint64_t x = k % 7 == 0 ? M - 1 : k % 7 == 1 ? 0 : k % 7 == 2 ? (uint64_t)p * (g() % q) : g() % M;
+        uint32_t rp = (uint32_t)(x % p), rq = (uint32_t)(x % q);
+        bad += m.value(rp, rq) != x, ++n;
+        for (int j = 0; j < 40; ++j) {
+            x = (uint64_t)((u128)x * x % M);
+            rp = m.P.sqr(rp);
+            rq = m.Q.sqr(rq);
+            bad += m.value(rp, rq) != x, ++n;
+            bad += m.low(rp, rq) != (uint32_t)x, ++n;
+        }
+    }
+    printf("square modulo p q: %ld of %ld differ (%ld moduli)\n", bad, n, taken);
+    all += bad;
+    if (all || taken < 1000) return 1;
+    printf("ok\n");
+    return 0;
+}
