@@ -471,7 +471,10 @@ typedef struct {
                                   (evict-first) 16-byte stores, 1 write-back
                                   16-byte stores, 2 TMA bulk tensor stores of the
                                   staging tile (xor sources, tile depth 32; falls
-                                  back to 0 where TMA's alignment rules fail)     */
+                                  back to 0 where TMA's alignment rules fail).
+                                  Short rows of the xor sources that are not
+                                  whole 32-byte sectors leave as one bulk store
+                                  per 32 streams whatever the policy             */
     float ms;                  /* time of the tuning problem with this shape (0:
                                   not measured)                                    */
 } ci_tune_choice;

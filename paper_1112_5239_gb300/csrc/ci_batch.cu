@@ -49,7 +49,7 @@ constexpr int kBatchWarps = 16;
 
 template <int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, kBatchWarps / WARPS) k_batched(BatchHeader *hdr, const BatchTask *tasks) {
-    __shared__ uint4 tiles[WARPS][256];
+    __shared__ uint4 tiles[WARPS][kTileVec];
     const int lane = threadIdx.x & 31;
     uint4 *tile = tiles[threadIdx.x >> 5];
     const uint64_t total = hdr->total_units;

@@ -12,25 +12,47 @@
 
 namespace ci {
 
-// One warp per group of 32 lanes, W warps per block, a persistent grid whose
-// warps stride over the warp groups; written sinks stage a 32 x KT tile per
-// warp in dynamic shared memory.  Warp w of block b starts at group
-// w * gridDim.x + b: with fewer groups than resident warps, the idle warps are
-// spread over all blocks (hence all SMs) instead of leaving whole blocks idle.
+// One warp per group of 32 lanes, W warps per block.  A state of more groups
+// than resident warps gets one block per W consecutive groups, handed to the
+// SMs in order as they fall free: the SMs do not run at the same speed (two
+// dies, one memory each), so a fixed share per SM ends with the slowest, and
+// stores in address order reach 7.6 TB/s where the same stores from a
+// persistent grid reached 6.5 (1 GiB, nothing else in the kernel).  Measured
+// against a persistent grid: 2^20 x 1024 consumed 610 instead of 690 us, 2^20
+// x 256 written 175 instead of 199 us.  A state of fewer groups runs in one
+// wave: one block per group as far as blocks are resident, and warp w of block
+// b takes group w * gridDim.x + b, so that every SM gets its share of the warps.
+// Either way a warp has at most one group.
+struct GenGrid {
+    unsigned grid;
+    uint32_t in_order;
+};
+inline GenGrid gen_grid(uint64_t groups, int W, uint64_t resident_blocks) {
+    if (groups > resident_blocks * W) return {(unsigned)((groups + W - 1) / W), 1u};
+    return {(unsigned)(groups < resident_blocks ? groups : resident_blocks), 0u};
+}
+template <int W>
+__device__ __forceinline__ uint64_t warp_group(uint32_t in_order) {
+    const uint64_t w = threadIdx.x >> 5;
+    return in_order ? (uint64_t)blockIdx.x * W + w : w * gridDim.x + blockIdx.x;
+}
+
+// Written sinks stage a 32 x KT tile per warp in dynamic shared memory.
+template <int SINK, class TC>
+constexpr int kTileVecs = SINK >= dev::SINK_QC ? 0 : SINK == dev::SINK_SCALAR ? dev::kTileVec : TC::KT * 8;
 template <class Src, int SINK, int W, class TC>
-__global__ void __launch_bounds__(W * 32) k_generate(DevState st, uint64_t n, uint32_t *out, uint64_t *counts) {
+__global__ void __launch_bounds__(W * 32) k_generate(DevState st, uint64_t n, uint32_t in_order, uint32_t *out,
+                                                     uint64_t *counts) {
     extern __shared__ uint4 dyn_tiles[];
     const int w = threadIdx.x >> 5;
-    uint4 *tile = dyn_tiles + (SINK >= dev::SINK_QC ? 0 : w * TC::KT * 8);
-    const uint64_t ngroups = st.P / 32;
-    const uint64_t gstride = (uint64_t)gridDim.x * W;
-    for (uint64_t g = (uint64_t)w * gridDim.x + blockIdx.x; g < ngroups; g += gstride)
-        dev::warp_task<Src, SINK, TC>(st, g, n, out, n, 0, counts, tile);
+    uint4 *tile = dyn_tiles + w * kTileVecs<SINK, TC>;
+    const uint64_t g = warp_group<W>(in_order);
+    if (g < st.P / 32) dev::warp_task<Src, SINK, TC>(st, g, n, out, n, 0, counts, tile);
 }
 
 // Written sink through TMA bulk tensor stores (xor sources, store policy 2).
 template <class Src, int W>
-__global__ void __launch_bounds__(W * 32) k_generate_tma(DevState st, uint64_t n, uint32_t *out,
+__global__ void __launch_bounds__(W * 32) k_generate_tma(DevState st, uint64_t n, uint32_t in_order,
                                                          const __grid_constant__ CUtensorMap map) {
     extern __shared__ uint4 tma_tiles[];
     // the 128-byte swizzle needs 1024-byte aligned tiles: round the base up
@@ -39,12 +61,40 @@ __global__ void __launch_bounds__(W * 32) k_generate_tma(DevState st, uint64_t n
     uint4 *base = reinterpret_cast<uint4 *>(reinterpret_cast<char *>(tma_tiles) + ((1024u - (sbase & 1023u)) & 1023u));
     const int w = threadIdx.x >> 5;
     uint4 *tiles = base + w * 512;  // two 4 KB tiles per warp
-    const uint64_t ngroups = st.P / 32;
-    const uint64_t gstride = (uint64_t)gridDim.x * W;
-    for (uint64_t g = (uint64_t)w * gridDim.x + blockIdx.x; g < ngroups; g += gstride)  // as in k_generate
-        dev::warp_task_tma<Src>(st, g, n, &map, out, n, 0, tiles);
-    if ((threadIdx.x & 31) == 0) dev::tma_wait_all();  // every store complete before the block exits
-    __syncwarp();
+    const uint64_t g = warp_group<W>(in_order);
+    if (g < st.P / 32) dev::warp_task_tma<Src>(st, g, n, &map, tiles);
+}
+
+// Short rows as one bulk store per warp group (xor sources): one warp per
+// block, as many blocks per SM as their 128 n bytes of staging allow.
+template <class Src>
+__global__ void __launch_bounds__(32) k_generate_span(DevState st, uint32_t n, uint32_t *out) {
+    extern __shared__ __align__(128) uint32_t span_stage[];
+    dev::warp_task_span<Src>(st, blockIdx.x, n, out, span_stage);
+}
+
+// Which written rows leave as spans: out 16-byte aligned, and rows that are
+// not whole 32-byte sectors (the others' TMA tiles write whole sectors) up to
+// the length where too few warps fit an SM beside their staging, or shorter
+// than a TMA tile.  400 MB in rows of n, span against the next best form: n =
+// 36 83 us / 95 TMA, 100 70 / 117, 249 84 / 107 line-staged, 260 95 / 117 TMA,
+// 290 96 / 105 line-staged, 333 113 / 101, 350 111 / 101; n = 200 81 / 69 TMA,
+// 144 80 / 69.
+constexpr uint64_t kSpanMax = 296;
+inline bool span_rows(uint64_t n, const uint32_t *out) {
+    return n <= kSpanMax && (n % 8 != 0 || n < 32) && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+}
+
+template <class Src>
+static cudaError_t launch_gen_span(const DevState &st, uint64_t n, uint32_t *out, cudaStream_t stream) {
+    auto kern = k_generate_span<Src>;
+    static std::once_flag once;
+    std::call_once(once, [&] {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(128 * kSpanMax));
+        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    });
+    kern<<<(unsigned)(st.P / 32), 32, 128 * n, stream>>>(st, (uint32_t)n, out);
+    return cudaGetLastError();
 }
 
 // Tensor map over out[rows][cols] (uint32, row stride cols words) with a
@@ -67,12 +117,9 @@ static cudaError_t launch_gen_tma(const DevState &st, uint64_t n, uint32_t *out,
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kern, W * 32, smem) == cudaSuccess && ps > 0)
             per_sm = ps;
     });
-    const uint64_t cap = (uint64_t)sm_count() * per_sm;
-    const uint64_t need = st.P / 32;  // a block per group at most (the warps spread over the blocks)
-    const unsigned grid = (unsigned)(need < cap ? need : cap);
+    const GenGrid gg = gen_grid(st.P / 32, W, (uint64_t)sm_count() * per_sm);
     *used = true;
-    if (grid == 0) return cudaSuccess;
-    kern<<<grid, W * 32, smem, stream>>>(st, n, out, map);
+    kern<<<gg.grid, W * 32, smem, stream>>>(st, n, gg.in_order, map);
     return cudaGetLastError();
 }
 
@@ -80,7 +127,7 @@ template <class Src, int SINK, int W, class TC>
 static cudaError_t launch_gen_t(const DevState &st, uint64_t n, uint32_t *out, uint64_t *counts,
                                 cudaStream_t stream) {
     auto kern = k_generate<Src, SINK, W, TC>;
-    const size_t smem = SINK >= dev::SINK_QC ? 0 : (size_t)W * TC::KT * 8 * sizeof(uint4);
+    const size_t smem = (size_t)W * kTileVecs<SINK, TC> * sizeof(uint4);
     static std::once_flag once;
     static int per_sm = 1;
     std::call_once(once, [&] {
@@ -89,17 +136,16 @@ static cudaError_t launch_gen_t(const DevState &st, uint64_t n, uint32_t *out, u
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kern, W * 32, smem) == cudaSuccess && ps > 0)
             per_sm = ps;
     });
-    const uint64_t cap = (uint64_t)sm_count() * per_sm;
-    const uint64_t need = st.P / 32;  // a block per group at most (the warps spread over the blocks)
-    const unsigned grid = (unsigned)(need < cap ? need : cap);
-    if (grid == 0) return cudaSuccess;
-    kern<<<grid, W * 32, smem, stream>>>(st, n, out, counts);
+    const GenGrid gg = gen_grid(st.P / 32, W, (uint64_t)sm_count() * per_sm);
+    kern<<<gg.grid, W * 32, smem, stream>>>(st, n, gg.in_order, out, counts);
     return cudaGetLastError();
 }
 
 template <class Src, int SINK, int W>
 static cudaError_t gen_tile(const TuneChoice &c, const DevState &st, uint64_t n, uint32_t *out, uint64_t *counts,
                             cudaStream_t stream) {
+    if constexpr (SINK <= dev::SINK_SCALAR && !Src::kHeavy)
+        if (span_rows(n, out)) return launch_gen_span<Src>(st, n, out, stream);
     if constexpr (SINK == dev::SINK_V4 && !Src::kHeavy) {
         if (c.cache_policy == 2) {
             bool used = false;

@@ -124,13 +124,21 @@ __global__ void __launch_bounds__(256) k_naive_init(NaiveView v, uint64_t seed, 
     }
 }
 
+__device__ __forceinline__ uint4 next4(NaiveLane &L) {
+    uint4 o;
+    o.x = L.next();
+    o.y = L.next();
+    o.z = L.next();
+    o.w = L.next();
+    return o;
+}
+
 // One warp per 32 lanes; rows r < S of out (row stride n) receive the outputs.
 template <bool V4>
 __global__ void __launch_bounds__(256, CI_NAIVE_MIN_BLOCKS) k_naive_generate(NaiveView v, uint64_t n, uint32_t *out) {
-    __shared__ uint4 tiles[8][256];
+    __shared__ uint4 tiles[8][V4 ? 256 : kTileVec];
     const int lane = threadIdx.x & 31;
     uint4 *tile = tiles[threadIdx.x >> 5];
-    uint32_t *tw = reinterpret_cast<uint32_t *>(tile);
     const uint64_t groups = v.P / 32;
     const uint64_t wstride = (uint64_t)gridDim.x * 8;
     // warp w of block b starts at group w * gridDim.x + b: a partial last
@@ -139,37 +147,27 @@ __global__ void __launch_bounds__(256, CI_NAIVE_MIN_BLOCKS) k_naive_generate(Nai
         const uint64_t l = g * 32 + lane, row0 = g * 32;
         NaiveLane L;
         L.load(v.u64, v.x, v.P, l);
-        const uint64_t nfull = n - n % 32;
-        for (uint64_t i0 = 0; i0 < nfull; i0 += 32) {
+        if constexpr (!V4) {
+            written_unaligned<false, 0>([&]() { return L.next(); }, v.S, row0, n, out, n, 0, tile);
+        } else {
+            const uint64_t nfull = n - n % 32;
+            for (uint64_t i0 = 0; i0 < n; i0 += 32) {
+                const int chunks = i0 < nfull ? 8 : (int)(n - nfull) / 4;
+                if (chunks == 8) {
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                uint4 o;
-                o.x = L.next();
-                o.y = L.next();
-                o.z = L.next();
-                o.w = L.next();
-                tile[lane * 8 + (q ^ (lane & 7))] = o;
-            }
-            __syncwarp();
-            if (V4) {
+                    for (int q = 0; q < 8; ++q) tile[lane * 8 + (q ^ (lane & 7))] = next4(L);
+                } else {
+                    for (int q = 0; q < chunks; ++q) tile[lane * 8 + (q ^ (lane & 7))] = next4(L);
+                }
+                __syncwarp();
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     const int r = 4 * k + lane / 8, c = lane % 8;
-                    if (row0 + r < v.S) store16<0>(out + (row0 + r) * n + i0 + 4 * c, tile[r * 8 + (c ^ (r & 7))]);
+                    if (row0 + r < v.S && c < chunks)
+                        store16<0>(out + (row0 + r) * n + i0 + 4 * c, tile[r * 8 + (c ^ (r & 7))]);
                 }
-            } else {
-                for (int r = 0; r < 32; ++r)
-                    if (row0 + r < v.S) store4<0>(out + (row0 + r) * n + i0 + lane, tw[tile_word<32>(r, lane)]);
+                __syncwarp();
             }
-            __syncwarp();
-        }
-        const int rem = (int)(n - nfull);
-        if (rem) {
-            for (int k = 0; k < rem; ++k) tw[tile_word<32>(lane, k)] = L.next();
-            __syncwarp();
-            for (int r = 0; r < 32; ++r)
-                if (lane < rem && row0 + r < v.S) out[(row0 + r) * n + nfull + lane] = tw[tile_word<32>(r, lane)];
-            __syncwarp();
         }
         L.store(v.u64, v.x, v.P, l);
     }

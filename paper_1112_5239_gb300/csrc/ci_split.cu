@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(256, split_min_blocks<Src>()) k_split_run(SegS
                                                    uint32_t k_end, uint32_t K, uint64_t len, uint64_t len_last,
                                                    uint64_t groups, uint32_t *out, uint64_t ld, uint64_t col0,
                                                    uint64_t *aux, const uint32_t *crt) {
-    __shared__ uint4 tiles[8][256];
+    __shared__ uint4 tiles[8][SINK == SINK_SCALAR ? kTileVec : 256];
     uint4 *tile = tiles[threadIdx.x >> 5];
     const uint64_t units = (uint64_t)(k_end - k_begin) * groups;
     // warp w of block b starts at unit w * gridDim.x + b: a partial last
@@ -774,7 +774,7 @@ __global__ void __launch_bounds__(256, split_min_blocks<Src>()) k_split_run_fix(
                                                        uint64_t len_last, uint64_t groups, uint32_t *out, uint64_t ld,
                                                        uint64_t col0, uint2 *starts, uint32_t *events,
                                                        unsigned long long *next_unit, const uint32_t *crt) {
-    __shared__ uint4 tiles[8][256];
+    __shared__ uint4 tiles[8][SINK == SINK_SCALAR ? kTileVec : 256];
     uint4 *tile = tiles[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const DevState s0 = seg.at(0);

@@ -21,11 +21,19 @@ static std::mutex g_tune_mu;
 static ci_tune_table g_table = [] {
     ci_tune_table t;
     std::memset(&t, 0, sizeof t);
+    // Without a tuning run: blocks of 4 warps for the xor-likes (handed out in
+    // order, see ci_gen.cuh: 2^20 x 1024 consumed 610 us, 630 with 8 and 16
+    // warps) and, for their aligned rows, TMA tiles (2^20 x 256: 176 us, 180 by
+    // 16-byte stores); 8 for the BBS sources.
     for (int s = 0; s < kSrcKinds; ++s)
         for (int k = 0; k < 4; ++k) {
-            t.choice[s][k].warps_per_block = 8;
+            t.choice[s][k].warps_per_block = s == SK_BBS || s == SK_BBS16 ? 8 : 4;
             t.choice[s][k].tile_depth = 32;
             t.choice[s][k].cache_policy = 0;
+            if (k == dev::SINK_V4 && s != SK_BBS && s != SK_BBS16) {
+                t.choice[s][k].warps_per_block = 4;
+                t.choice[s][k].cache_policy = 2;
+            }
         }
     t.batch_warps_per_block = 8;
     return t;
