@@ -103,6 +103,54 @@ static ci_status check_params(const ci_params *p, uint64_t S) {
     return CI_OK;
 }
 
+// ------------------------------------------------- workspace pools
+namespace {
+constexpr int kPoolDevices = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pools[kPoolDevices];  // per device, created on first use
+uint64_t g_live_handles = 0;
+
+// The pool of the current device, or null (the default pool serves then).
+cudaMemPool_t workspace_pool() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kPoolDevices) return nullptr;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (!g_pools[dev]) {
+        cudaMemPoolProps props;
+        std::memset(&props, 0, sizeof props);
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        uint64_t keep = kWorkspaceKept;
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        g_pools[dev] = pool;
+    }
+    return g_pools[dev];
+}
+
+void handle_made() {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    ++g_live_handles;
+}
+// Trimming releases unused memory only: workspaces of calls still running stay.
+void handle_gone() {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (--g_live_handles) return;
+    for (cudaMemPool_t p : g_pools)
+        if (p) cudaMemPoolTrimTo(p, 0);
+}
+}  // namespace
+
+cudaError_t workspace_alloc(void **p, size_t bytes, cudaStream_t stream) {
+    const cudaMemPool_t pool = workspace_pool();
+    return pool ? cudaMallocFromPoolAsync(p, bytes, pool, stream) : cudaMallocAsync(p, bytes, stream);
+}
+
 static uint64_t lanes_for(uint64_t S) { return (S + 31ull) & ~31ull; }
 
 ci_status prepare_handle(const ci_params *p, uint64_t S, void *dev, uint64_t bytes, bool owns, ci_states *out) {
@@ -124,6 +172,7 @@ ci_status prepare_handle(const ci_params *p, uint64_t S, void *dev, uint64_t byt
     else
         derive_comb(p->variant, h->C, p->comb_seed, h->comb);
     build_table(p->variant, h->C, h->comb, h->table);
+    handle_made();
     *out = h;
     return CI_OK;
 }
@@ -147,6 +196,7 @@ static ci_status make_handle(const ci_params *p, uint64_t S, void *dev, uint64_t
     if (e != cudaSuccess) {
         h->magic = 0;
         delete h;
+        handle_gone();
         return cuda_fail(e, "state initialisation");
     }
     *out = h;
@@ -344,7 +394,7 @@ ci_status ci_init_states_many(const ci_params *params, const uint64_t *n_streams
     }
     InitTask *dtasks = nullptr;
     if (rc == CI_OK) {
-        cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&dtasks), sizeof(InitTask) * n, cs);
+        cudaError_t e = workspace_alloc(reinterpret_cast<void **>(&dtasks), sizeof(InitTask) * n, cs);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(dtasks, tasks.data(), sizeof(InitTask) * n, cudaMemcpyHostToDevice, cs);
         if (e == cudaSuccess) e = launch_init_batched(dtasks, n, lanes, cs);
@@ -367,6 +417,7 @@ ci_status ci_free_states(ci_states s) {
     cudaError_t e = cudaSuccess;
     if (s->owns) e = cudaFree(s->dev);
     delete s;
+    handle_gone();
     return e == cudaSuccess ? CI_OK : cuda_fail(e, "cudaFree of the state");
 }
 

@@ -341,22 +341,32 @@ struct SrcBbs {
 // shorter factors, which keep the 62-bit form).
 constexpr int kCrtWords = 4;  // mu_p, mu_q, beta (0: not usable), beta_s
 
+// Lane l's residue constants: false (beta stored as 0) where the residue form
+// does not apply.
+__device__ __forceinline__ bool crt_store(const DevState &s, uint64_t l, uint32_t *crt) {
+    CrtModulus C{};
+    const bool ok = C.set(s.u32[F_P * s.P + l], s.u32[F_Q * s.P + l]);
+    crt[l] = C.P.mu;
+    crt[s.P + l] = C.Q.mu;
+    crt[2 * s.P + l] = ok ? C.beta : 0u;
+    crt[3 * s.P + l] = C.beta_s;
+    return ok;
+}
+__device__ __forceinline__ bool crt_load(const DevState &s, uint64_t l, const uint32_t *crt, CrtModulus &C) {
+    const uint32_t a = s.u32[F_P * s.P + l], b = s.u32[F_Q * s.P + l];
+    C.P.set(min(a, b), crt[l]);
+    C.Q.set(max(a, b), crt[s.P + l]);
+    C.beta = crt[2 * s.P + l];
+    C.beta_s = crt[3 * s.P + l];
+    return C.beta != 0u;
+}
+
 struct SrcBbsCrt {
     static constexpr bool kHeavy = true, kOneStep = true;
     CrtModulus C;
     uint32_t rp, rq, sel;
     __device__ __forceinline__ bool load(const DevState &s, uint64_t l, const uint32_t *crt) {
-        const uint32_t a = s.u32[F_P * s.P + l], b = s.u32[F_Q * s.P + l];
-        bool ok;
-        if (crt) {
-            C.P.set(min(a, b), crt[l]);
-            C.Q.set(max(a, b), crt[s.P + l]);
-            C.beta = crt[2 * s.P + l];
-            C.beta_s = crt[3 * s.P + l];
-            ok = C.beta != 0u;
-        } else {
-            ok = C.set(a, b);
-        }
+        const bool ok = crt ? crt_load(s, l, crt, C) : C.set(s.u32[F_P * s.P + l], s.u32[F_Q * s.P + l]);
         if (!__all_sync(kFull, ok)) return false;
         const uint64_t y = s.u64[G_Y * s.P + l];
         rp = (uint32_t)(y % C.P.p);
@@ -391,16 +401,6 @@ struct SrcBbsCrt {
     }
 };
 
-// Lane l's residue constants, for SrcBbsCrt::load.
-__device__ __forceinline__ void crt_store(const DevState &s, uint64_t l, uint32_t *crt) {
-    CrtModulus C{};
-    const bool ok = C.set(s.u32[F_P * s.P + l], s.u32[F_Q * s.P + l]);
-    crt[l] = C.P.mu;
-    crt[s.P + l] = C.Q.mu;
-    crt[2 * s.P + l] = ok ? C.beta : 0u;
-    crt[3 * s.P + l] = C.beta_s;
-}
-
 // Shortest unit that takes the residue form when its constants have to be
 // computed first (2^16 streams, written: 12 outputs 21.3 us against 23.1 in
 // the 62-bit form, 16 outputs 25.2 against 29.2; 8 outputs 18.8 against 17.6).
@@ -410,19 +410,21 @@ constexpr uint64_t kCrtMinLength = 12;
 // 2^16, so x^2 fits 32 bits.  x^2 mod M by Barrett reduction with
 // mu = floor(2^32 / M): q = mulhi(x^2, mu) is floor(x^2 / M) or one less, so a
 // single conditional subtraction gives the canonical residue, taken as the
-// unsigned minimum of r and r - M (r - M wraps above r when r < M).  The
+// unsigned minimum of r and r - M (r - M wraps above r when r < M), addition
+// and minimum in one instruction.  The
 // arrays are read from BBS1 and BBS2 when the call starts; at the end of the
 // call generator k (state and modulus) is stored in place k + 1.
 struct SrcBbs16 {
     static constexpr bool kHeavy = true, kOneStep = false;
-    uint32_t y[8], M[8], mu[8];
+    uint32_t y[8], nM[8], mu[8];  // nM = -M
     uint32_t sel1, sel2;
     __device__ __forceinline__ void load(const DevState &s, uint64_t l) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             y[k] = s.u32[(F_Y16 + k) * s.P + l];
-            M[k] = s.u32[(F_M16 + k) * s.P + l];
-            mu[k] = (uint32_t)((1ull << 32) / M[k]);
+            const uint32_t M = s.u32[(F_M16 + k) * s.P + l];
+            nM[k] = 0u - M;
+            mu[k] = (uint32_t)((1ull << 32) / M);
         }
         sel1 = y[0] & 7u;
         sel2 = y[1] & 7u;
@@ -431,7 +433,7 @@ struct SrcBbs16 {
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             s.u32[(F_Y16 + (k + 1) % 8) * s.P + l] = y[k];
-            s.u32[(F_M16 + (k + 1) % 8) * s.P + l] = M[k];
+            s.u32[(F_M16 + (k + 1) % 8) * s.P + l] = 0u - nM[k];
         }
     }
     __device__ __forceinline__ void arrays(const DevState &, uint64_t, int &a1, int &a2) const {
@@ -441,8 +443,7 @@ struct SrcBbs16 {
     template <int K>
     __device__ __forceinline__ uint32_t bbs() {  // BBS(K+1)
         const uint32_t a = y[K] * y[K];
-        const uint32_t r = a - __umulhi(a, mu[K]) * M[K];
-        y[K] = min(r, r - M[K]);
+        y[K] = addmin32(a + __umulhi(a, mu[K]) * nM[K], nM[K]);
         return y[K];
     }
     __device__ __forceinline__ uint32_t next() {

@@ -103,4 +103,13 @@ void fill_init_task(const ci_states_s &h, uint64_t seed, uint64_t first, uint64_
 
 int sm_count();
 
+// Stream-ordered workspaces of the calls, from a pool of the library's own on
+// the current device (cudaFreeAsync gives them back).  The pool keeps up to
+// kWorkspaceKept bytes between calls: the default pool gives its memory back
+// to the system at every synchronisation, and a call after one then spent
+// 200 us on getting it again.  All of it is released when the last handle is
+// freed.
+constexpr uint64_t kWorkspaceKept = 256ull << 20;
+cudaError_t workspace_alloc(void **p, size_t bytes, cudaStream_t stream);
+
 }  // namespace ci

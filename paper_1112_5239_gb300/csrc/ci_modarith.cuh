@@ -90,6 +90,13 @@ struct Mont32 {
         one = (0u - mod) % mod;  // (2^32 - m) mod m = R mod m
         r2 = (uint32_t)((uint64_t)one * one % mod);
     }
+    // From a stored `one`, without R^2 (for redc, mul, from and the powers).
+    __host__ __device__ __forceinline__ Mont32(uint32_t mod, uint32_t one_) : m(mod), one(one_), r2(0u) {
+        uint32_t inv = mod;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) inv *= 2u - mod * inv;
+        np = 0u - inv;
+    }
     __host__ __device__ __forceinline__ uint32_t redc(uint64_t t) const {  // t < m R
         const uint32_t u = (uint32_t)t * np;
         const uint64_t r = (t >> 32) + umulhi32(u, m) + ((uint32_t)t != 0u ? 1u : 0u);
@@ -126,13 +133,13 @@ struct Mont32 {
     // (2^e in Montgomery form), left to right: a squaring per bit and, for a
     // set bit, a doubling (the Montgomery form is linear, so 2 x R mod m is
     // the doubled form), taken by a select.
-    __host__ __device__ __forceinline__ uint32_t pow2_m(uint32_t e) const {
+    __host__ __device__ __forceinline__ uint32_t pow2_m(uint64_t e) const {
         uint32_t r = one;
-        for (int i = 31 - clz32(e | 1u); i >= 0; --i) {
+        for (int i = 63 - clz64(e | 1u); i >= 0; --i) {
             r = mul(r, r);
             const uint64_t d = 2ull * r;
             const uint32_t rd = (uint32_t)(d >= m ? d - m : d);
-            r = (e >> i) & 1u ? rd : r;
+            r = (e >> i) & 1ull ? rd : r;
         }
         return r;
     }

@@ -35,7 +35,7 @@
 //      end states are needed); k_split_carry, one block per warp group,
 //      scans the segments: the true start of segment k is its predecessor's
 //      particular end plus (Q s_a, x_a ^ S s_a) with Q = P^len,
-//      S = P + ... + P^len (a chunked parallel scan over up to 16 warps);
+//      S = P + ... + P^len (a chunked parallel scan over up to 32 warps);
 //      pass 2 (k_split_run) runs every segment from its true start, with the
 //      own words k_split_setup jumped to, into the sink;
 //   5. the last segment's end state becomes the caller's state, and the
@@ -157,7 +157,7 @@ cudaError_t ensure_jump_tables(cudaStream_t stream) {
 // ------------------------------------------------ BBS jump
 // x <- x^(2^E) mod M with E = 11 * dist squarings, through the exponent
 // 2^E mod lambda(M), lambda = lcm(p - 1, q - 1) (x is a unit mod M);
-// lambda and its Barrett reciprocal come from k_split_lambda.
+// lambda and its Barrett reciprocal come from k_split_constants.
 __device__ __forceinline__ uint64_t gcd64(uint64_t a, uint64_t b) {
     while (b) {
         const uint64_t t = a % b;
@@ -242,19 +242,45 @@ struct SrcBbs16Seg : SrcBbs16 {
 // one chunk each, then BBS3 and BBS1, BBS7 and BBS2 for the two shift steps.
 __constant__ uint32_t c_bbs16_squarings[8] = {2, 2, 2, 1, 1, 1, 2, 1};
 
-// lambda(M) = lcm(p - 1, q - 1) of each lane's BBS modulus and its Barrett
-// reciprocal, once per lane (every segment's jump uses them):
-// lam[l] = lambda, lam[P + l] = barrett_mu(lambda); likewise the constants of
-// the residue form (every segment's run uses them).
-__global__ void __launch_bounds__(256) k_split_lambda(DevState src, uint64_t *lam, uint32_t *crt) {
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < src.P; l += stride) {
-        const uint64_t p = src.u32[F_P * src.P + l], q = src.u32[F_Q * src.P + l];
-        const uint64_t v = (p - 1) / gcd64(p - 1, q - 1) * (q - 1);
-        lam[l] = v;
-        lam[src.P + l] = barrett_mu(v);
-        crt_store(src, l, crt);
+// Once per lane, for every segment: the constants of the residue form
+// (crt_store) and, in kJumpWords fields behind them, what its jump starts from
+// (the Montgomery forms of y mod p, y mod q, 1 mod p and 1 mod q, p < q).
+// Lanes that do not take the residue form get lambda(M) = lcm(p - 1, q - 1)
+// and its Barrett reciprocal instead: lam[l] = lambda, lam[P + l] =
+// barrett_mu(lambda).
+constexpr int kJumpWords = 4;
+__global__ void __launch_bounds__(256) k_split_constants(DevState src, uint64_t *lam, uint32_t *crt) {
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, P = src.P;
+    for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < P; l += stride) {
+        const uint32_t a = src.u32[F_P * P + l], b = src.u32[F_Q * P + l];
+        if (crt_store(src, l, crt)) {
+            const uint64_t y = src.u64[G_Y * P + l];
+            const Mont32 Mp(min(a, b)), Mq(max(a, b));
+            uint32_t *jump = crt + kCrtWords * P + l;
+            jump[0] = Mp.to((uint32_t)(y % Mp.m));
+            jump[P] = Mq.to((uint32_t)(y % Mq.m));
+            jump[2 * P] = Mp.one;
+            jump[3 * P] = Mq.one;
+        } else {
+            const uint64_t p = a, q = b, v = (p - 1) / gcd64(p - 1, q - 1) * (q - 1);
+            lam[l] = v;
+            lam[P + l] = barrett_mu(v);
+        }
     }
+}
+
+// The lane's BBS state after `squarings` more squarings.
+__device__ __forceinline__ uint64_t bbs_jump_lane(const DevState &src, uint64_t l, uint64_t squarings,
+                                                  const uint64_t *lam, const uint32_t *crt) {
+    const uint64_t P = src.P;
+    CrtModulus C;
+    if (crt_load(src, l, crt, C)) {
+        const uint32_t *jump = crt + kCrtWords * P + l;
+        const Mont32 Mp(C.P.p, jump[2 * P]), Mq(C.Q.p, jump[3 * P]);
+        return C.value(Mp.from(squarings_m(C.P.p, Mp.one, jump[0], squarings)),
+                       Mq.from(squarings_m(C.Q.p, Mq.one, jump[P], squarings)));
+    }
+    return bbs_jump(src.u64[G_Y * P + l], src.u64[G_M * P + l], src.u64[G_MU * P + l], lam[l], lam[P + l], squarings);
 }
 
 // lambda(M) = lcm(p - 1, q - 1) of each 16-bit modulus M = p q (p != q primes,
@@ -281,14 +307,15 @@ __global__ void __launch_bounds__(256) k_split_lambda16(DevState src, uint32_t *
         }
 }
 
-__device__ __forceinline__ uint32_t pow_mod32(uint32_t a, uint64_t e, uint32_t m) {
-    uint64_t r = 1 % m, b = a % m;
+// a^e mod m for m < 2^16 (products fit 32 bits).
+__device__ __forceinline__ uint32_t pow_mod16(uint32_t a, uint64_t e, uint32_t m) {
+    uint32_t r = 1 % m, b = a % m;
     while (e) {
         if (e & 1ull) r = r * b % m;
         b = b * b % m;
         e >>= 1;
     }
-    return (uint32_t)r;
+    return r;
 }
 
 // Thread (k, l): segment k's lane l.  Copies the caller's lane (and the
@@ -296,7 +323,7 @@ __device__ __forceinline__ uint32_t pow_mod32(uint32_t a, uint64_t e, uint32_t m
 // k >= 1, clears slot and x.
 __global__ void __launch_bounds__(256) k_split_setup(DevState src, SegSpace seg, uint32_t K, uint64_t len,
                                                      int variant, int xl, OwnSave own, const uint32_t *lam16,
-                                                     const uint64_t *lam64) {
+                                                     const uint64_t *lam64, const uint32_t *crt) {
     const int nf = variant == CI_VAR_BBS16 ? kU32FieldsBbs16 : kU32Fields;
     const uint64_t total = (uint64_t)(K + (variant == CI_VAR_BBS16 ? 1 : 0)) * src.P;  // BBS16: slot K, a copy of the start
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -318,12 +345,11 @@ __global__ void __launch_bounds__(256) k_split_setup(DevState src, SegSpace seg,
         if (variant == CI_VAR_BBS16) {
             for (int g = 0; g < 8; ++g) {  // x <- x^(2^(c_g dist) mod lambda(M)) mod M
                 const uint32_t M = src.u32[(F_M16 + g) * src.P + l], lam = lam16[(uint64_t)g * src.P + l];
-                const uint32_t e = pow_mod32(2, c_bbs16_squarings[g] * dist, lam);
-                d.u32[(F_Y16 + g) * src.P + l] = pow_mod32(src.u32[(F_Y16 + g) * src.P + l], e, M);
+                const uint32_t e = pow_mod16(2, c_bbs16_squarings[g] * dist, lam);
+                d.u32[(F_Y16 + g) * src.P + l] = pow_mod16(src.u32[(F_Y16 + g) * src.P + l], e, M);
             }
         } else if (variant == CI_VAR_BBS) {
-            d.u64[G_Y * src.P + l] = bbs_jump(src.u64[G_Y * src.P + l], src.u64[G_M * src.P + l],
-                                              src.u64[G_MU * src.P + l], lam64[l], lam64[src.P + l], 11ull * dist);
+            d.u64[G_Y * src.P + l] = bbs_jump_lane(src, l, 11ull * dist, lam64, crt);
         } else if (xl == CI_XL_XOR128) {
             uint32_t v[4];
             for (int w = 0; w < 4; ++w) v[w] = src.u32[(F_A + w) * src.P + l];
@@ -361,18 +387,32 @@ __device__ __forceinline__ uint32_t mat_mul(uint32_t a_row, uint32_t b_row) {
     return c;
 }
 
-__device__ __forceinline__ uint32_t mat_vec(uint32_t m_row, uint32_t v) {
-    uint32_t r = 0;
+// (M v, N v) of two matrices and one vector, by the method of four Russians:
+// the warp tabulates the 16 XORs of each four consecutive lanes' words in
+// shared memory, and every lane looks its eight nibbles per row up (lanes that
+// read one group's table hit 16 banks).
+struct MatVecScratch {
+    uint32_t v[32], tab[8][16];
+};
+__device__ __forceinline__ uint2 mat_vec2(uint32_t m_row, uint32_t n_row, uint32_t v, MatVecScratch &sc) {
+    const int lane = threadIdx.x & 31;
+    sc.v[lane] = v;
+    __syncwarp();
+    const uint4 w = reinterpret_cast<const uint4 *>(sc.v)[lane >> 2];
+    const uint32_t h = ((lane & 1) ? w.z : 0u) ^ ((lane & 2) ? w.w : 0u);
+    reinterpret_cast<uint4 *>(sc.tab[lane >> 2])[lane & 3] = make_uint4(h, h ^ w.x, h ^ w.y, h ^ w.x ^ w.y);
+    __syncwarp();
+    uint2 r = make_uint2(0u, 0u);
 #pragma unroll
-    for (int m = 0; m < 32; ++m) {
-        const uint32_t b = __shfl_sync(kFull, v, m);
-        r ^= ((m_row >> m) & 1u) ? b : 0u;
+    for (int g = 0; g < 8; ++g) {
+        r.x ^= sc.tab[g][(m_row >> (4 * g)) & 15u];
+        r.y ^= sc.tab[g][(n_row >> (4 * g)) & 15u];
     }
     return r;
 }
 
 // The carry scan over the segments of one warp group, with one block of NW
-// (up to 16) warps per group.  c_j, the true (slot, x) at the start of segment j, obeys
+// (up to 32) warps per group.  c_j, the true (slot, x) at the start of segment j, obeys
 // c_j = e_{j-1} ^ H(c_{j-1}), c_0 = 0 (segment 0 ran from the true state),
 // with e_{j-1} the particular end of segment j-1 and H(s, x) = (Q s, x ^ S s).
 // Warp w owns steps j in [j0, j1) (m = ceil((K-1) / NW) each):
@@ -382,14 +422,20 @@ __device__ __forceinline__ uint32_t mat_vec(uint32_t m_row, uint32_t v) {
 //      whose pair (Q_m, T_m) follows from (Q, S) by the binary method on m
 //      (H^(a+b) = (Q_a Q_b, T_b ^ T_a Q_b));
 //   3. c_j = d_j ^ H^(j - j0 + 1)(c_{j0-1}).
+// The segments' words are loaded kCarryAhead steps at a time: a step is short
+// next to a memory round trip.  (32 streams in 256 segments: 118 us with
+// shuffled matrix-vector products, 64-step powers and one load ahead.)
 // Fix-up form (`own` == nullptr): c_j goes to starts[j].  Regenerate form:
 // c_j and the saved own words of segment j's start go into its state.
+constexpr int kCarryWarps = 32, kCarryAhead = 8;
 template <class Src>
-__global__ void __launch_bounds__(512) k_split_carry(SegSpace seg, uint32_t K, uint64_t len, uint2 *starts,
-                                                      OwnSave own) {
-    __shared__ uint32_t end_s[16][32], end_x[16][32];
+__global__ void __launch_bounds__(32 * kCarryWarps) k_split_carry(SegSpace seg, uint32_t K, uint64_t len, uint2 *starts,
+                                                                  OwnSave own) {
+    __shared__ uint32_t end_s[kCarryWarps][32], end_x[kCarryWarps][32];
+    __shared__ __align__(16) MatVecScratch scratch[kCarryWarps];
     const uint64_t g = blockIdx.x;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, NW = blockDim.x >> 5;
+    MatVecScratch &sc = scratch[w];
     const DevState s0 = seg.at(0);
     const uint64_t P = s0.P, l = g * 32 + lane;
     CI_WARP_CHECK(s0, g < P / 32, CHK_GROUP, g);  // g = blockIdx.x: every warp of the block returns together
@@ -400,8 +446,8 @@ __global__ void __launch_bounds__(512) k_split_carry(SegSpace seg, uint32_t K, u
     const uint32_t prow = (1u << s0.table[a1 * 32 + lane]) ^ (1u << s0.table[a2 * 32 + lane]);
     // Q = P^len, S = P + ... + P^len, by the bits of len from the top:
     // (Q, S) for k -> 2k: S <- S ^ Q S, Q <- Q Q; k -> k + 1: Q <- Q P, S <- S ^ Q.
-    uint32_t Q = 1u << lane, S = 0;
-    for (int b = 63; b >= 0; --b) {
+    uint32_t Q = prow, S = prow;
+    for (int b = 62 - __clzll((long long)len); b >= 0; --b) {
         S ^= mat_mul(Q, S);
         Q = mat_mul(Q, Q);
         if ((len >> b) & 1ull) {
@@ -411,32 +457,31 @@ __global__ void __launch_bounds__(512) k_split_carry(SegSpace seg, uint32_t K, u
     }
     const uint32_t m = (K - 1 + NW - 1) / NW;
     const uint32_t j0 = 1 + w * m, j1 = min(K, j0 + m);
-    // 1. local scan; segment ends loaded one step ahead
+    // 1. local scan
     uint32_t ds = 0, dx = 0;
-    if (j0 < j1) {
-        DevState d = seg.at(j0 - 1);
-        uint32_t es = d.u32[F_SLOT * P + l], ex = d.u32[F_X * P + l];
-        for (uint32_t j = j0; j < j1; ++j) {
-            uint32_t ns_e = 0, nx_e = 0;
-            if (j + 1 < j1) {
-                d = seg.at(j);
-                ns_e = d.u32[F_SLOT * P + l];
-                nx_e = d.u32[F_X * P + l];
+    for (uint32_t jb = j0; jb < j1; jb += kCarryAhead) {
+        uint32_t es[kCarryAhead], ex[kCarryAhead];
+#pragma unroll
+        for (int i = 0; i < kCarryAhead; ++i)
+            if (jb + i < j1) {
+                const DevState d = seg.at(jb + i - 1);
+                es[i] = d.u32[F_SLOT * P + l];
+                ex[i] = d.u32[F_X * P + l];
             }
-            const uint32_t ns = es ^ mat_vec(Q, ds);
-            dx = ex ^ dx ^ mat_vec(S, ds);
-            ds = ns;
-            starts[(uint64_t)j * P + l] = make_uint2(ds, dx);
-            es = ns_e;
-            ex = nx_e;
-        }
+#pragma unroll
+        for (int i = 0; i < kCarryAhead; ++i)
+            if (jb + i < j1) {
+                const uint2 hv = mat_vec2(Q, S, ds, sc);
+                dx = ex[i] ^ dx ^ hv.y;
+                ds = es[i] ^ hv.x;
+                starts[(uint64_t)(jb + i) * P + l] = make_uint2(ds, dx);
+            }
     }
     end_s[w][lane] = ds;
     end_x[w][lane] = dx;
-    __syncthreads();
     // 2. H^m and this warp's carry-in
-    uint32_t Qm = 1u << lane, Tm = 0;
-    for (int b = 31; b >= 0; --b) {
+    uint32_t Qm = Q, Tm = S;
+    for (int b = 30 - __clz((int)m); b >= 0; --b) {
         Tm ^= mat_mul(Tm, Qm);
         Qm = mat_mul(Qm, Qm);
         if ((m >> b) & 1u) {
@@ -444,28 +489,38 @@ __global__ void __launch_bounds__(512) k_split_carry(SegSpace seg, uint32_t K, u
             Tm = S ^ mat_mul(Tm, Q);
         }
     }
+    __syncthreads();
     uint32_t cs = 0, cx = 0;
     for (int v = 0; v < w; ++v) {
-        const uint32_t ns = end_s[v][lane] ^ mat_vec(Qm, cs);
-        cx = end_x[v][lane] ^ cx ^ mat_vec(Tm, cs);
-        cs = ns;
+        const uint2 hv = mat_vec2(Qm, Tm, cs, sc);
+        cx = end_x[v][lane] ^ cx ^ hv.y;
+        cs = end_s[v][lane] ^ hv.x;
     }
     // 3. true starts of this warp's segments
-    for (uint32_t j = j0; j < j1; ++j) {
-        const uint32_t ns = mat_vec(Q, cs);
-        cx ^= mat_vec(S, cs);
-        cs = ns;
-        const uint2 dj = starts[(uint64_t)j * P + l];
-        const uint32_t ts = dj.x ^ cs, tx = dj.y ^ cx;
-        if (!own.u32) {
-            starts[(uint64_t)j * P + l] = make_uint2(ts, tx);
-        } else {
-            const DevState d = seg.at(j);
-            d.u32[F_SLOT * P + l] = ts;
-            d.u32[F_X * P + l] = tx;
-            for (int f = 0; f < own.count; ++f) d.u32[(own.first + f) * P + l] = own.u32[((uint64_t)f * K + j) * P + l];
-            if (own.u64) d.u64[G_Y * P + l] = own.u64[(uint64_t)j * P + l];
-        }
+    for (uint32_t jb = j0; jb < j1; jb += kCarryAhead) {
+        uint2 dj[kCarryAhead];
+#pragma unroll
+        for (int i = 0; i < kCarryAhead; ++i)
+            if (jb + i < j1) dj[i] = starts[(uint64_t)(jb + i) * P + l];
+#pragma unroll
+        for (int i = 0; i < kCarryAhead; ++i)
+            if (jb + i < j1) {
+                const uint32_t j = jb + i;
+                const uint2 hv = mat_vec2(Q, S, cs, sc);
+                cs = hv.x;
+                cx ^= hv.y;
+                const uint32_t ts = dj[i].x ^ cs, tx = dj[i].y ^ cx;
+                if (!own.u32) {
+                    starts[(uint64_t)j * P + l] = make_uint2(ts, tx);
+                } else {
+                    const DevState d = seg.at(j);
+                    d.u32[F_SLOT * P + l] = ts;
+                    d.u32[F_X * P + l] = tx;
+                    for (int f = 0; f < own.count; ++f)
+                        d.u32[(own.first + f) * P + l] = own.u32[((uint64_t)f * K + j) * P + l];
+                    if (own.u64) d.u64[G_Y * P + l] = own.u64[(uint64_t)j * P + l];
+                }
+            }
     }
 }
 
@@ -477,7 +532,11 @@ __global__ void __launch_bounds__(512) k_split_carry(SegSpace seg, uint32_t K, u
 // as 16-byte row segments (V4) or words.  Another warp wrote those outputs,
 // so they are read through L2 (ld.global.cg).  Returns H(c) = (h, acc) at the
 // segment's end.
-template <bool V4>
+// kAhead: the tile's outputs are loaded before its steps, whose 32 serial
+// shuffles then hide the round trip (the fix-ups as a kernel of their own; among
+// the squaring warps of the one-launch form other warps hide it, and the 32
+// registers are not to be had).
+template <bool V4, bool kAhead>
 __device__ __forceinline__ uint2 fix_segment(uint2 c, int p1, int p2, uint64_t n, uint32_t *base, uint64_t row0,
                                              uint64_t S, uint64_t ld, uint4 *tile) {
     const int lane = threadIdx.x & 31;
@@ -490,6 +549,15 @@ __device__ __forceinline__ uint2 fix_segment(uint2 c, int p1, int p2, uint64_t n
     };
     const uint64_t nfull = n - n % 32;
     for (uint64_t i0 = 0; i0 < nfull; i0 += 32) {
+        uint4 ahead[kAhead ? 8 : 1];
+        if (V4 && kAhead) {
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) {
+                const int r = 4 * kk + lane / 8;
+                if (row0 + r < S)
+                    ahead[kk] = __ldcg(reinterpret_cast<const uint4 *>(base + (row0 + r) * ld + i0 + 4 * (lane % 8)));
+            }
+        }
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             uint4 f;
@@ -507,7 +575,7 @@ __device__ __forceinline__ uint2 fix_segment(uint2 c, int p1, int p2, uint64_t n
                 if (row0 + r < S) {
                     uint4 *p = reinterpret_cast<uint4 *>(base + (row0 + r) * ld + i0 + 4 * cc);
                     const uint4 v = tile[r * 8 + (cc ^ (r & 7))];
-                    uint4 o = __ldcg(p);
+                    uint4 o = kAhead ? ahead[kk] : __ldcg(p);
                     o.x ^= v.x;
                     o.y ^= v.y;
                     o.z ^= v.z;
@@ -551,7 +619,7 @@ __global__ void __launch_bounds__(256) k_split_fixup(SegSpace seg, const uint2 *
     const DevState s0 = seg.at(0);
     const uint64_t P = s0.P;
     const uint64_t units = (uint64_t)(K - 1) * groups;
-    for (uint64_t u = (uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5); u < units; u += (uint64_t)gridDim.x * 8) {
+    for (uint64_t u = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; u < units; u += (uint64_t)gridDim.x * 8) {
         const uint64_t k = 1 + u / groups, g = u % groups, l = g * 32 + lane;
         CI_WARP_CHECK(s0, k < K && g < P / 32, CHK_SEGMENT, k);
         CI_WARP_CHECK(s0, col0 + k * len + (k + 1 == K ? len_last : len) <= ld, CHK_SEG_COLS, k);
@@ -560,7 +628,7 @@ __global__ void __launch_bounds__(256) k_split_fixup(SegSpace seg, const uint2 *
         src.load(s0, l);
         int a1, a2;
         src.arrays(s0, l, a1, a2);
-        const uint2 hk = fix_segment<V4>(starts[k * P + l], s0.table[a1 * 32 + lane], s0.table[a2 * 32 + lane],
+        const uint2 hk = fix_segment<V4, true>(starts[k * P + l], s0.table[a1 * 32 + lane], s0.table[a2 * 32 + lane],
                                          k + 1 == K ? len_last : len, out + col0 + k * len, g * 32, s0.S, ld, tile);
         if (k + 1 == K) {
             const DevState d = seg.at(K - 1);
@@ -671,6 +739,7 @@ __global__ void __launch_bounds__(256) k_consume_rows(const uint32_t *rows, uint
 // ------------------------------------------------ host side
 constexpr uint32_t kMaxSegments = kSplitMaxSegments;
 constexpr uint64_t kMinSegment = 256;       // iterations per segment (auto choice, BBS)
+constexpr uint64_t kMinShortSegment = 64;   // ... while they do not fill the GPU (BBS sources)
 constexpr uint64_t kMinAutoSegment = 1024;  // ... xor-likes, and when a single call splits on its own
 constexpr uint64_t kScratchWords = 1ull << 29;  // scratch outputs of a BBS-source consumer call (2 GiB)
 // Written BBS-source outputs take the one-launch fix-up form from this many
@@ -805,7 +874,7 @@ __global__ void __launch_bounds__(256, split_min_blocks<Src>()) k_split_run_fix(
                 p1 = s0.table[a1 * 32 + lane];
                 p2 = s0.table[a2 * 32 + lane];
             }
-            const uint2 hk = fix_segment<SINK == SINK_V4>(__ldcg(starts + k * P + l), p1, p2,
+            const uint2 hk = fix_segment<SINK == SINK_V4, false>(__ldcg(starts + k * P + l), p1, p2,
                                                           k + 1 == K ? len_last : len, out + col0 + k * len, g * 32,
                                                           s0.S, ld, tile);
             const DevState d = seg.at(k);
@@ -917,6 +986,11 @@ uint64_t split_auto_bbs(const ci_states_s &h, uint64_t n, int sink) {
         // form, four in the three-launch form; segments of at least 256.
         K = groups >= kOneLaunchGroupsPerSm * sms ? (400 * sms + groups / 2) / groups : 160 * sms / groups;
         K = std::min<uint64_t>(K, n / kMinSegment);
+        // ... or shorter, down to 64, while the segments are fewer than the
+        // resident warps (24 per SM): 32 streams x 4096 82 us, 103 from 128
+        // on, 309 from 256 on; x 65536 149 us, 171 down to 32; 1000 x 16384
+        // 295 us, 337 up to 16 warps per SM.
+        K = std::max<uint64_t>(K, std::min<uint64_t>(n / kMinShortSegment, 24 * sms / groups));
     } else {
         // Larger consumer calls generate twice (pass 1, then pass 2 from the
         // true starts): only states that fill less than about two waves.
@@ -938,9 +1012,11 @@ uint64_t split_auto(const ci_states_s &h, uint64_t n, int sink) {
         // so only states of at most one warp group per SM gain from more
         // warps (measured, written: 1 group 39x, 32 groups 7x, 128 groups
         // 2.8x faster; 512 groups slower), with about two waves of the split
-        // kernels' 16 resident warps per SM and segments of at least 256.
+        // kernels' 16 resident warps per SM and segments of at least 256, or
+        // 64 while they fill less than one wave.
         if (groups > sms) return 1;
         uint64_t K = std::min<uint64_t>(sms * 32 / groups, n / kMinSegment);
+        K = std::max<uint64_t>(K, std::min<uint64_t>(sms * 16 / groups, n / kMinShortSegment));
         K = std::min<uint64_t>(K, kMaxSegments);
         if (K <= 1) return 1;
         const uint64_t len = ((n + K - 1) / K + 31) / 32 * 32;
@@ -981,7 +1057,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
     // twice; larger calls take the regenerate form below.
     if (sink != CI_SINK_WRITTEN && (bbs || b16) && h->S <= kScratchWords / n) {
         uint32_t *rows = nullptr;
-        if ((e = cudaMallocAsync(reinterpret_cast<void **>(&rows), 4 * h->S * n, stream)) != cudaSuccess)
+        if ((e = workspace_alloc(reinterpret_cast<void **>(&rows), 4 * h->S * n, stream)) != cudaSuccess)
             return cuda_fail(e, "scratch outputs");
         ci_status st = CI_OK;
         if (sink == CI_SINK_DIGEST && (e = cudaMemsetAsync(aux, 0, 8 * h->S, stream)) != cudaSuccess)
@@ -1017,9 +1093,9 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
     const int own_first = b16 ? (int)F_Y16 : (int)F_A, own_count = b16 ? 8 : kOwnWords;
     const uint64_t res_bytes = 8ull * K * h->P;  // per-segment consumer results
     const uint64_t own_bytes = fixup ? 0 : (4ull * own_count + (bbs ? 8ull : 0ull)) * K * h->P;
-    const uint64_t lam_bytes = b16 ? 4ull * 8 * h->P : bbs ? (16ull + 4ull * kCrtWords) * h->P : 0;
+    const uint64_t lam_bytes = b16 ? 4ull * 8 * h->P : bbs ? (16ull + 4ull * (kCrtWords + kJumpWords)) * h->P : 0;
     uint8_t *ws = nullptr;
-    if ((e = cudaMallocAsync(reinterpret_cast<void **>(&ws), stride * slots + 2 * res_bytes + own_bytes + lam_bytes,
+    if ((e = workspace_alloc(reinterpret_cast<void **>(&ws), stride * slots + 2 * res_bytes + own_bytes + lam_bytes,
                              stream)) != cudaSuccess)
         return cuda_fail(e, "workspace");
     uint64_t *res1 = reinterpret_cast<uint64_t *>(ws + stride * slots);
@@ -1034,22 +1110,22 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
     uint64_t *lam64 = bbs ? reinterpret_cast<uint64_t *>(after + own_bytes) : nullptr;
     uint32_t *crt = bbs ? reinterpret_cast<uint32_t *>(lam64 + 2 * h->P) : nullptr;  // residue-form constants
 
-    // Handles over the segment states (host copies of the caller's, moved).
-    std::vector<ci_states_s> segs(slots, *h);
-    for (uint64_t k = 0; k < slots; ++k) {
-        segs[k].dev = ws + k * stride;
-        segs[k].owns = false;
-    }
+    // Views over the segment states (the caller's, moved).
+    auto segment = [&](uint64_t k) {
+        ci_states_s moved = *h;
+        moved.dev = ws + k * stride;
+        return moved.view();
+    };
     SegSpace sp;
-    sp.v0 = segs[0].view();
+    sp.v0 = segment(0);
     sp.stride = stride;
     const DevState src = h->view();
 
     ci_status st = CI_OK;
     if (b16) k_split_lambda16<<<split_block_count(h->P), 256, 0, stream>>>(src, lam16);
-    if (bbs) k_split_lambda<<<split_block_count(h->P), 256, 0, stream>>>(src, lam64, crt);
+    if (bbs) k_split_constants<<<split_block_count(h->P), 256, 0, stream>>>(src, lam64, crt);
     k_split_setup<<<split_block_count(slots * h->P), 256, 0, stream>>>(src, sp, (uint32_t)K, len, h->variant, h->xl,
-                                                                       own, lam16, lam64);
+                                                                       own, lam16, lam64, crt);
     if ((e = cudaGetLastError()) != cudaSuccess) st = cuda_fail(e, "split setup");
 
     if (st == CI_OK && fixup && groups >= kOneLaunchGroupsPerSm * (uint64_t)sm_count()) {
@@ -1072,7 +1148,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
                                                                         starts, events, next_unit, crt, stream);
         }
         if (e == cudaSuccess) {
-            k_split_copy_back<<<split_block_count(h->P), 256, 0, stream>>>(src, segs[K - 1].view(), h->variant);
+            k_split_copy_back<<<split_block_count(h->P), 256, 0, stream>>>(src, segment(K - 1), h->variant);
             e = cudaGetLastError();
         }
         if (e != cudaSuccess) st = cuda_fail(e, "split pass 1 with fix-ups");
@@ -1090,7 +1166,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
     }
     uint2 *starts = reinterpret_cast<uint2 *>(res1);  // K * P (slot, x) pairs, after pass 1
     if (st == CI_OK) {
-        const unsigned threads = 32u * (unsigned)std::min<uint64_t>(16, K - 1);
+        const unsigned threads = 32u * (unsigned)std::min<uint64_t>(kCarryWarps, K - 1);
         if (bbs)
             k_split_carry<SrcBbs><<<(unsigned)groups, threads, 0, stream>>>(sp, (uint32_t)K, len, starts, own);
         else if (b16)
@@ -1101,7 +1177,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
     }
     if (st == CI_OK && fixup) {  // homogeneous parts into segments 1 .. K-1, then the final state
         const bool v4 = (reinterpret_cast<uintptr_t>(out) & 15u) == 0 && ld % 4 == 0 && col0 % 4 == 0;
-        const int blocks = split_block_count((K - 1) * groups * 32);
+        const int blocks = (int)std::min<uint64_t>((K - 1) * groups, (uint64_t)sm_count() * 8);  // spread over every SM
         if (bbs)
             v4 ? k_split_fixup<SrcBbs, true><<<blocks, 256, 0, stream>>>(sp, starts, (uint32_t)K, len, len_last,
                                                                           groups, out, ld, col0)
@@ -1113,7 +1189,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
                : k_split_fixup<SrcBbs16Seg, false><<<blocks, 256, 0, stream>>>(sp, starts, (uint32_t)K, len,
                                                                                 len_last, groups, out, ld, col0);
         if ((e = cudaGetLastError()) == cudaSuccess)
-            k_split_copy_back<<<split_block_count(h->P), 256, 0, stream>>>(src, segs[K - 1].view(), h->variant);
+            k_split_copy_back<<<split_block_count(h->P), 256, 0, stream>>>(src, segment(K - 1), h->variant);
         if ((e = cudaGetLastError()) != cudaSuccess) st = cuda_fail(e, "split fix-up");
         cudaFreeAsync(ws, stream);
         return st;
@@ -1126,7 +1202,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
         if (e != cudaSuccess) st = cuda_fail(e, "split pass 2");
     }
     if (st == CI_OK) {
-        k_split_copy_back<<<split_block_count(h->P), 256, 0, stream>>>(src, segs[K - 1].view(), h->variant);
+        k_split_copy_back<<<split_block_count(h->P), 256, 0, stream>>>(src, segment(K - 1), h->variant);
         if (!written)
             k_split_combine<<<(unsigned)((h->S + 255) / 256), 256, 0, stream>>>(res3, aux, h->P, h->S, (uint32_t)K,
                                                                                 len, len_last, sink == CI_SINK_DIGEST);

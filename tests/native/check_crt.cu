@@ -86,6 +86,32 @@ int main() {
     }
     printf("square modulo p q: %ld of %ld differ (%ld moduli)\n", bad, n, taken);
     all += bad;
+
+    // squarings_m and pow2_mod_order over Blum primes and primes = 1 mod 4
+    bad = n = 0;
+    for (int k = 0; k < 400; ++k) {
+        uint32_t p = (k < 20 ? (k < 10 ? lo : hi - 4000u) + 2u * (uint32_t)(g() % 1000) : lo + (uint32_t)(g() % (hi - lo + 1))) | 1u;
+        while (!is_prime_u32(p)) p += 2;
+        if (p > hi) continue;
+        const Mont32 M(p);
+        for (int j = 0; j < 60; ++j) {
+            const uint64_t e = j < 40 ? 1 + (uint64_t)j : 1 + (g() >> (20 + g() % 40));
+            u128 r = 1, b = 2;
+            for (uint64_t t = e; t; t >>= 1) {
+                if (t & 1) r = r * b % (p - 1);
+                b = b * b % (p - 1);
+            }
+            bad += pow2_mod_order(p, e) != (uint32_t)r, ++n;
+            const uint32_t x = (uint32_t)(j % 7 == 0 ? 0 : g() % p);
+            uint32_t y = x;
+            if (e <= 64) {
+                for (uint64_t t = 0; t < e; ++t) y = (uint32_t)((uint64_t)y * y % p);
+                bad += M.from(squarings_m(p, M.one, M.to(x), e)) != y, ++n;
+            }
+        }
+    }
+    printf("repeated squarings: %ld of %ld differ\n", bad, n);
+    all += bad;
     if (all || taken < 1000) return 1;
     printf("ok\n");
     return 0;
