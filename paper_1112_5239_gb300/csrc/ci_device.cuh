@@ -470,7 +470,7 @@ struct SrcBbs16 {
 };
 
 // ----------------------------------------------------- generation loop
-enum Sink { SINK_V4 = 0, SINK_SCALAR = 1, SINK_QC = 2, SINK_DIGEST = 3 };
+enum Sink { SINK_V4 = 0, SINK_SCALAR = 1, SINK_QC = 2, SINK_DIGEST = 3, SINK_NONE = 4 };  // NONE: the end state alone
 
 // Multiplier of the per-stream output digest D <- D * K + x (mod 2^64),
 // an odd 64-bit constant.
@@ -671,7 +671,10 @@ __device__ __forceinline__ void warp_loop(Lane<Src> &s, const DevState &st, uint
     uint64_t hits = 0;
 
     for (uint64_t i0 = 0; i0 < nfull; i0 += KT) {
-        if (SINK == SINK_DIGEST) {
+        if (SINK == SINK_NONE) {
+#pragma unroll(Src::kHeavy ? 1 : 32)
+            for (int k = 0; k < 32; ++k) s.step();
+        } else if (SINK == SINK_DIGEST) {
 #pragma unroll(Src::kHeavy ? 1 : 32)
             for (int k = 0; k < 32; ++k) hits = hits * kDigestMul + s.step();
         } else if (SINK == SINK_QC) {
@@ -712,7 +715,9 @@ __device__ __forceinline__ void warp_loop(Lane<Src> &s, const DevState &st, uint
 
     const int rem = (int)(n - nfull);
     if (rem) {
-        if (SINK == SINK_DIGEST) {
+        if (SINK == SINK_NONE) {
+            for (int k = 0; k < rem; ++k) s.step();
+        } else if (SINK == SINK_DIGEST) {
             for (int k = 0; k < rem; ++k) hits = hits * kDigestMul + s.step();
         } else if (SINK == SINK_QC) {
             uint32_t m = 0;

@@ -31,8 +31,7 @@
 //      k_split_fixup runs all fix-ups at once;
 //   4. otherwise (xor-like outputs are cheaper to generate again than to
 //      read back, and consumer sinks have no outputs to fix): pass 1
-//      (k_split_run) runs segments 0 .. K-2 into a digest sink (only their
-//      end states are needed); k_split_carry, one block per warp group,
+//      (k_split_run) runs segments 0 .. K-2 for their end states alone; k_split_carry, one block per warp group,
 //      scans the segments: the true start of segment k is its predecessor's
 //      particular end plus (Q s_a, x_a ^ S s_a) with Q = P^len,
 //      S = P + ... + P^len (a chunked parallel scan over up to 32 warps);
@@ -40,6 +39,7 @@
 //      own words k_split_setup jumped to, into the sink;
 //   5. the last segment's end state becomes the caller's state, and the
 //      per-segment quarter-circle counts or digests are combined.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -61,11 +61,17 @@ using namespace dev;
 // ------------------------------------------------ xor-like jump tables
 // Column form of the GF(2)-linear step A of a xor-like with W 32-bit words:
 // T[i][j] = A^(2^i) e_j, so v <- A^(2^i) v is the XOR of the columns j at the
-// set bits of v.  Built on the device from the sources' own next().
+// set bits of v.  Built on the device from the sources' own next(); the jumps
+// use the XORs of each four columns, N[i][g][b] = XOR of T[i][4 g + k] over
+// the set bits k of b, so a level takes 8 W lookups instead of 32 W
+// conditional XORs (256 xor128 streams in 64 segments: setup 52 us by columns).
 constexpr int kJumpLevels = 64;
-__device__ uint32_t g_jump_xor128[kJumpLevels][128][4];
-__device__ uint32_t g_jump_xor64[kJumpLevels][64][2];
-__device__ uint32_t g_jump_xs32[kJumpLevels][32][1];
+__device__ uint32_t g_columns_xor128[kJumpLevels][128][4];
+__device__ uint32_t g_columns_xor64[kJumpLevels][64][2];
+__device__ uint32_t g_columns_xs32[kJumpLevels][32][1];
+__device__ __align__(16) uint32_t g_jump_xor128[kJumpLevels][32][16][4];
+__device__ __align__(16) uint32_t g_jump_xor64[kJumpLevels][16][16][2];
+__device__ __align__(16) uint32_t g_jump_xs32[kJumpLevels][8][16][1];
 
 template <int W>
 __device__ __forceinline__ void step_words(uint32_t (&v)[W]) {
@@ -116,18 +122,71 @@ __global__ void k_build_jump(uint32_t (*T)[32 * W][W]) {
     }
 }
 
+// Thread (i, g, b) of the nibble tables.
 template <int W>
-__device__ __forceinline__ void jump_words(uint32_t (&v)[W], uint64_t dist, const uint32_t (*T)[32 * W][W]) {
+__global__ void __launch_bounds__(256) k_build_nibbles(const uint32_t (*T)[32 * W][W], uint32_t (*N)[8 * W][16][W]) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= kJumpLevels * 8 * W * 16) return;
+    const int b = t % 16, g = t / 16 % (8 * W), i = t / (16 * 8 * W);
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        uint32_t r = 0;
+        for (int k = 0; k < 4; ++k)
+            if ((b >> k) & 1) r ^= T[i][4 * g + k][w];
+        N[i][g][b][w] = r;
+    }
+}
+
+template <int W>
+struct JumpWord {
+    using type = uint32_t;
+};
+template <>
+struct JumpWord<2> {
+    using type = uint2;
+};
+template <>
+struct JumpWord<4> {
+    using type = uint4;
+};
+
+template <int W>
+__device__ __forceinline__ void jump_words(uint32_t (&v)[W], uint64_t dist, const uint32_t (*N)[8 * W][16][W]) {
+    using Word = typename JumpWord<W>::type;
     for (int i = 0; dist; ++i, dist >>= 1) {
         if (!(dist & 1ull)) continue;
         uint32_t r[W] = {};
-        for (int b = 0; b < 32 * W; ++b)
-            if ((v[b / 32] >> (b % 32)) & 1u)
 #pragma unroll
-                for (int w = 0; w < W; ++w) r[w] ^= T[i][b][w];
+        for (int w = 0; w < W; ++w)
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+                const Word e = __ldg(reinterpret_cast<const Word *>(N[i][8 * w + g][(v[w] >> (4 * g)) & 15u]));
+                if constexpr (W == 1) r[0] ^= e;
+                if constexpr (W >= 2) {
+                    r[0] ^= e.x;
+                    r[1] ^= e.y;
+                }
+                if constexpr (W == 4) {
+                    r[2] ^= e.z;
+                    r[3] ^= e.w;
+                }
+            }
 #pragma unroll
         for (int w = 0; w < W; ++w) v[w] = r[w];
     }
+}
+
+// Builds one source's tables on `stream`.
+template <int W>
+cudaError_t build_jump_tables(const void *columns_symbol, const void *jump_symbol, cudaStream_t stream) {
+    void *columns = nullptr, *jump = nullptr;
+    cudaError_t e = cudaGetSymbolAddress(&columns, columns_symbol);
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(&jump, jump_symbol);
+    if (e != cudaSuccess) return e;
+    k_build_jump<W><<<1, 32 * W, 0, stream>>>(static_cast<uint32_t(*)[32 * W][W]>(columns));
+    k_build_nibbles<W><<<(kJumpLevels * 8 * W * 16 + 255) / 256, 256, 0, stream>>>(
+        static_cast<const uint32_t(*)[32 * W][W]>(columns), static_cast<uint32_t(*)[8 * W][16][W]>(jump));
+    return cudaGetLastError();
 }
 
 std::mutex g_tables_mu;
@@ -140,14 +199,9 @@ cudaError_t ensure_jump_tables(cudaStream_t stream) {
     std::lock_guard<std::mutex> lk(g_tables_mu);
     if ((int)g_tables_ready.size() <= dev) g_tables_ready.resize(dev + 1, 0);
     if (g_tables_ready[dev]) return cudaSuccess;
-    void *p128 = nullptr, *p64 = nullptr, *p32 = nullptr;
-    if ((e = cudaGetSymbolAddress(&p128, g_jump_xor128)) != cudaSuccess) return e;
-    if ((e = cudaGetSymbolAddress(&p64, g_jump_xor64)) != cudaSuccess) return e;
-    if ((e = cudaGetSymbolAddress(&p32, g_jump_xs32)) != cudaSuccess) return e;
-    k_build_jump<4><<<1, 128, 0, stream>>>(static_cast<uint32_t(*)[128][4]>(p128));
-    k_build_jump<2><<<1, 64, 0, stream>>>(static_cast<uint32_t(*)[64][2]>(p64));
-    k_build_jump<1><<<1, 32, 0, stream>>>(static_cast<uint32_t(*)[32][1]>(p32));
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = build_jump_tables<4>(g_columns_xor128, g_jump_xor128, stream)) != cudaSuccess) return e;
+    if ((e = build_jump_tables<2>(g_columns_xor64, g_jump_xor64, stream)) != cudaSuccess) return e;
+    if ((e = build_jump_tables<1>(g_columns_xs32, g_jump_xs32, stream)) != cudaSuccess) return e;
     // Wait once, so that calls on any stream of this device find finished tables.
     if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return e;
     g_tables_ready[dev] = 1;
@@ -287,24 +341,23 @@ __device__ __forceinline__ uint64_t bbs_jump_lane(const DevState &src, uint64_t 
 // as seeded), by trial division; lam[k * P + l] for generator k of lane l.
 __global__ void __launch_bounds__(256) k_split_lambda16(DevState src, uint32_t *lam) {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < src.P; l += stride)
-        for (int k = 0; k < 8; ++k) {
-            const uint32_t M = src.u32[(F_M16 + k) * src.P + l];
-            uint32_t p = M;  // a prime M (not seeded) gets lambda = M - 1
-            for (uint32_t d = 3; d * d <= M; d += 2)
-                if (M % d == 0) {
-                    p = d;
-                    break;
-                }
-            const uint32_t q = p == M ? 2u : M / p;
-            uint32_t a = p - 1, b = q - 1;
-            while (b) {
-                const uint32_t t = a % b;
-                a = b;
-                b = t;
+    for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < 8 * src.P; t += stride) {
+        const uint32_t M = src.u32[F_M16 * src.P + t];  // generator t / P of lane t % P
+        uint32_t p = M;  // a prime M (not seeded) gets lambda = M - 1
+        for (uint32_t d = 3; d * d <= M; d += 2)
+            if (M % d == 0) {
+                p = d;
+                break;
             }
-            lam[(uint64_t)k * src.P + l] = (p - 1) / a * (q - 1);
+        const uint32_t q = p == M ? 2u : M / p;
+        uint32_t a = p - 1, b = q - 1;
+        while (b) {
+            const uint32_t t2 = a % b;
+            a = b;
+            b = t2;
         }
+        lam[t] = (p - 1) / a * (q - 1);
+    }
 }
 
 // a^e mod m for m < 2^16 (products fit 32 bits).
@@ -333,7 +386,9 @@ __global__ void __launch_bounds__(256) k_split_setup(DevState src, SegSpace seg,
         for (uint64_t w = l; w < kTableBytes / 4; w += src.P)
             reinterpret_cast<uint32_t *>(const_cast<uint8_t *>(d.table))[w] =
                 reinterpret_cast<const uint32_t *>(src.table)[w];
-        for (int f = 0; f < nf; ++f) d.u32[f * src.P + l] = src.u32[f * src.P + l];
+#pragma unroll
+        for (int f = 0; f < kU32FieldsBbs16; ++f)
+            if (f < nf) d.u32[f * src.P + l] = src.u32[f * src.P + l];
         if (variant == CI_VAR_BBS)
             for (int f = 0; f < kU64Fields; ++f) d.u64[f * src.P + l] = src.u64[f * src.P + l];
         if (variant == CI_VAR_BBS16)  // the arrays the call chose at its start, for every segment
@@ -411,8 +466,10 @@ __device__ __forceinline__ uint2 mat_vec2(uint32_t m_row, uint32_t n_row, uint32
     return r;
 }
 
-// The carry scan over the segments of one warp group, with one block of NW
-// (up to 32) warps per group.  c_j, the true (slot, x) at the start of segment j, obeys
+// The carry scan over the segments of one warp group, with a cluster of
+// kCarryBlocks blocks, NW = 32 warps together, per group: a step is some 20
+// shared-memory operations of a warp, which 32 warps on one SM queued for (60
+// us for 1024 segments of one group).  c_j, the true (slot, x) at the start of segment j, obeys
 // c_j = e_{j-1} ^ H(c_{j-1}), c_0 = 0 (segment 0 ran from the true state),
 // with e_{j-1} the particular end of segment j-1 and H(s, x) = (Q s, x ^ S s).
 // Warp w owns steps j in [j0, j1) (m = ceil((K-1) / NW) each):
@@ -427,18 +484,22 @@ __device__ __forceinline__ uint2 mat_vec2(uint32_t m_row, uint32_t n_row, uint32
 // shuffled matrix-vector products, 64-step powers and one load ahead.)
 // Fix-up form (`own` == nullptr): c_j goes to starts[j].  Regenerate form:
 // c_j and the saved own words of segment j's start go into its state.
-constexpr int kCarryWarps = 32, kCarryAhead = 8;
+constexpr int kCarryBlocks = 8, kCarryWarps = 4, kCarryAhead = 8;
 template <class Src>
-__global__ void __launch_bounds__(32 * kCarryWarps) k_split_carry(SegSpace seg, uint32_t K, uint64_t len, uint2 *starts,
-                                                                  OwnSave own) {
-    __shared__ uint32_t end_s[kCarryWarps][32], end_x[kCarryWarps][32];
+__global__ void __cluster_dims__(kCarryBlocks, 1, 1) __launch_bounds__(32 * kCarryWarps)
+    k_split_carry(SegSpace seg, uint32_t K, uint64_t len, uint2 *starts, OwnSave own) {
+    constexpr int NW = kCarryBlocks * kCarryWarps;
+    __shared__ uint2 ends[kCarryWarps][32];  // this block's warps' (slot, x)
+    __shared__ uint2 all[NW][32];            // every warp's
     __shared__ __align__(16) MatVecScratch scratch[kCarryWarps];
-    const uint64_t g = blockIdx.x;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, NW = blockDim.x >> 5;
-    MatVecScratch &sc = scratch[w];
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const uint64_t g = blockIdx.x / kCarryBlocks;
+    const int lane = threadIdx.x & 31, bw = threadIdx.x >> 5, w = (int)cluster.block_rank() * kCarryWarps + bw;
+    MatVecScratch &sc = scratch[bw];
     const DevState s0 = seg.at(0);
     const uint64_t P = s0.P, l = g * 32 + lane;
-    CI_WARP_CHECK(s0, g < P / 32, CHK_GROUP, g);  // g = blockIdx.x: every warp of the block returns together
+    CI_WARP_CHECK(s0, g < P / 32, CHK_GROUP, g);  // the same in the whole cluster: its warps return together
     Src src;
     src.load(s0, l);
     int a1, a2;
@@ -477,8 +538,7 @@ __global__ void __launch_bounds__(32 * kCarryWarps) k_split_carry(SegSpace seg, 
                 starts[(uint64_t)(jb + i) * P + l] = make_uint2(ds, dx);
             }
     }
-    end_s[w][lane] = ds;
-    end_x[w][lane] = dx;
+    ends[bw][lane] = make_uint2(ds, dx);
     // 2. H^m and this warp's carry-in
     uint32_t Qm = Q, Tm = S;
     for (int b = 30 - __clz((int)m); b >= 0; --b) {
@@ -489,12 +549,15 @@ __global__ void __launch_bounds__(32 * kCarryWarps) k_split_carry(SegSpace seg, 
             Tm = S ^ mat_mul(Tm, Q);
         }
     }
-    __syncthreads();
+    cluster.sync();
+    for (int v = bw; v < NW; v += kCarryWarps)
+        all[v][lane] = cluster.map_shared_rank(&ends[0][0], v / kCarryWarps)[(v % kCarryWarps) * 32 + lane];
+    cluster.sync();  // every warp's ends are here, and no block is read any more
     uint32_t cs = 0, cx = 0;
     for (int v = 0; v < w; ++v) {
         const uint2 hv = mat_vec2(Qm, Tm, cs, sc);
-        cx = end_x[v][lane] ^ cx ^ hv.y;
-        cs = end_s[v][lane] ^ hv.x;
+        cx ^= all[v][lane].y ^ hv.y;
+        cs = all[v][lane].x ^ hv.x;
     }
     // 3. true starts of this warp's segments
     for (uint32_t jb = j0; jb < j1; jb += kCarryAhead) {
@@ -642,17 +705,18 @@ __global__ void __launch_bounds__(256) k_split_fixup(SegSpace seg, const uint2 *
 // generation never changes, stays the caller's).  CI_VAR_BBS16: generator k
 // (state and modulus) moves to place k + 1, the call's one rotation.
 __global__ void __launch_bounds__(256) k_split_copy_back(DevState dst, DevState last, int variant) {
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < dst.P; l += stride) {
-        for (int f = 0; f < kU32Fields; ++f)
-            if (f != F_SEL) dst.u32[f * dst.P + l] = last.u32[f * dst.P + l];
-        if (variant == CI_VAR_BBS16)
-            for (int k = 0; k < 8; ++k) {
-                dst.u32[(F_Y16 + (k + 1) % 8) * dst.P + l] = last.u32[(F_Y16 + k) * dst.P + l];
-                dst.u32[(F_M16 + (k + 1) % 8) * dst.P + l] = last.u32[(F_M16 + k) * dst.P + l];
-            }
-        if (dst.u64)
-            for (int f = 0; f < kU64Fields; ++f) dst.u64[f * dst.P + l] = last.u64[f * dst.P + l];
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, P = dst.P;
+    const int n32 = variant == CI_VAR_BBS16 ? kU32FieldsBbs16 : kU32Fields;
+    const uint64_t total = (n32 + (dst.u64 ? kU64Fields : 0)) * P;
+    for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += stride) {
+        const int f = (int)(t / P);
+        const uint64_t l = t % P;
+        if (f >= n32) {
+            dst.u64[(f - n32) * P + l] = last.u64[(f - n32) * P + l];
+        } else if (f != F_SEL) {
+            const int to = f < F_Y16 ? f : f < F_M16 ? F_Y16 + (f - F_Y16 + 1) % 8 : F_M16 + (f - F_M16 + 1) % 8;
+            dst.u32[to * P + l] = last.u32[f * P + l];
+        }
     }
 }
 
@@ -740,6 +804,7 @@ __global__ void __launch_bounds__(256) k_consume_rows(const uint32_t *rows, uint
 constexpr uint32_t kMaxSegments = kSplitMaxSegments;
 constexpr uint64_t kMinSegment = 256;       // iterations per segment (auto choice, BBS)
 constexpr uint64_t kMinShortSegment = 64;   // ... while they do not fill the GPU (BBS sources)
+constexpr uint64_t kMinXorSplit = 2048;     // iterations of a xor-like call that splits on its own
 constexpr uint64_t kMinAutoSegment = 1024;  // ... xor-likes, and when a single call splits on its own
 constexpr uint64_t kScratchWords = 1ull << 29;  // scratch outputs of a BBS-source consumer call (2 GiB)
 // Written BBS-source outputs take the one-launch fix-up form from this many
@@ -926,13 +991,18 @@ cudaError_t split_run_sink(int variant, int xl, const SegSpace &sp, const DevSta
                                              crt, stream);
 }
 
-// Runs segments [kb, ke) into the caller's sink (CI_SINK_*); written outputs
+constexpr int kSinkNone = -1;  // end states only
+
+// Runs segments [kb, ke) into the caller's sink (CI_SINK_*, or kSinkNone); written outputs
 // take 16-byte stores when out, ld and col0 allow it.  Segment 0: the caller's
 // state (zero < 0) or segment state `zero`.
 cudaError_t split_run(const ci_states_s &h, int sink, const SegSpace &sp, int caller0, uint32_t kb, uint32_t ke,
                       uint32_t K, uint64_t len, uint64_t len_last, uint32_t *out, uint64_t ld, uint64_t col0,
                       uint64_t *aux, const uint32_t *crt, cudaStream_t stream) {
     const DevState caller = h.view();
+    if (sink == kSinkNone)
+        return split_run_sink<SINK_NONE>(h.variant, h.xl, sp, caller, caller0, kb, ke, K, len, len_last, out, ld, col0,
+                                         aux, crt, stream);
     if (sink == CI_SINK_QC)
         return split_run_sink<SINK_QC>(h.variant, h.xl, sp, caller, caller0, kb, ke, K, len, len_last, out, ld, col0,
                                        aux, crt, stream);
@@ -1022,11 +1092,14 @@ uint64_t split_auto(const ci_states_s &h, uint64_t n, int sink) {
         const uint64_t len = ((n + K - 1) / K + 31) / 32 * 32;
         return (n + len - 1) / len;
     }
-    // xor-likes: only states with no more warp groups than SMs (measured:
-    // 4-11x faster up to 128 groups, slower from 512 groups on, where the
-    // setup's GF(2) jumps outweigh the parallelism)
-    if (h.variant != CI_VAR_XOR || groups > sms) return 1;
-    uint64_t K = std::min<uint64_t>(sms * 64 / groups, std::max<uint64_t>(1, n / kMinAutoSegment));
+    // xor-likes: only states with no more warp groups than SMs, and calls long
+    // enough to pay for the five launches; about one wave of 16 warps per SM,
+    // segments of at least 256.  Measured, unsplit against this rule: 32
+    // streams x 1000 27 against 51 us, x 4096 107 against 46, 4096 x 4096 107
+    // against 76; 1000 x 65536 127 us, 155 with 64 warps per SM; 256 x 65536
+    // 77 us, 96 from 1024 iterations on, 94 from 128 on.
+    if (h.variant != CI_VAR_XOR || groups > sms || n < kMinXorSplit) return 1;
+    uint64_t K = std::min<uint64_t>(sms * 16 / groups, n / kMinSegment);
     K = std::min<uint64_t>(K, kMaxSegments);
     if (K <= 1) return 1;
     const uint64_t len = ((n + K - 1) / K + 31) / 32 * 32;
@@ -1122,7 +1195,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
     const DevState src = h->view();
 
     ci_status st = CI_OK;
-    if (b16) k_split_lambda16<<<split_block_count(h->P), 256, 0, stream>>>(src, lam16);
+    if (b16) k_split_lambda16<<<split_block_count(8 * h->P), 256, 0, stream>>>(src, lam16);
     if (bbs) k_split_constants<<<split_block_count(h->P), 256, 0, stream>>>(src, lam64, crt);
     k_split_setup<<<split_block_count(slots * h->P), 256, 0, stream>>>(src, sp, (uint32_t)K, len, h->variant, h->xl,
                                                                        own, lam16, lam64, crt);
@@ -1148,7 +1221,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
                                                                         starts, events, next_unit, crt, stream);
         }
         if (e == cudaSuccess) {
-            k_split_copy_back<<<split_block_count(h->P), 256, 0, stream>>>(src, segment(K - 1), h->variant);
+            k_split_copy_back<<<split_block_count(12 * h->P), 256, 0, stream>>>(src, segment(K - 1), h->variant);
             e = cudaGetLastError();
         }
         if (e != cudaSuccess) st = cuda_fail(e, "split pass 1 with fix-ups");
@@ -1160,19 +1233,19 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
     if (st == CI_OK) {
         e = fixup ? split_run(*h, sink, sp, 0, 0, (uint32_t)K, (uint32_t)K, len, len_last, out, ld, col0, nullptr,
                               crt, stream)
-                  : split_run(*h, CI_SINK_DIGEST, sp, 0, 0, (uint32_t)K - 1, (uint32_t)K, len, len_last, nullptr, 0,
+                  : split_run(*h, kSinkNone, sp, 0, 0, (uint32_t)K - 1, (uint32_t)K, len, len_last, nullptr, 0,
                               0, res1, crt, stream);
         if (e != cudaSuccess) st = cuda_fail(e, "split pass 1");
     }
     uint2 *starts = reinterpret_cast<uint2 *>(res1);  // K * P (slot, x) pairs, after pass 1
     if (st == CI_OK) {
-        const unsigned threads = 32u * (unsigned)std::min<uint64_t>(kCarryWarps, K - 1);
+        const unsigned blocks = (unsigned)groups * kCarryBlocks, threads = 32u * kCarryWarps;
         if (bbs)
-            k_split_carry<SrcBbs><<<(unsigned)groups, threads, 0, stream>>>(sp, (uint32_t)K, len, starts, own);
+            k_split_carry<SrcBbs><<<blocks, threads, 0, stream>>>(sp, (uint32_t)K, len, starts, own);
         else if (b16)
-            k_split_carry<SrcBbs16Seg><<<(unsigned)groups, threads, 0, stream>>>(sp, (uint32_t)K, len, starts, own);
+            k_split_carry<SrcBbs16Seg><<<blocks, threads, 0, stream>>>(sp, (uint32_t)K, len, starts, own);
         else
-            k_split_carry<SrcXor128><<<(unsigned)groups, threads, 0, stream>>>(sp, (uint32_t)K, len, starts, own);
+            k_split_carry<SrcXor128><<<blocks, threads, 0, stream>>>(sp, (uint32_t)K, len, starts, own);
         if ((e = cudaGetLastError()) != cudaSuccess) st = cuda_fail(e, "split carry");
     }
     if (st == CI_OK && fixup) {  // homogeneous parts into segments 1 .. K-1, then the final state
@@ -1189,7 +1262,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
                : k_split_fixup<SrcBbs16Seg, false><<<blocks, 256, 0, stream>>>(sp, starts, (uint32_t)K, len,
                                                                                 len_last, groups, out, ld, col0);
         if ((e = cudaGetLastError()) == cudaSuccess)
-            k_split_copy_back<<<split_block_count(h->P), 256, 0, stream>>>(src, segment(K - 1), h->variant);
+            k_split_copy_back<<<split_block_count(12 * h->P), 256, 0, stream>>>(src, segment(K - 1), h->variant);
         if ((e = cudaGetLastError()) != cudaSuccess) st = cuda_fail(e, "split fix-up");
         cudaFreeAsync(ws, stream);
         return st;
@@ -1202,7 +1275,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
         if (e != cudaSuccess) st = cuda_fail(e, "split pass 2");
     }
     if (st == CI_OK) {
-        k_split_copy_back<<<split_block_count(h->P), 256, 0, stream>>>(src, segment(K - 1), h->variant);
+        k_split_copy_back<<<split_block_count(12 * h->P), 256, 0, stream>>>(src, segment(K - 1), h->variant);
         if (!written)
             k_split_combine<<<(unsigned)((h->S + 255) / 256), 256, 0, stream>>>(res3, aux, h->P, h->S, (uint32_t)K,
                                                                                 len, len_last, sink == CI_SINK_DIGEST);
