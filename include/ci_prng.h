@@ -168,9 +168,11 @@ ci_status ci_states_query(ci_states states, ci_states_desc *out);
  * o = group base + comb[s % C]); slot[s] = t; x ^= t; output x.
  * Errors: CI_E_STATE (BBS handle), CI_E_INVAL (null output, or
  * out_capacity_u32 < n_streams * n_per_stream), CI_E_CUDA.
- * n_per_stream == 0 is a no-op.  A state of at most one warp group (32
- * streams) per SM is run as time segments, as ci_generate_split does, with
- * identical results; that form allocates a stream-ordered workspace. */
+ * n_per_stream == 0 is a no-op.  A state of few warp groups (32 streams each)
+ * is run as time segments with identical results: a call of some hundred to
+ * 16384 iterations of at most two warp groups per SM in one launch of thread
+ * block clusters, a longer one of at most one per SM as ci_generate_split
+ * does; that form allocates a stream-ordered workspace. */
 ci_status ci_generate(ci_states states, uint64_t n_per_stream, uint32_t *out_dev,
                       uint64_t out_capacity_u32, void *cuda_stream);
 
@@ -207,7 +209,9 @@ ci_status ci_generate_bbs(ci_states states, uint64_t n_per_stream, uint32_t *out
  * in ci_generate / ci_generate_bbs; CI_VAR_BBS states as in ci_generate_bbs
  * while n_streams * n_per_stream <= 2^29 (the outputs then pass through a
  * stream-ordered scratch and are counted from there), otherwise under about
- * two waves of resident warps. */
+ * two waves of resident warps.  Stream-ordered workspaces come from a memory
+ * pool of the library's own, which keeps up to 256 MiB between calls and gives
+ * it back when the last state is freed. */
 ci_status ci_generate_fused_qc(ci_states states, uint64_t n_per_stream, uint64_t *counts_dev,
                                void *cuda_stream);
 
@@ -543,8 +547,8 @@ ci_status ci_naive_generate(void *state_dev, uint64_t n_streams, uint64_t n_per_
  * outputs unless the state fills about ten waves of resident warps, BBS
  * consumer sinks likewise up to 2^29 outputs per call and under about two
  * waves above that, xor-like states of at most one warp
- * group per SM, with segments of at least 1024 iterations, and CI_VAR_BBS16
- * states of at most one warp group per SM.)
+ * group per SM in calls of at least 2048 iterations (up to 16384 in one launch
+ * of their own), and CI_VAR_BBS16 states of at most one warp group per SM.)
  * Method: each segment's own generator is jumped ahead (xor-likes: GF(2)
  * matrix powers of their step; BBS: x <- x^(2^(11 k len) mod lcm(p-1, q-1))
  * mod M), the segments run from a zero mixing state, a per-warp scan restores

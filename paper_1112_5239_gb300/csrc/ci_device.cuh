@@ -651,20 +651,19 @@ __device__ __forceinline__ void written_unaligned(Step step, uint64_t S, uint64_
 // D = sum_i x_i K^(n-1-i) mod 2^64, to counts[r].  `tile` is this warp's
 // 32 x TC::KT words of shared memory (written sinks).  SINK_V4 needs out, ld
 // and col0 aligned to 4 words.
+// Runs n steps of a loaded lane into the sink; returns the lane's
+// quarter-circle hits or the Horner digest of these outputs (0 for the others).
+// Written outputs go to out[r * ld + col0 + i], rows r = row0 + lane < S.
 template <class Src, int SINK, class TC>
-__device__ __forceinline__ void warp_loop(Lane<Src> &s, const DevState &st, uint64_t g, uint64_t n, uint32_t *out,
-                                          uint64_t ld, uint64_t col0, uint64_t *counts, uint4 *tile) {
+__device__ __forceinline__ uint64_t warp_run(Lane<Src> &s, uint64_t S, uint64_t row0, uint64_t n, uint32_t *out,
+                                             uint64_t ld, uint64_t col0, uint4 *tile) {
     constexpr int KT = (SINK == SINK_V4 || SINK == SINK_SCALAR) ? TC::KT : 32;
     constexpr int CH = KT / 4;
     const int lane = threadIdx.x & 31;
-    const uint64_t l = g * 32 + lane;
-    s.load(st, l);
-    const uint64_t row0 = g * 32;
     if constexpr (SINK == SINK_SCALAR) {
-        written_unaligned<!Src::kHeavy, TC::CACHE>([&]() { return s.step(); }, st.S, row0, n, out,
+        written_unaligned<!Src::kHeavy, TC::CACHE>([&]() { return s.step(); }, S, row0, n, out,
                                                    ld, col0, tile);
-        s.store(st, l);
-        return;
+        return 0;
     }
     const uint64_t nfull = n - n % KT;
     uint32_t *tw = reinterpret_cast<uint32_t *>(tile);
@@ -707,7 +706,7 @@ __device__ __forceinline__ void warp_loop(Lane<Src> &s, const DevState &st, uint
             for (int k = 0; k < CH; ++k) {
                 const int r = RPI * k + lane / CH, c = lane % CH;
                 const uint4 v = tile[r * CH + (c ^ (r & 7))];
-                if (row0 + r < st.S) store16<TC::CACHE>(out + (row0 + r) * ld + col0 + i0 + 4 * c, v);
+                if (row0 + r < S) store16<TC::CACHE>(out + (row0 + r) * ld + col0 + i0 + 4 * c, v);
             }
             __syncwarp();
         }
@@ -734,7 +733,7 @@ __device__ __forceinline__ void warp_loop(Lane<Src> &s, const DevState &st, uint
 #pragma unroll 2
             for (int k = 0; k < CH; ++k) {
                 const int r = RPI * k + lane / CH, c = lane % CH;
-                if (row0 + r < st.S)
+                if (row0 + r < S)
                     store_words<TC::CACHE>(out + (row0 + r) * ld + col0 + nfull + 4 * c, tile[r * CH + (c ^ (r & 7))],
                                            -4 * c, rem - 4 * c);
             }
@@ -742,10 +741,20 @@ __device__ __forceinline__ void warp_loop(Lane<Src> &s, const DevState &st, uint
         }
     }
 
+    return hits;
+}
+
+template <class Src, int SINK, class TC>
+__device__ __forceinline__ void warp_loop(Lane<Src> &s, const DevState &st, uint64_t g, uint64_t n, uint32_t *out,
+                                          uint64_t ld, uint64_t col0, uint64_t *counts, uint4 *tile) {
+    const uint64_t l = g * 32 + (threadIdx.x & 31);
+    s.load(st, l);
+    const uint64_t hits = warp_run<Src, SINK, TC>(s, st.S, g * 32, n, out, ld, col0, tile);
     s.store(st, l);
     if (SINK == SINK_QC && l < st.S) counts[l] += hits;
     if (SINK == SINK_DIGEST && l < st.S) counts[l] = hits;
 }
+
 
 template <class Src, int SINK, class TC = TileDefault>
 __device__ __forceinline__ void warp_task(const DevState &st, uint64_t g, uint64_t n, uint32_t *out,

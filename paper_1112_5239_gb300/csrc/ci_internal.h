@@ -112,4 +112,7 @@ int sm_count();
 constexpr uint64_t kWorkspaceKept = 256ull << 20;
 cudaError_t workspace_alloc(void **p, size_t bytes, cudaStream_t stream);
 
+// Whether `stream` is being captured into a graph.
+bool stream_capturing(cudaStream_t stream);
+
 }  // namespace ci

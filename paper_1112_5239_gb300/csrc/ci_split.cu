@@ -429,19 +429,10 @@ __global__ void __launch_bounds__(256) k_split_setup(DevState src, SegSpace seg,
 }
 
 // 32 x 32 GF(2) matrices over a warp's lanes, lane l holding row l (bit m of
-// row l = entry (l, m)).  C = A B: row_l(C) = XOR of row_m(B) over the set
-// bits m of row_l(A).  M v for a vector of words v (one per lane): lane l
-// takes the XOR of v_m over the set bits m of row_l(M).
-__device__ __forceinline__ uint32_t mat_mul(uint32_t a_row, uint32_t b_row) {
-    uint32_t c = 0;
-#pragma unroll
-    for (int m = 0; m < 32; ++m) {
-        const uint32_t b = __shfl_sync(kFull, b_row, m);
-        c ^= ((a_row >> m) & 1u) ? b : 0u;
-    }
-    return c;
-}
-
+// row l = entry (l, m)); M v for a vector of words v (one per lane): lane l
+// takes the XOR of v_m over the set bits m of row_l(M).  A product A B is A
+// applied to the words of B's rows.
+//
 // (M v, N v) of two matrices and one vector, by the method of four Russians:
 // the warp tabulates the 16 XORs of each four consecutive lanes' words in
 // shared memory, and every lane looks its eight nibbles per row up (lanes that
@@ -464,6 +455,22 @@ __device__ __forceinline__ uint2 mat_vec2(uint32_t m_row, uint32_t n_row, uint32
         r.y ^= sc.tab[g][(n_row >> (4 * g)) & 15u];
     }
     return r;
+}
+
+// Q = P^len and S = P + ... + P^len, len >= 1, by the bits of len from the
+// top: (Q, S) for k -> 2k: S <- S ^ S Q, Q <- Q Q; k -> k + 1: Q <- Q P,
+// S <- S ^ Q (all are polynomials in P, so they commute).
+__device__ __forceinline__ void power_sums(uint32_t prow, uint64_t len, uint32_t &Q, uint32_t &S, MatVecScratch &sc) {
+    Q = S = prow;
+    for (int b = 62 - __clzll((long long)len); b >= 0; --b) {
+        const uint2 sq = mat_vec2(Q, S, Q, sc);
+        Q = sq.x;
+        S ^= sq.y;
+        if ((len >> b) & 1ull) {
+            Q = mat_vec2(Q, Q, prow, sc).x;
+            S ^= Q;
+        }
+    }
 }
 
 // The carry scan over the segments of one warp group, with a cluster of
@@ -505,17 +512,8 @@ __global__ void __cluster_dims__(kCarryBlocks, 1, 1) __launch_bounds__(32 * kCar
     int a1, a2;
     src.arrays(s0, l, a1, a2);
     const uint32_t prow = (1u << s0.table[a1 * 32 + lane]) ^ (1u << s0.table[a2 * 32 + lane]);
-    // Q = P^len, S = P + ... + P^len, by the bits of len from the top:
-    // (Q, S) for k -> 2k: S <- S ^ Q S, Q <- Q Q; k -> k + 1: Q <- Q P, S <- S ^ Q.
-    uint32_t Q = prow, S = prow;
-    for (int b = 62 - __clzll((long long)len); b >= 0; --b) {
-        S ^= mat_mul(Q, S);
-        Q = mat_mul(Q, Q);
-        if ((len >> b) & 1ull) {
-            Q = mat_mul(Q, prow);
-            S ^= Q;
-        }
-    }
+    uint32_t Q, S;
+    power_sums(prow, len, Q, S, sc);
     const uint32_t m = (K - 1 + NW - 1) / NW;
     const uint32_t j0 = 1 + w * m, j1 = min(K, j0 + m);
     // 1. local scan
@@ -542,11 +540,13 @@ __global__ void __cluster_dims__(kCarryBlocks, 1, 1) __launch_bounds__(32 * kCar
     // 2. H^m and this warp's carry-in
     uint32_t Qm = Q, Tm = S;
     for (int b = 30 - __clz((int)m); b >= 0; --b) {
-        Tm ^= mat_mul(Tm, Qm);
-        Qm = mat_mul(Qm, Qm);
+        const uint2 sq = mat_vec2(Qm, Tm, Qm, sc);
+        Qm = sq.x;
+        Tm ^= sq.y;
         if ((m >> b) & 1u) {
-            Qm = mat_mul(Qm, Q);
-            Tm = S ^ mat_mul(Tm, Q);
+            const uint2 up = mat_vec2(Qm, Tm, Q, sc);
+            Qm = up.x;
+            Tm = S ^ up.y;
         }
     }
     cluster.sync();
@@ -800,6 +800,138 @@ __global__ void __launch_bounds__(256) k_consume_rows(const uint32_t *rows, uint
     }
 }
 
+// ------------------------------------------------ narrow xor-like calls
+// A call of few warp groups in one launch: a cluster of up to kNarrowBlocks
+// blocks per group, whose up to 32 warps take one time segment of `len`
+// iterations each (len a multiple of 32; K segments, the last one shorter).  Bound by latency:
+// a warp alone on its scheduler takes 55 cycles a step, so 4096 x 1024 unsplit
+// spent 27 us on one chain of 1024 steps per SM, and five launches of the
+// general form take 45.  Per warp:
+//   1. the own generator jumps to its segment's start;
+//   2. pass 1 from a zero mixing state (segment 0: from the true one), for the
+//      particular end alone; then H = (Q, S) = (P^len, P + ... + P^len);
+//   3. carries: the four ends of a block are folded through H, the
+//      blocks' aggregates, exchanged by distributed shared memory, through
+//      H^4;
+//   4. pass 2 from the true start into the sink.
+// All state is read before the first cluster barrier; the last segment's warp
+// writes it back after it.
+constexpr int kNarrowBlocks = 8, kNarrowWarps = 4;  // most blocks of a cluster; warps of a block
+
+__device__ __forceinline__ void jump_source(SrcXor128 &s, uint64_t dist) {
+    uint32_t v[4] = {s.a, s.b, s.c, s.d};
+    jump_words<4>(v, dist, g_jump_xor128);
+    s.a = v[0];
+    s.b = v[1];
+    s.c = v[2];
+    s.d = v[3];
+}
+__device__ __forceinline__ void jump_source(SrcXor64 &s, uint64_t dist) {
+    uint32_t v[2] = {(uint32_t)s.z, (uint32_t)(s.z >> 32)};
+    jump_words<2>(v, dist, g_jump_xor64);
+    s.z = (uint64_t)v[0] | ((uint64_t)v[1] << 32);
+}
+__device__ __forceinline__ void jump_source(SrcXorshift32 &s, uint64_t dist) {
+    uint32_t v[1] = {s.z};
+    jump_words<1>(v, dist, g_jump_xs32);
+    s.z = v[0];
+}
+
+template <class Src, int SINK>
+__global__ void __launch_bounds__(32 * kNarrowWarps)
+    k_narrow(DevState st, uint64_t n, uint64_t len, uint32_t K, uint32_t *out, uint64_t *aux) {
+    __shared__ uint4 tiles[kNarrowWarps][SINK == SINK_V4 ? 256 : SINK == SINK_SCALAR ? kTileVec : 1];
+    __shared__ __align__(16) MatVecScratch scratch[kNarrowWarps];
+    __shared__ uint2 ends[kNarrowWarps][32], aggregate[32], all[kNarrowBlocks][32];
+    __shared__ uint64_t results[kNarrowWarps][32];
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int nb = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const uint64_t g = blockIdx.x / nb;
+    const int lane = threadIdx.x & 31, bw = threadIdx.x >> 5;
+    const uint32_t seg = rank * kNarrowWarps + bw;
+    CI_WARP_CHECK(st, g < st.P / 32, CHK_GROUP, g);  // the same in the whole cluster: its warps return together
+    CI_WARP_CHECK(st, (uint64_t)(K - 1) * len < n && n <= K * len, CHK_SEG_COLS, K);
+    MatVecScratch &sc = scratch[bw];
+    const uint64_t l = g * 32 + lane;
+    Lane<Src> s;
+    s.src.load(st, l);
+    s.load(st, l);
+    const uint32_t slot0 = s.slot, x0 = s.x;
+    if (seg > 0 && seg < K) jump_source(s.src, seg * len);
+    const Src start = s.src;
+    if (seg > 0) s.slot = s.x = 0;
+    if (seg + 1 < K) warp_run<Src, SINK_NONE, TileDefault>(s, 0, 0, len, nullptr, 0, 0, nullptr);
+    const uint2 e = make_uint2(s.slot, s.x);
+    ends[bw][lane] = e;
+    uint32_t Q, S;
+    power_sums((1u << s.p1) ^ (1u << s.p2), len, Q, S, sc);
+    __syncthreads();
+    // H(c) ^ e for c = (slot, x)
+    auto advance = [&](uint32_t q, uint32_t t, uint2 c, uint2 add) {
+        const uint2 h = mat_vec2(q, t, c.x, sc);
+        return make_uint2(add.x ^ h.x, add.y ^ c.y ^ h.y);
+    };
+    const uint2 zero = make_uint2(0u, 0u);
+    uint2 pre = zero;  // the carry into this warp's segment from the block's earlier ones
+    for (int v = 0; v < bw; ++v) pre = v ? advance(Q, S, pre, ends[v][lane]) : ends[0][lane];
+    if (bw == kNarrowWarps - 1) aggregate[lane] = advance(Q, S, pre, e);
+    uint32_t Q4 = Q, S4 = S;  // H^4
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const uint2 sq = mat_vec2(Q4, S4, Q4, sc);
+        Q4 = sq.x;
+        S4 ^= sq.y;
+    }
+    cluster.sync();
+    for (int v = bw; v < nb; v += kNarrowWarps) all[v][lane] = cluster.map_shared_rank(aggregate, v)[lane];
+    cluster.sync();  // every aggregate is here, and no block's is read any more
+    uint2 c = zero;  // the carry into this block's first segment
+    for (int v = 0; v < rank; ++v) c = v ? advance(Q4, S4, c, all[v][lane]) : all[0][lane];
+    if (rank)
+        for (int i = 0; i < bw; ++i) c = advance(Q, S, c, zero);
+    s.src = start;
+    s.slot = seg ? pre.x ^ c.x : slot0;
+    s.x = seg ? pre.y ^ c.y : x0;
+    uint64_t r = 0;
+    if (seg < K) {
+        const uint64_t from = seg * len, m = seg + 1 == K ? n - from : len;
+        r = warp_run<Src, SINK, TileDefault>(s, st.S, g * 32, m, out, n, from, tiles[bw]);
+        if (SINK == SINK_DIGEST) r *= digest_pow(n - from - m);
+        if (seg + 1 == K) s.store(st, l);
+    }
+    if (SINK == SINK_QC || SINK == SINK_DIGEST) {
+        results[bw][lane] = r;
+        cluster.sync();
+        if (seg == 0) {
+            uint64_t sum = 0;
+            for (int v = 0; v < nb * kNarrowWarps; ++v)
+                sum += cluster.map_shared_rank(&results[0][0], v / kNarrowWarps)[(v % kNarrowWarps) * 32 + lane];
+            if (l < st.S) aux[l] = SINK == SINK_QC ? aux[l] + sum : sum;
+        }
+        cluster.sync();
+    }
+}
+
+template <class Src>
+cudaError_t launch_narrow_src(const DevState &st, int sink, int blocks, uint64_t n, uint64_t len, uint32_t K,
+                              uint32_t *out, uint64_t *aux, cudaStream_t stream) {
+    cudaLaunchAttribute cluster;
+    cluster.id = cudaLaunchAttributeClusterDimension;
+    cluster.val.clusterDim = {(unsigned)blocks, 1, 1};
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(st.P / 32) * blocks);
+    cfg.blockDim = dim3(32 * kNarrowWarps);
+    cfg.stream = stream;
+    cfg.attrs = &cluster;
+    cfg.numAttrs = 1;
+    auto kern = sink == SINK_V4       ? k_narrow<Src, SINK_V4>
+                : sink == SINK_SCALAR ? k_narrow<Src, SINK_SCALAR>
+                : sink == SINK_QC     ? k_narrow<Src, SINK_QC>
+                                      : k_narrow<Src, SINK_DIGEST>;
+    return cudaLaunchKernelEx(&cfg, kern, st, n, len, K, out, aux);
+}
+
 // ------------------------------------------------ host side
 constexpr uint32_t kMaxSegments = kSplitMaxSegments;
 constexpr uint64_t kMinSegment = 256;       // iterations per segment (auto choice, BBS)
@@ -1028,6 +1160,53 @@ namespace ci {
 
 cudaError_t split_prepare(cudaStream_t stream) { return ensure_jump_tables(stream); }
 
+namespace {
+
+bool jump_tables_ready() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lk(g_tables_mu);
+    return dev < (int)g_tables_ready.size() && g_tables_ready[dev];
+}
+
+// Blocks per cluster of the one-launch form for a call of n iterations; 0: it
+// does not apply.  From where its jumps and carries (some 7 us) are repaid up
+// to where segments of a thirty-second are longer than the general form's.
+// About 8 warps per SM, 16 for long calls.  Measured, xor128 written, unsplit
+// or general split against this form: 1000 x 448 14 / 10.5 us, 4096 x 512 15 /
+// 12, 4096 x 1024 27 / 16 (19 with 16 warps per SM), 9000 x 600 17 / 19, 9000 x
+// 2000 49 / 33, 4096 x 4096 72 / 35 (37 with 8), 32 x 4096 44 / 17, 256 x 16384
+// 55 / 35, 256 x 65536 76 / 107, 16000 x 2000 51 / 50.
+constexpr uint64_t kNarrowMin = 448, kNarrowWideMin = 1024, kNarrowLong = 2048, kNarrowMax = 16384;
+int narrow_blocks(const ci_states_s &h, uint64_t n) {
+    const uint64_t groups = h.P / 32, sms = (uint64_t)sm_count();
+    if (h.variant != CI_VAR_XOR || groups > 2 * sms || n > kNarrowMax) return 0;
+    if (n < (groups > sms ? kNarrowWideMin : kNarrowMin)) return 0;
+    const uint64_t warps = (n < kNarrowLong ? 8 : 16) * sms;
+    int blocks = kNarrowBlocks;
+    while (blocks > 1 && groups * kNarrowWarps * blocks > warps) blocks /= 2;
+    return blocks;
+}
+
+cudaError_t launch_narrow(const ci_states_s &h, int blocks, uint64_t n, int sink, uint32_t *out, uint64_t *aux,
+                          cudaStream_t stream) {
+    const cudaError_t e = ensure_jump_tables(stream);
+    if (e != cudaSuccess) return e;
+    const uint64_t segments = (uint64_t)blocks * kNarrowWarps;
+    const uint64_t len = ((n + segments - 1) / segments + 31) / 32 * 32;
+    const uint32_t K = (uint32_t)((n + len - 1) / len);
+    const int kind = sink == CI_SINK_QC       ? SINK_QC
+                     : sink == CI_SINK_DIGEST ? SINK_DIGEST
+                     : (reinterpret_cast<uintptr_t>(out) & 15u) == 0 && n % 4 == 0 ? SINK_V4
+                                                                                   : SINK_SCALAR;
+    const DevState st = h.view();
+    if (h.xl == CI_XL_XORSHIFT32) return launch_narrow_src<SrcXorshift32>(st, kind, blocks, n, len, K, out, aux, stream);
+    if (h.xl == CI_XL_XOR64) return launch_narrow_src<SrcXor64>(st, kind, blocks, n, len, K, out, aux, stream);
+    return launch_narrow_src<SrcXor128>(st, kind, blocks, n, len, K, out, aux, stream);
+}
+
+}  // namespace
+
 uint64_t split_segments(const ci_states_s &h, uint64_t n, uint64_t requested) {
     const uint64_t groups = h.P / 32;
     uint64_t K = requested;
@@ -1044,7 +1223,16 @@ uint64_t split_segments(const ci_states_s &h, uint64_t n, uint64_t requested) {
     return (n + len - 1) / len;
 }
 
-uint64_t split_auto_bbs(const ci_states_s &h, uint64_t n, int sink) {
+namespace {
+
+// Segment count a single call uses for a CI_VAR_BBS state.  Written sink, and
+// consumer sinks whose outputs fit the scratch (they are written, fixed up and
+// reduced): from the GPU size and the form split_launch takes; larger consumer
+// calls, which generate twice: > 1 only for states that fill less than about
+// two waves of resident warps.  `captured`: calls too short for segments of
+// kMinSegment stay one plain launch (a split allocates its workspace, which a
+// graph then has to own).
+uint64_t split_auto_bbs(const ci_states_s &h, uint64_t n, int sink, bool captured) {
     if (h.variant != CI_VAR_BBS) return 1;
     const uint64_t groups = h.P / 32, sms = (uint64_t)sm_count();
     uint64_t K;
@@ -1060,7 +1248,7 @@ uint64_t split_auto_bbs(const ci_states_s &h, uint64_t n, int sink) {
         // resident warps (24 per SM): 32 streams x 4096 82 us, 103 from 128
         // on, 309 from 256 on; x 65536 149 us, 171 down to 32; 1000 x 16384
         // 295 us, 337 up to 16 warps per SM.
-        K = std::max<uint64_t>(K, std::min<uint64_t>(n / kMinShortSegment, 24 * sms / groups));
+        if (!captured) K = std::max<uint64_t>(K, std::min<uint64_t>(n / kMinShortSegment, 24 * sms / groups));
     } else {
         // Larger consumer calls generate twice (pass 1, then pass 2 from the
         // true starts): only states that fill less than about two waves.
@@ -1074,8 +1262,9 @@ uint64_t split_auto_bbs(const ci_states_s &h, uint64_t n, int sink) {
     return (n + len - 1) / len;
 }
 
-uint64_t split_auto(const ci_states_s &h, uint64_t n, int sink) {
-    if (h.variant == CI_VAR_BBS) return split_auto_bbs(h, n, sink);
+// ... and for any state; 1: unsplit.
+uint64_t split_auto(const ci_states_s &h, uint64_t n, int sink, bool captured) {
+    if (h.variant == CI_VAR_BBS) return split_auto_bbs(h, n, sink, captured);
     const uint64_t groups = h.P / 32, sms = (uint64_t)sm_count();
     if (h.variant == CI_VAR_BBS16) {
         // Algorithm 5 as printed: each warp is bound by its own eight chains,
@@ -1086,7 +1275,7 @@ uint64_t split_auto(const ci_states_s &h, uint64_t n, int sink) {
         // 64 while they fill less than one wave.
         if (groups > sms) return 1;
         uint64_t K = std::min<uint64_t>(sms * 32 / groups, n / kMinSegment);
-        K = std::max<uint64_t>(K, std::min<uint64_t>(sms * 16 / groups, n / kMinShortSegment));
+        if (!captured) K = std::max<uint64_t>(K, std::min<uint64_t>(sms * 16 / groups, n / kMinShortSegment));
         K = std::min<uint64_t>(K, kMaxSegments);
         if (K <= 1) return 1;
         const uint64_t len = ((n + K - 1) / K + 31) / 32 * 32;
@@ -1104,6 +1293,25 @@ uint64_t split_auto(const ci_states_s &h, uint64_t n, int sink) {
     if (K <= 1) return 1;
     const uint64_t len = ((n + K - 1) / K + 31) / 32 * 32;
     return (n + len - 1) / len;
+}
+
+}  // namespace
+
+ci_status single_call(const ci_states_s &h, uint64_t n, int sink, uint32_t *out, uint64_t *aux, cudaStream_t stream) {
+    const bool captured = stream_capturing(stream);
+    cudaError_t e;
+    // building the jump tables waits for the stream once, which a capture forbids
+    const int blocks = narrow_blocks(h, n);
+    if (blocks && (!captured || jump_tables_ready())) {
+        e = launch_narrow(h, blocks, n, sink, out, aux, stream);
+    } else {
+        const uint64_t K = split_auto(h, n, sink, captured);
+        if (K > 1) return split_launch(h, n, sink, out, n, 0, aux, K, stream);
+        e = sink == CI_SINK_QC       ? launch_fused_qc(h, n, aux, stream)
+            : sink == CI_SINK_DIGEST ? launch_digest(h, n, aux, stream)
+                                     : launch_generate(h, n, out, stream);
+    }
+    return e == cudaSuccess ? CI_OK : cuda_fail(e, "generation kernel launch");
 }
 
 ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *out, uint64_t ld, uint64_t col0,
@@ -1152,7 +1360,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
         cudaFreeAsync(rows, stream);
         return st;
     }
-    if ((e = ensure_jump_tables(stream)) != cudaSuccess) return cuda_fail(e, "jump tables");
+    if (h->variant == CI_VAR_XOR && (e = ensure_jump_tables(stream)) != cudaSuccess) return cuda_fail(e, "jump tables");
     const uint64_t groups = h->P / 32;
     const uint64_t len = ((n + K - 1) / K + 31) / 32 * 32;
     const uint64_t len_last = n - (K - 1) * len;

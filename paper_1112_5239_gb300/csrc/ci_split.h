@@ -17,20 +17,12 @@ constexpr uint32_t kSplitMaxSegments = 8192;
 // 1 means unsplit.
 uint64_t split_segments(const ci_states_s &h, uint64_t n, uint64_t requested);
 
-// Segment count ci_generate_bbs (and the BBS consumer calls) use on their
-// own for CI_VAR_BBS states, 1 for others.  Written sink, and consumer sinks
-// whose outputs fit the scratch (2^29 words; they are written, fixed up and
-// reduced): from the GPU size and the form split_launch takes (one launch
-// from 12 warp groups per SM on, three launches below); larger consumer
-// calls, which generate twice: > 1 only for states that fill less than about
-// two waves of resident warps.
-uint64_t split_auto_bbs(const ci_states_s &h, uint64_t n, int sink);
-
-// Segment count the single-call entry points use on their own for `sink`
-// (CI_SINK_*): split_auto_bbs for CI_VAR_BBS; for xor-like states only with
-// no more warp groups than SMs (and segments of at least 1024 iterations);
-// for CI_VAR_BBS16 likewise (segments of at least 256); 1 otherwise.
-uint64_t split_auto(const ci_states_s &h, uint64_t n, int sink);
+// One public single call (ci_generate, ci_generate_bbs, ci_generate_fused_qc,
+// ci_generate_digest; CI_SINK_*), by the form that suits the state and length:
+// one launch of clusters (narrow xor-like states), time segments (narrow
+// xor-like and CI_VAR_BBS16 states; CI_VAR_BBS unless it fills the GPU by
+// itself), or the generation kernel.  Identical results.
+ci_status single_call(const ci_states_s &h, uint64_t n, int sink, uint32_t *out, uint64_t *aux, cudaStream_t stream);
 
 // n iterations of h as K segments into `sink` (written: out[r * ld + col0 + i];
 // consumers: aux[r]), with results equal to one sequential call.  Calls on
