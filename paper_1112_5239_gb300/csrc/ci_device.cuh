@@ -523,6 +523,29 @@ __device__ __forceinline__ uint32_t qc_miss(uint32_t o0, uint32_t o1) {
     return __umulhi((uint32_t)(s >> 32), c_qc_mul[1]);
 }
 
+// The same test by the high halves of o0^2 and o1^2, for blocks of pairs: with
+// h = floor(o0^2 / 2^32) + floor(o1^2 / 2^32) and V = (a^2 + b^2) / 2^16 (miss
+// iff V >= 2^32), h - 1024 < V < h + 2, since the low bytes that a and b leave
+// out add less than 1024 and the two floors take less than 2.  So h >= 2^32 is
+// the answer except for h in [2^32 - 1, 2^32 + 1023], one pair in 5 million;
+// `near` keeps the smallest (h + 1) mod 2^32 of a block, at most kQcNear if any
+// pair was that close, and the block is then run again by the exact test.  Two
+// wide products, a carry and a minimum a pair instead of five wide products and
+// an addition: the loop is bound by what its schedulers can dispatch (a cycle
+// for a narrow multiply or an addition, two for an ALU operation or a wide
+// multiply).  2^20 x 1024 xor128 outputs: 622 us by the exact test (23.3 cycles
+// a step), 563 so; 605 with the two halves and 1 added in 64 bits and one
+// three-way minimum for two pairs.
+constexpr uint32_t kQcNear = 1024;
+__device__ __forceinline__ void qc_miss_high(uint32_t o0, uint32_t o1, uint32_t &miss, uint32_t &near) {
+    uint32_t h;
+    asm("add.cc.u32 %0, %2, %3;\n\t"
+        "addc.u32 %1, %1, 0;"
+        : "=r"(h), "+r"(miss)
+        : "r"(__umulhi(o0, o0)), "r"(__umulhi(o1, o1)));
+    near = __viaddmin_u32(h, 1u, near);
+}
+
 // Launch-shape choices of the written sinks, picked by the autotuner:
 // KT = outputs per stream staged per flush (tile depth: 32 or 64, i.e. 128- or
 // 256-byte row segments), CACHE = store policy (0: streaming st.global.cs,
@@ -571,10 +594,9 @@ __device__ __forceinline__ void store_words(uint32_t *p, const uint4 &v, int lo,
 // whole lines, four rows' per warp-wide store.  (A line, or a 32-byte sector,
 // written in two parts 32 steps apart costs its memory write twice: 400 MB in
 // rows of 401 took 132 us by 16-byte, 108 by 32-byte boundaries.)  Output j of
-// a 32-step tile stands at word j + ph_r of the row's 64; after the first 32
-// are stored, the rest move down and open the next tile.  Each step's store
-// has a fixed offset, and the lanes of one step write 32 different banks when
-// ld is odd.  `step` makes the lane's next output; kUnroll: it is short (the
+// the call stands at word (j + ph_r) mod 64 of the row's two lines, of which one
+// is stored after every 32 steps.  The lanes of one step write 32 different
+// banks when ld is odd.  `step` makes the lane's next output; kUnroll: it is short (the
 // tile's 32 steps are unrolled).
 // (50001 x 1001 XORshift outputs: the word-wise form this replaces, a row per
 // warp-wide store, issued 34 instructions per step of a warp, 20 of them for
@@ -590,24 +612,24 @@ __device__ __forceinline__ void written_unaligned(Step step, uint64_t S, uint64_
     uint32_t *w = reinterpret_cast<uint32_t *>(tile + lane * 16) + ph;
     // the rows this lane stores: 4 k + lane / 8, 16-byte word c of their lines
     const int c = lane & 7;
-    uint4 *stored = tile + (lane >> 3) * 16 + c;
+    const uint4 *stored = tile + (lane >> 3) * 16 + c;
     const uint64_t row = row0 + (lane >> 3);
     const bool all_rows = row0 + 32 <= S;
     uint32_t *dst = out + row * ld + col0;  // output `at` of row `row`
 
-    // stores the first 32 words of every staging row, moves the others down
-    // and goes on to the next line
+    // stores line `half` / 32 of every staging row and goes on to the next
     int64_t at = 0;
     const int64_t len = (int64_t)n;
+    int half = 0;
     auto flush = [&]() {
         __syncwarp();
         uint32_t *q = dst;
+        const uint4 *from = stored + half / 4;
         if (at > 0 && at + 32 <= len && all_rows) {  // words of the rows only
 #pragma unroll(kUnroll ? 8 : 2)
             for (int k = 0; k < 8; ++k, q += 4 * ld) {
                 uint32_t *line = reinterpret_cast<uint32_t *>(reinterpret_cast<uintptr_t>(q) & ~(uintptr_t)127);
-                store16<CACHE>(line + 4 * c, stored[64 * k]);
-                stored[64 * k] = stored[64 * k + 8];
+                store16<CACHE>(line + 4 * c, from[64 * k]);
             }
         } else {
 #pragma unroll 1
@@ -618,39 +640,37 @@ __device__ __forceinline__ void written_unaligned(Step step, uint64_t S, uint64_
                 // words [lo, hi) of this 16-byte word belong to the row
                 const int64_t hi = len - at + p - 4 * c;
                 if (row + 4 * k < S)
-                    store_words<CACHE>(line + 4 * c, stored[64 * k], at == 0 ? p - 4 * c : 0, hi > 4 ? 4 : (int)hi);
-                stored[64 * k] = stored[64 * k + 8];
+                    store_words<CACHE>(line + 4 * c, from[64 * k], at == 0 ? p - 4 * c : 0, hi > 4 ? 4 : (int)hi);
             }
         }
         dst += 32;
         at += 32;
+        half ^= 32;
         __syncwarp();
     };
+    // word (ph + j + half) mod 64 of the lane's row, ph + j < 64
+    auto place = [&](int j) { return j + ph < 32 ? w + half + j : w - half + j; };
     while (at + 32 <= len) {
-        if (kUnroll) {
+        if (!kUnroll) {
+#pragma unroll 1
+            for (int j = 0; j < 32; ++j) *place(j) = step();
+        } else if (half == 0) {
 #pragma unroll
             for (int j = 0; j < 32; ++j) w[j] = step();
         } else {
-#pragma unroll 1
-            for (int j = 0; j < 32; ++j) w[j] = step();
+#pragma unroll
+            for (int j = 0; j < 32; ++j) *place(j) = step();
         }
         flush();
     }
     // the rest: up to 31 steps behind the words kept from the last tile, at
     // most 62 words of a row
     const int rem = (int)(n % 32);
-    for (int j = 0; j < rem; ++j) w[j] = step();
+    for (int j = 0; j < rem; ++j) *place(j) = step();
     if (__any_sync(kFull, rem + ph > 0)) flush();
     if (__any_sync(kFull, rem + ph > 32)) flush();
 }
 
-// Runs n iterations of warp group g (lanes 32g .. 32g+31) of state `st`.
-// Written sinks store stream r's outputs at out[r * ld + col0 + i]
-// (r = 32g + lane < st.S only); SINK_QC adds the lane's quarter-circle hits
-// to counts[r]; SINK_DIGEST stores the Horner digest of the call's outputs,
-// D = sum_i x_i K^(n-1-i) mod 2^64, to counts[r].  `tile` is this warp's
-// 32 x TC::KT words of shared memory (written sinks).  SINK_V4 needs out, ld
-// and col0 aligned to 4 words.
 // Runs n steps of a loaded lane into the sink; returns the lane's
 // quarter-circle hits or the Horner digest of these outputs (0 for the others).
 // Written outputs go to out[r * ld + col0 + i], rows r = row0 + lane < S.
@@ -677,12 +697,25 @@ __device__ __forceinline__ uint64_t warp_run(Lane<Src> &s, uint64_t S, uint64_t 
 #pragma unroll(Src::kHeavy ? 1 : 32)
             for (int k = 0; k < 32; ++k) hits = hits * kDigestMul + s.step();
         } else if (SINK == SINK_QC) {
-            uint32_t m = 0;
-#pragma unroll(Src::kHeavy ? 1 : 16)
-            for (int k = 0; k < 16; ++k) {
-                const uint32_t o0 = s.step();
-                const uint32_t o1 = s.step();
-                m += qc_miss(o0, o1);
+            uint32_t m = 0, near = ~0u;
+            const Lane<Src> before = s;
+            if (!Src::kHeavy) {
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                    const uint32_t o0 = s.step();
+                    const uint32_t o1 = s.step();
+                    qc_miss_high(o0, o1, m, near);
+                }
+            }
+            if (Src::kHeavy || __any_sync(kFull, near <= kQcNear)) {
+                s = before;
+                m = 0;
+#pragma unroll 1
+                for (int k = 0; k < 16; ++k) {
+                    const uint32_t o0 = s.step();
+                    const uint32_t o1 = s.step();
+                    m += qc_miss(o0, o1);
+                }
             }
             hits += 16u - m;
         } else {

@@ -77,10 +77,9 @@ __global__ void __launch_bounds__(32) k_generate_span(DevState st, uint32_t n, u
 // not whole 32-byte sectors (the others' TMA tiles write whole sectors) up to
 // the length where too few warps fit an SM beside their staging, or shorter
 // than a TMA tile.  400 MB in rows of n, span against the next best form: n =
-// 36 83 us / 95 TMA, 100 70 / 117, 249 84 / 107 line-staged, 260 95 / 117 TMA,
-// 290 96 / 105 line-staged, 333 113 / 101, 350 111 / 101; n = 200 81 / 69 TMA,
-// 144 80 / 69.
-constexpr uint64_t kSpanMax = 296;
+// 36 83 us / 95 TMA, 100 70 / 117, 249 84 / 92 line-staged, 260 95 / 117 TMA,
+// 290 96 / 95 line-staged, 333 113 / 90; n = 200 81 / 69 TMA, 144 80 / 69.
+constexpr uint64_t kSpanMax = 280;
 inline bool span_rows(uint64_t n, const uint32_t *out) {
     return n <= kSpanMax && (n % 8 != 0 || n < 32) && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
 }

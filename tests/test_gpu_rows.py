@@ -8,7 +8,7 @@ from gpu_util import cuda_or_skip, oracle_gen, u32
 
 pytestmark = pytest.mark.gpu
 
-LENGTHS = (1, 3, 8, 16, 31, 32, 33, 36, 63, 64, 65, 100, 104, 295, 296, 297, 300, 301, 320, 333)
+LENGTHS = (1, 3, 8, 16, 31, 32, 33, 36, 63, 64, 65, 100, 104, 279, 280, 281, 282, 284, 300, 301, 320, 333)
 GUARD = 0x5A5A5A5A
 
 
