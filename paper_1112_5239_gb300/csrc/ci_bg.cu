@@ -39,8 +39,8 @@ namespace {
 using namespace dev;
 
 // Resident blocks per SM asked of the register allocator: 64 registers, no
-// spills (2^18 x 1024: decryption 390 us, 398 with 5 blocks, 422 with 6;
-// encryption 437, 446 and 454).
+// spills (2^18 x 1024: decryption 365 us, 375 with 5 blocks, 379 with 3;
+// encryption 437, 447 and 457).
 constexpr int kBgMinBlocks = 4;
 
 constexpr int kBgWarps = 8;    // warps per block
@@ -106,6 +106,18 @@ __device__ __forceinline__ bool bg_setup_encrypt(uint64_t N, uint64_t r, Barrett
     return ok;
 }
 
+// ((p + 1) / 4)^L mod (p - 1) for p = 3 mod 4 and L >= 1.  p - 1 = 2 m with m
+// odd: the power mod m (Montgomery), and its parity, that of (p + 1) / 4, from
+// which the residue mod 2 m follows.
+template <bool k31>
+__device__ __forceinline__ uint32_t root_exponent(uint32_t p, uint64_t L) {
+    const uint32_t m = (p - 1) / 2, h = (uint32_t)(((uint64_t)p + 1) / 4);  // h = (m + 1) / 2 <= m
+    if (m == 1) return 1;
+    const Mont<k31> M(m);
+    const uint32_t e = M.from(M.pow_m(M.to(h), L));
+    return ((e ^ h) & 1u) ? e + m : e;
+}
+
 // Decryption key check: p != q, both prime, = 3 mod 4, below 2^32, p q < 2^62.
 // The residues of x_0, the square root of y taken L times mod p and mod q,
 // and p^-1 mod q for joining them (Garner: x_0 = r_p + p ((r_q - r_p) p^-1
@@ -113,16 +125,15 @@ __device__ __forceinline__ bool bg_setup_encrypt(uint64_t N, uint64_t r, Barrett
 struct BgRoots {
     uint32_t p, q, rp, rq, pinv;
 };
+template <bool k31>  // k31: every factor of the warp is below 2^31
 __device__ __forceinline__ bool bg_setup_decrypt(uint64_t a, uint64_t b, uint64_t y, uint64_t L, BgRoots &s) {
     const uint64_t p = a < b ? a : b, q = a < b ? b : a;
     const bool ok = q < (1ull << 32) && (p & 3ull) == 3 && (q & 3ull) == 3 && p != q && p * q < (1ull << 62) &&
-                    is_prime_u32(p) && is_prime_u32(q);
+                    is_prime_u32<k31>(p) && is_prime_u32<k31>(q);
     s = BgRoots{(1u << 30) + 3u, (1u << 31) - 1u, 0u, 0u, 1u};
     if (ok) {
-        const Barrett32 Bp1(p - 1), Bq1(q - 1);      // even moduli: Barrett
-        const Mont32 Mp((uint32_t)p), Mq((uint32_t)q);  // odd primes: Montgomery
-        const uint64_t ep = Bp1.pow((p + 1) / 4, L);  // ((p+1)/4)^L mod (p-1)
-        const uint64_t eq = Bq1.pow((q + 1) / 4, L);
+        const Mont<k31> Mp((uint32_t)p), Mq((uint32_t)q);
+        const uint32_t ep = root_exponent<k31>((uint32_t)p, L), eq = root_exponent<k31>((uint32_t)q, L);
         // y mod N < p q, below p 2^32 and q 2^32: taken to Montgomery form by REDC
         const uint64_t yN = y < p * q ? y : y % (p * q);
         s.p = (uint32_t)p;
@@ -207,7 +218,11 @@ __global__ void __launch_bounds__(kBgWarps * 32, kBgMinBlocks)
         bool ok = false;
         if constexpr (kDecrypt) {
             BgRoots k{(1u << 30) + 3u, (1u << 31) - 1u, 0u, 0u, 1u};  // dead lanes: the dummy pair
-            if (live) ok = bg_setup_decrypt(key_a[msg], key_b[msg], y_in[msg], L, k);
+            const uint64_t fa = live ? key_a[msg] : 3, fb = live ? key_b[msg] : 3;
+            const bool short31 = __all_sync(0xFFFFFFFFu, fa < (1ull << 31) && fb < (1ull << 31));
+            if (live)
+                ok = short31 ? bg_setup_decrypt<true>(fa, fb, y_in[msg], L, k)
+                             : bg_setup_decrypt<false>(fa, fb, y_in[msg], L, k);
             if (live) key = S0[msg];
             if (live && !ok && n_rejected) atomicAdd(n_rejected, 1u);
             const uint32_t keep = ok ? 0xFFFFFFFFu : 0u;  // a rejected key's row is written as zeros

@@ -28,17 +28,6 @@ __host__ __device__ __forceinline__ uint32_t funnel_r32(uint32_t lo, uint32_t hi
 
 __host__ __device__ __forceinline__ uint32_t min32(uint32_t a, uint32_t b) { return a < b ? a : b; }
 
-// min(r + a, r) as unsigned words: one instruction on the device.  With
-// a = -m and r in [0, 2m) it is the residue r mod m (r - m wraps above r when
-// r < m).
-__host__ __device__ __forceinline__ uint32_t addmin32(uint32_t r, uint32_t a) {
-#ifdef __CUDA_ARCH__
-    return __viaddmin_u32(r, a, r);
-#else
-    return r + a < r ? r + a : r;
-#endif
-}
-
 // r^2 mod p for an odd modulus p in (2^30, 2^31) and r in [0, p), by Barrett
 // reduction with one subtraction.  r and p - r have the same square, so the
 // smaller of the two is squared: t <= (p - 1)^2 / 4 < 2^60.  With h = t >> 29
@@ -83,7 +72,7 @@ struct CrtModulus {
     __host__ __device__ __forceinline__ bool set(uint32_t a, uint32_t b) {
         const uint32_t lo = a < b ? a : b, hi = a < b ? b : a;
         if (lo <= (1u << 30) || hi >= (1u << 31) || lo == hi || !(lo & hi & 1u)) return false;
-        const Mont32 Mq(hi);
+        const Mont31 Mq(hi);
         const uint32_t pm = Mq.to(lo), inv = Mq.pow_m(pm, hi - 2);
         if (Mq.mul(inv, pm) != Mq.one) return false;
         set_inverse(lo, hi, Mq.from(inv));
@@ -110,7 +99,7 @@ struct CrtModulus {
     }
 };
 
-// 2^e mod (p - 1) for a prime p > 2, through the odd part of p - 1.
+// 2^e mod (p - 1) for a prime 2 < p < 2^31, through the odd part of p - 1.
 __host__ __device__ __forceinline__ uint32_t pow2_mod_order(uint32_t p, uint64_t e) {
     uint32_t m = p - 1, v = 0;
     while (!(m & 1u)) {
@@ -118,14 +107,14 @@ __host__ __device__ __forceinline__ uint32_t pow2_mod_order(uint32_t p, uint64_t
         ++v;
     }
     if (e < v || m == 1) return e < v ? 1u << e : 0u;
-    const Mont32 M(m);
+    const Mont31 M(m);
     return M.from(M.pow2_m(e - v)) << v;
 }
 
-// x^(2^e) mod p for a prime p, from and to the Montgomery form of x (`one`:
+// x^(2^e) mod p for a prime p < 2^31, from and to the Montgomery form of x (`one`:
 // that of 1): the exponent reduced mod p - 1.  e >= 1.
 __host__ __device__ __forceinline__ uint32_t squarings_m(uint32_t p, uint32_t one, uint32_t xm, uint64_t e) {
-    return Mont32(p, one).pow_m(xm, pow2_mod_order(p, e));
+    return Mont31(p, one).pow_m(xm, pow2_mod_order(p, e));
 }
 
 }  // namespace dev

@@ -5,6 +5,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "ci_device.cuh"
@@ -87,13 +88,23 @@ inline bool span_rows(uint64_t n, const uint32_t *out) {
 template <class Src>
 static cudaError_t launch_gen_span(const DevState &st, uint64_t n, uint32_t *out, cudaStream_t stream) {
     auto kern = k_generate_span<Src>;
-    static std::once_flag once;
-    std::call_once(once, [&] {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(128 * kSpanMax));
-        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    });
+    static_assert(128 * kSpanMax <= 48 * 1024, "staging within the default shared-memory limit");
+    static std::once_flag once;  // a hint: as many warps per SM as the shared memory holds
+    std::call_once(once, [&] { cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100); });
     kern<<<(unsigned)(st.P / 32), 32, 128 * n, stream>>>(st, (uint32_t)n, out);
     return cudaGetLastError();
+}
+
+// Lets `kern` use `smem` bytes of dynamic shared memory on the current device,
+// once per device (`done`: a bit per device ordinal, the kernel's own).
+template <class Kernel>
+static void allow_smem(Kernel kern, size_t smem, std::atomic<uint64_t> &done) {
+    if (smem <= 48 * 1024) return;
+    int dev = 0;
+    const bool known = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64;
+    if (known && (done.load(std::memory_order_relaxed) >> dev & 1u)) return;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (known) done.fetch_or(1ull << dev, std::memory_order_relaxed);
 }
 
 // Tensor map over out[rows][cols] (uint32, row stride cols words) with a
@@ -108,10 +119,11 @@ static cudaError_t launch_gen_tma(const DevState &st, uint64_t n, uint32_t *out,
     if (!make_out_tensor_map(&map, out, st.S, n)) return cudaSuccess;
     auto kern = k_generate_tma<Src, W>;
     const size_t smem = (size_t)W * 2 * 4096 + 1024;  // + slack for the 1024-byte alignment of the base
+    static std::atomic<uint64_t> smem_set{0};
+    allow_smem(kern, smem, smem_set);
     static std::once_flag once;
     static int per_sm = 1;
     std::call_once(once, [&] {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int ps = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kern, W * 32, smem) == cudaSuccess && ps > 0)
             per_sm = ps;
@@ -127,10 +139,11 @@ static cudaError_t launch_gen_t(const DevState &st, uint64_t n, uint32_t *out, u
                                 cudaStream_t stream) {
     auto kern = k_generate<Src, SINK, W, TC>;
     const size_t smem = (size_t)W * kTileVecs<SINK, TC> * sizeof(uint4);
+    static std::atomic<uint64_t> smem_set{0};
+    allow_smem(kern, smem, smem_set);
     static std::once_flag once;
     static int per_sm = 1;
     std::call_once(once, [&] {
-        if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int ps = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kern, W * 32, smem) == cudaSuccess && ps > 0)
             per_sm = ps;

@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(256) k_init_xor(DevState st, TableParam tp, ui
         init_xor_lane(st, seed, first, xl, l);
 }
 
-// Blum prime candidate from a draw: 2^30 + (d >> 34), forced to 3 mod 4.
+// Blum prime candidate from a draw: 2^30 + (d >> 34), forced to 3 mod 4 (below 2^31).
 __device__ __forceinline__ uint32_t blum_candidate(uint64_t d) {
     return (uint32_t)((1ull << 30) + (d >> 34)) | 3u;
 }
@@ -84,11 +84,11 @@ __device__ void init_bbs_lane(const DevState &st, uint64_t seed, uint64_t first,
     do {
         d = lane_draw(seed, first + l, k++);
         p = blum_candidate(d);
-    } while (!is_prime_u32(p));
+    } while (!is_prime_u32<true>(p));
     do {
         d = lane_draw(seed, first + l, k++);
         q = blum_candidate(d);
-    } while (q == p || !is_prime_u32(q));
+    } while (q == p || !is_prime_u32<true>(q));
     const uint64_t M = (uint64_t)p * q;
     uint64_t v;
     do {

@@ -27,6 +27,17 @@ __host__ __device__ __forceinline__ uint64_t umulhi64(uint64_t a, uint64_t b) {
 #endif
 }
 
+// min(r + a, r) as unsigned words: one instruction on the device.  With
+// a = -m and r in [0, 2m), 2m <= 2^32, it is the residue r mod m (r - m wraps
+// above r when r < m).
+__host__ __device__ __forceinline__ uint32_t addmin32(uint32_t r, uint32_t a) {
+#ifdef __CUDA_ARCH__
+    return __viaddmin_u32(r, a, r);
+#else
+    return r + a < r ? r + a : r;
+#endif
+}
+
 // Leading zeros of a nonzero word.
 __host__ __device__ __forceinline__ int clz32(uint32_t x) {
 #ifdef __CUDA_ARCH__
@@ -77,21 +88,30 @@ struct Barrett32 {
 // computed without the 65-bit sum: the low halves of t and u m cancel, with a
 // carry exactly when t mod R != 0.  Operands are 32-bit words, so a product
 // is one 32 x 32 -> 64-bit multiply and REDC one low and one high product.
-struct Mont32 {
+// k31: m < 2^31, where t + u m fits 64 bits and one multiply-add gives it: four
+// instructions a product (two of them wide) instead of about ten.
+template <bool k31>
+struct Mont {
     uint32_t m;
     uint32_t np;   // -m^-1 mod 2^32
     uint32_t one;  // R mod m, the Montgomery form of 1
     uint32_t r2;   // R^2 mod m
-    __host__ __device__ __forceinline__ explicit Mont32(uint32_t mod) : m(mod) {
+    __host__ __device__ __forceinline__ explicit Mont(uint32_t mod) : m(mod) {
         uint32_t inv = mod;  // Newton: each step doubles the correct low bits (3 to start)
 #pragma unroll
         for (int i = 0; i < 4; ++i) inv *= 2u - mod * inv;
         np = 0u - inv;
         one = (0u - mod) % mod;  // (2^32 - m) mod m = R mod m
-        r2 = (uint32_t)((uint64_t)one * one % mod);
+        if (k31) {  // the form of 2, squared five times: that of 2^32
+            r2 = addmin32(one + one, 0u - mod);
+#pragma unroll
+            for (int i = 0; i < 5; ++i) r2 = mul(r2, r2);
+        } else {
+            r2 = (uint32_t)((uint64_t)one * one % mod);
+        }
     }
     // From a stored `one`, without R^2 (for redc, mul, from and the powers).
-    __host__ __device__ __forceinline__ Mont32(uint32_t mod, uint32_t one_) : m(mod), one(one_), r2(0u) {
+    __host__ __device__ __forceinline__ Mont(uint32_t mod, uint32_t one_) : m(mod), one(one_), r2(0u) {
         uint32_t inv = mod;
 #pragma unroll
         for (int i = 0; i < 4; ++i) inv *= 2u - mod * inv;
@@ -99,6 +119,7 @@ struct Mont32 {
     }
     __host__ __device__ __forceinline__ uint32_t redc(uint64_t t) const {  // t < m R
         const uint32_t u = (uint32_t)t * np;
+        if (k31) return addmin32((uint32_t)((t + (uint64_t)u * m) >> 32), 0u - m);
         const uint64_t r = (t >> 32) + umulhi32(u, m) + ((uint32_t)t != 0u ? 1u : 0u);
         return (uint32_t)(r >= m ? r - m : r);
     }
@@ -138,20 +159,24 @@ struct Mont32 {
         for (int i = 63 - clz64(e | 1u); i >= 0; --i) {
             r = mul(r, r);
             const uint64_t d = 2ull * r;
-            const uint32_t rd = (uint32_t)(d >= m ? d - m : d);
+            const uint32_t rd = k31 ? addmin32(r + r, 0u - m) : (uint32_t)(d >= m ? d - m : d);
             r = (e >> i) & 1ull ? rd : r;
         }
         return r;
     }
 };
 
+using Mont32 = Mont<false>;
+using Mont31 = Mont<true>;
+
 // Miller-Rabin with bases 2, 7, 61: exact for odd n < 4,759,123,141
 // (Jaeschke 1993), so for every odd n in [3, 2^32).  A base that is a multiple
 // of n (n = 7, 61) proves nothing and is skipped.
+template <bool k31 = false>  // k31: n < 2^31
 __host__ __device__ __forceinline__ bool is_prime_u32(uint64_t n64) {
     if (n64 < 3 || n64 >= (1ull << 32) || (n64 & 1ull) == 0) return n64 == 2;
     const uint32_t n = (uint32_t)n64;
-    const Mont32 M(n);
+    const Mont<k31> M(n);
     const uint32_t one = M.one, minus_one = n - M.one;  // Montgomery forms of 1 and n - 1
     uint32_t d = n - 1;
     int s = 0;

@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(256) k_split_constants(DevState src, uint64_t 
         const uint32_t a = src.u32[F_P * P + l], b = src.u32[F_Q * P + l];
         if (crt_store(src, l, crt)) {
             const uint64_t y = src.u64[G_Y * P + l];
-            const Mont32 Mp(min(a, b)), Mq(max(a, b));
+            const Mont31 Mp(min(a, b)), Mq(max(a, b));
             uint32_t *jump = crt + kCrtWords * P + l;
             jump[0] = Mp.to((uint32_t)(y % Mp.m));
             jump[P] = Mq.to((uint32_t)(y % Mq.m));
@@ -330,7 +330,7 @@ __device__ __forceinline__ uint64_t bbs_jump_lane(const DevState &src, uint64_t 
     CrtModulus C;
     if (crt_load(src, l, crt, C)) {
         const uint32_t *jump = crt + kCrtWords * P + l;
-        const Mont32 Mp(C.P.p, jump[2 * P]), Mq(C.Q.p, jump[3 * P]);
+        const Mont31 Mp(C.P.p, jump[2 * P]), Mq(C.Q.p, jump[3 * P]);
         return C.value(Mp.from(squarings_m(C.P.p, Mp.one, jump[0], squarings)),
                        Mq.from(squarings_m(C.Q.p, Mq.one, jump[P], squarings)));
     }

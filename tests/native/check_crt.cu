@@ -87,6 +87,36 @@ int main() {
     printf("square modulo p q: %ld of %ld differ (%ld moduli)\n", bad, n, taken);
     all += bad;
 
+    // Mont31: products, conversions, powers; primality against the 32-bit form
+    bad = n = 0;
+    const uint32_t edge[] = {3u, 5u, 7u, 61u, 65535u, 1073741827u, 2147483629u, 2147483647u};
+    for (int t = 0; t < 60000; ++t) {
+        const uint32_t mod = t < 8 ? edge[t] : (uint32_t)((g() >> (33 + g() % 20)) | 3u);
+        const Mont31 M(mod);
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t a = k == 0 ? mod - 1 : (uint32_t)(g() % mod), b = k < 2 ? mod - 1 : (uint32_t)(g() % mod);
+            bad += M.from(M.mul(M.to(a), M.to(b))) != (uint32_t)((uint64_t)a * b % mod), ++n;
+            const uint64_t w = g() % ((uint64_t)mod << 32);
+            bad += M.from(M.to_wide(w)) != w % mod, ++n;
+            const uint64_t e = g() >> (g() % 64);
+            uint64_t r = 1 % mod, c = a, d = 1 % mod;
+            for (uint64_t x = e; x; x >>= 1) {
+                if (x & 1) r = r * c % mod;
+                c = c * c % mod;
+            }
+            c = 2 % mod;
+            for (uint64_t x = e; x; x >>= 1) {
+                if (x & 1) d = d * c % mod;
+                c = c * c % mod;
+            }
+            bad += M.from(M.pow_m(M.to(a), e)) != r, ++n;
+            bad += M.from(M.pow2_m(e)) != d, ++n;
+        }
+        bad += is_prime_u32<true>(mod) != is_prime_u32<false>(mod), ++n;
+    }
+    printf("31-bit Montgomery: %ld of %ld differ\n", bad, n);
+    all += bad;
+
     // squarings_m and pow2_mod_order over Blum primes and primes = 1 mod 4
     bad = n = 0;
     for (int k = 0; k < 400; ++k) {
