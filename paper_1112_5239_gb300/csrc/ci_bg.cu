@@ -29,6 +29,7 @@
 
 #include "ci_crt.cuh"
 #include "ci_device.cuh"
+#include "ci_gen.cuh"
 #include "ci_internal.h"
 #include "ci_modarith.cuh"
 #include "ci_trace.h"
@@ -198,16 +199,13 @@ template <bool kDecrypt, bool kVec>
 __global__ void __launch_bounds__(kBgWarps * 32, kBgMinBlocks)
     k_bg(uint64_t n_msgs, uint64_t L, const uint64_t *__restrict__ key_a, const uint64_t *__restrict__ key_b,
          const uint8_t *__restrict__ S0, const uint64_t *__restrict__ y_in, const uint8_t *in, uint8_t *out,
-         uint64_t *__restrict__ y_out, uint32_t *__restrict__ n_rejected) {
+         uint64_t *__restrict__ y_out, uint32_t *__restrict__ n_rejected, uint32_t in_order) {
     __shared__ __align__(16) uint8_t stage[kBgWarps][32 * kBgRowPad];
     const uint32_t lane = threadIdx.x & 31u;
     uint8_t *tile = stage[threadIdx.x >> 5];
     uint8_t *row = tile + lane * kBgRowPad;
-    const uint64_t n_groups = (n_msgs + 31) / 32;
-    const uint64_t stride = (uint64_t)gridDim.x * kBgWarps;
-    // warp w of block b starts at group w * gridDim.x + b, so a partial last
-    // round of warps is spread over every block (and SM)
-    for (uint64_t g = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; g < n_groups; g += stride) {
+    const uint64_t g = warp_group<kBgWarps>(in_order);  // at most one group a warp (gen_grid)
+    if (g < (n_msgs + 31) / 32) {
         const uint64_t m0 = g * 32;
         const uint64_t msg = m0 + lane;
         const bool live = msg < n_msgs;
@@ -236,7 +234,7 @@ __global__ void __launch_bounds__(kBgWarps * 32, kBgMinBlocks)
                 s.mask = mask;
                 s.key = key;
                 bg_rows<kVec>(s, keep, live, msg, m0, rows, L, in, out, tile, row, lane);
-                continue;
+                return;
             }
             // x_0 by Garner; p < q, so r_p < q
             const Mont32 Mq(k.q);
@@ -267,15 +265,14 @@ __global__ void __launch_bounds__(kBgWarps * 32, kBgMinBlocks)
 }
 
 template <bool kDecrypt, bool kVec>
-int bg_grid(uint64_t n_msgs) {
+GenGrid bg_grid(uint64_t n_msgs) {
     static int per_sm = 0;
     static std::once_flag once;
     std::call_once(once, [] {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bg<kDecrypt, kVec>, kBgWarps * 32, 0);
         if (per_sm <= 0) per_sm = 1;
     });
-    const uint64_t blocks = (n_msgs + 31) / 32;  // a block per warp group at most
-    return (int)std::min<uint64_t>(blocks, (uint64_t)sm_count() * per_sm);
+    return gen_grid((n_msgs + 31) / 32, kBgWarps, (uint64_t)sm_count() * per_sm);
 }
 
 ci_status bg_check(uint64_t n_msgs, uint64_t n_chunks, const void *a, const void *b, const void *S0,
@@ -296,12 +293,10 @@ template <bool kDecrypt>
 cudaError_t bg_launch(uint64_t n_msgs, uint64_t L, const uint64_t *a, const uint64_t *b, const uint8_t *S0,
                       const uint64_t *y_in, const uint8_t *in, uint8_t *out, uint64_t *y_out, uint32_t *n_rejected,
                       cudaStream_t stream) {
-    if (bg_vec(L, in, out))
-        k_bg<kDecrypt, true><<<bg_grid<kDecrypt, true>(n_msgs), kBgWarps * 32, 0, stream>>>(
-            n_msgs, L, a, b, S0, y_in, in, out, y_out, n_rejected);
-    else
-        k_bg<kDecrypt, false><<<bg_grid<kDecrypt, false>(n_msgs), kBgWarps * 32, 0, stream>>>(
-            n_msgs, L, a, b, S0, y_in, in, out, y_out, n_rejected);
+    const bool vec = bg_vec(L, in, out);
+    const GenGrid gg = vec ? bg_grid<kDecrypt, true>(n_msgs) : bg_grid<kDecrypt, false>(n_msgs);
+    auto kern = vec ? k_bg<kDecrypt, true> : k_bg<kDecrypt, false>;
+    kern<<<gg.grid, kBgWarps * 32, 0, stream>>>(n_msgs, L, a, b, S0, y_in, in, out, y_out, n_rejected, gg.in_order);
     return cudaGetLastError();
 }
 

@@ -596,13 +596,13 @@ __device__ __forceinline__ void store_words(uint32_t *p, const uint4 &v, int lo,
 // rows of 401 took 132 us by 16-byte, 108 by 32-byte boundaries.)  Output j of
 // the call stands at word (j + ph_r) mod 64 of the row's two lines, of which one
 // is stored after every 32 steps.  The lanes of one step write 32 different
-// banks when ld is odd.  `step` makes the lane's next output; kUnroll: it is short (the
-// tile's 32 steps are unrolled).
+// banks when ld is odd.  `step` makes the lane's next output; kUnroll of a
+// tile's 32 steps are unrolled.
 // (50001 x 1001 XORshift outputs: the word-wise form this replaces, a row per
 // warp-wide store, issued 34 instructions per step of a warp, 20 of them for
 // the stores.)
 constexpr int kTileVec = 32 * 16;  // 16-byte words of a warp's staging tile (the aligned 32 x 32 form: 256)
-template <bool kUnroll, int CACHE, class Step>
+template <int kUnroll, int CACHE, class Step>
 __device__ __forceinline__ void written_unaligned(Step step, uint64_t S, uint64_t row0, uint64_t n, uint32_t *out,
                                                   uint64_t ld, uint64_t col0, uint4 *tile) {
     const int lane = threadIdx.x & 31;
@@ -626,7 +626,7 @@ __device__ __forceinline__ void written_unaligned(Step step, uint64_t S, uint64_
         uint32_t *q = dst;
         const uint4 *from = stored + half / 4;
         if (at > 0 && at + 32 <= len && all_rows) {  // words of the rows only
-#pragma unroll(kUnroll ? 8 : 2)
+#pragma unroll(kUnroll > 1 ? 8 : 2)
             for (int k = 0; k < 8; ++k, q += 4 * ld) {
                 uint32_t *line = reinterpret_cast<uint32_t *>(reinterpret_cast<uintptr_t>(q) & ~(uintptr_t)127);
                 store16<CACHE>(line + 4 * c, from[64 * k]);
@@ -651,8 +651,8 @@ __device__ __forceinline__ void written_unaligned(Step step, uint64_t S, uint64_
     // word (ph + j + half) mod 64 of the lane's row, ph + j < 64
     auto place = [&](int j) { return j + ph < 32 ? w + half + j : w - half + j; };
     while (at + 32 <= len) {
-        if (!kUnroll) {
-#pragma unroll 1
+        if (kUnroll < 32) {
+#pragma unroll(kUnroll)
             for (int j = 0; j < 32; ++j) *place(j) = step();
         } else if (half == 0) {
 #pragma unroll
@@ -681,7 +681,7 @@ __device__ __forceinline__ uint64_t warp_run(Lane<Src> &s, uint64_t S, uint64_t 
     constexpr int CH = KT / 4;
     const int lane = threadIdx.x & 31;
     if constexpr (SINK == SINK_SCALAR) {
-        written_unaligned<!Src::kHeavy, TC::CACHE>([&]() { return s.step(); }, S, row0, n, out,
+        written_unaligned<Src::kHeavy ? 1 : 32, TC::CACHE>([&]() { return s.step(); }, S, row0, n, out,
                                                    ld, col0, tile);
         return 0;
     }

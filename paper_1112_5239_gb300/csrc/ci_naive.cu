@@ -148,23 +148,30 @@ __global__ void __launch_bounds__(256, CI_NAIVE_MIN_BLOCKS) k_naive_generate(Nai
         NaiveLane L;
         L.load(v.u64, v.x, v.P, l);
         if constexpr (!V4) {
-            written_unaligned<false, 0>([&]() { return L.next(); }, v.S, row0, n, out, n, 0, tile);
+            written_unaligned<4, 0>([&]() { return L.next(); }, v.S, row0, n, out, n, 0, tile);
         } else {
             const uint64_t nfull = n - n % 32;
-            for (uint64_t i0 = 0; i0 < n; i0 += 32) {
-                const int chunks = i0 < nfull ? 8 : (int)(n - nfull) / 4;
-                if (chunks == 8) {
+            for (uint64_t i0 = 0; i0 < nfull; i0 += 32) {
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) tile[lane * 8 + (q ^ (lane & 7))] = next4(L);
-                } else {
-                    for (int q = 0; q < chunks; ++q) tile[lane * 8 + (q ^ (lane & 7))] = next4(L);
-                }
+                for (int q = 0; q < 8; ++q) tile[lane * 8 + (q ^ (lane & 7))] = next4(L);
                 __syncwarp();
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     const int r = 4 * k + lane / 8, c = lane % 8;
+                    if (row0 + r < v.S) store16<0>(out + (row0 + r) * n + i0 + 4 * c, tile[r * 8 + (c ^ (r & 7))]);
+                }
+                __syncwarp();
+            }
+            const int chunks = (int)(n - nfull) / 4;
+            if (chunks) {
+#pragma unroll 1
+                for (int q = 0; q < chunks; ++q) tile[lane * 8 + (q ^ (lane & 7))] = next4(L);
+                __syncwarp();
+#pragma unroll 1
+                for (int k = 0; k < 8; ++k) {
+                    const int r = 4 * k + lane / 8, c = lane % 8;
                     if (row0 + r < v.S && c < chunks)
-                        store16<0>(out + (row0 + r) * n + i0 + 4 * c, tile[r * 8 + (c ^ (r & 7))]);
+                        store16<0>(out + (row0 + r) * n + nfull + 4 * c, tile[r * 8 + (c ^ (r & 7))]);
                 }
                 __syncwarp();
             }
