@@ -833,20 +833,27 @@ __device__ __forceinline__ void tma_store_tile(const CUtensorMap *map, const voi
                  : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
-// Wait until at most one committed store still reads its shared-memory source.
-__device__ __forceinline__ void tma_wait_read_1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
-__device__ __forceinline__ void tma_wait_read_0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+// Wait until at most kLeft committed stores still read their shared-memory source.
+template <int kLeft>
+__device__ __forceinline__ void tma_wait_read() {
+    asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kLeft) : "memory");
+}
 // Make this thread's ordinary shared-memory writes visible to the TMA unit.
 __device__ __forceinline__ void fence_smem_to_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// Written sink through TMA: per 32-iteration tile, the lanes fill one of two
-// 4 KB tiles (double buffering: a tile is refilled only after the store issued
-// from it two tiles earlier has read it), then lane 0 issues the tile's bulk
+// Written sink through TMA: per 32-iteration tile, the lanes fill one of
+// kTmaTiles 4 KB tiles in turn (refilled only after the store issued from it
+// has read it), then lane 0 issues the tile's bulk
 // tensor store at (column i0, row 32 g).  The TMA unit clips rows past the
 // tensor's row count (streams >= S) and, in a last tile of fewer than 32
-// iterations, columns past n.  `tiles` is 2 x 4 KB, 1024-byte aligned.
+// iterations, columns past n.  `tiles` is kTmaTiles x 4 KB, 1024-byte aligned.
 // Requires out 16-byte aligned and n % 4 == 0 (checked by the host when it
 // builds the tensor map).
+// Tiles per warp.  A third one covers the time a store waits behind the others
+// of a busy memory: 100000 x 1500 xor64 188 us with two, 162 with three, 156
+// with four; 2^20 x 256 xor128 176 / 173 / 175, xor64 189 / 193 / 199 (fewer
+// warps beside the tiles).
+constexpr int kTmaTiles = 3;
 template <class Src>
 __device__ __forceinline__ void warp_task_tma(const DevState &st, uint64_t g, uint64_t n, const CUtensorMap *map,
                                               uint4 *tiles) {
@@ -860,9 +867,9 @@ __device__ __forceinline__ void warp_task_tma(const DevState &st, uint64_t g, ui
     const uint64_t policy = l2_evict_first_policy();
     int k = 0;
     for (uint64_t i0 = 0; i0 < n; i0 += 32, ++k) {
-        uint4 *tile = tiles + (k & 1) * 256;
-        if (k >= 2) {
-            if (lane == 0) tma_wait_read_1();
+        uint4 *tile = tiles + k % kTmaTiles * 256;
+        if (k >= kTmaTiles) {
+            if (lane == 0) tma_wait_read<kTmaTiles - 1>();
             __syncwarp();
         }
         auto chunk = [&](int q) {
@@ -885,7 +892,7 @@ __device__ __forceinline__ void warp_task_tma(const DevState &st, uint64_t g, ui
         if (lane == 0) tma_store_tile(map, tile, (int)i0, (int)(g * 32), policy);
     }
     s.store(st, l);
-    if (lane == 0) tma_wait_read_0();  // every store has read its tile before the block exits
+    if (lane == 0) tma_wait_read<0>();  // every store has read its tile before the block exits
     __syncwarp();
 }
 
@@ -947,7 +954,7 @@ __device__ __forceinline__ void warp_task_span(const DevState &st, uint64_t g, u
         for (uint32_t i = lane; i < words; i += 32) dst[i] = stage[i];
     }
     s.store(st, l);
-    if (lane == 0) tma_wait_read_0();  // the store has read the stage before the block exits
+    if (lane == 0) tma_wait_read<0>();  // the store has read the stage before the block exits
     __syncwarp();
 }
 

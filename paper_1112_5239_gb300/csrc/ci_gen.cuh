@@ -19,8 +19,8 @@ namespace ci {
 // dies, one memory each), so a fixed share per SM ends with the slowest, and
 // stores in address order reach 7.6 TB/s where the same stores from a
 // persistent grid reached 6.5 (1 GiB, nothing else in the kernel).  Measured
-// against a persistent grid: 2^20 x 1024 consumed 610 instead of 690 us, 2^20
-// x 256 written 175 instead of 199 us.  A state of fewer groups runs in one
+// against a persistent grid when it was brought in: 2^20 x 1024 consumed 610
+// instead of 690 us, 2^20 x 256 written 175 instead of 199 us.  A state of fewer groups runs in one
 // wave: one block per group as far as blocks are resident, and warp w of block
 // b takes group w * gridDim.x + b, so that every SM gets its share of the warps.
 // Either way a warp has at most one group.
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(W * 32) k_generate_tma(DevState st, uint64_t n
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(tma_tiles);
     uint4 *base = reinterpret_cast<uint4 *>(reinterpret_cast<char *>(tma_tiles) + ((1024u - (sbase & 1023u)) & 1023u));
     const int w = threadIdx.x >> 5;
-    uint4 *tiles = base + w * 512;  // two 4 KB tiles per warp
+    uint4 *tiles = base + w * 256 * dev::kTmaTiles;
     const uint64_t g = warp_group<W>(in_order);
     if (g < st.P / 32) dev::warp_task_tma<Src>(st, g, n, &map, tiles);
 }
@@ -118,7 +118,7 @@ static cudaError_t launch_gen_tma(const DevState &st, uint64_t n, uint32_t *out,
     CUtensorMap map;
     if (!make_out_tensor_map(&map, out, st.S, n)) return cudaSuccess;
     auto kern = k_generate_tma<Src, W>;
-    const size_t smem = (size_t)W * 2 * 4096 + 1024;  // + slack for the 1024-byte alignment of the base
+    const size_t smem = (size_t)W * dev::kTmaTiles * 4096 + 1024;  // + slack for the 1024-byte alignment of the base
     static std::atomic<uint64_t> smem_set{0};
     allow_smem(kern, smem, smem_set);
     static std::once_flag once;

@@ -22,8 +22,8 @@ static ci_tune_table g_table = [] {
     ci_tune_table t;
     std::memset(&t, 0, sizeof t);
     // Without a tuning run: blocks of 4 warps for the xor-likes (handed out in
-    // order, see ci_gen.cuh: 2^20 x 1024 consumed 610 us, 630 with 8 and 16
-    // warps) and, for their aligned rows, TMA tiles (2^20 x 256: 176 us, 180 by
+    // order, see ci_gen.cuh: 2^20 x 1024 consumed 610 us then, 630 with 8 and
+    // 16 warps) and, for their aligned rows, TMA tiles (2^20 x 256: 173 us, 180 by
     // 16-byte stores); 8 for the BBS sources.
     for (int s = 0; s < kSrcKinds; ++s)
         for (int k = 0; k < 4; ++k) {
