@@ -185,8 +185,9 @@ ci_status ci_generate(ci_states states, uint64_t n_per_stream, uint32_t *out_dev
  * generator k (state and modulus) moves to place k + 1.
  * For CI_VAR_BBS, each strategy word takes ceil(32/w) BBS outputs' low w bits (w = floor(log2 log2 M) = 5
  * for these 62-bit moduli), then twice: shift = BBS & 3; t <<= shift;
- * t |= BBS & {0,1,3,7}[shift] -- 11 modular squarings per output, done with
- * 64x64->128-bit multiplies and Barrett reduction.  The stream's two
+ * t |= BBS & {0,1,3,7}[shift] -- 11 modular squarings per output, done on the
+ * residues of the two factors of M (62-bit Barrett squares where an imported
+ * modulus has a factor outside (2^30, 2^31)).  The stream's two
  * combination arrays are comb[sel1] and comb[8 + sel2] with sel1 = v & 7,
  * sel2 = (v >> 3) & 7 of its BBS seed v.  A CI_VAR_BBS state is run as
  * time segments, as ci_generate_split does, with identical results, unless

@@ -20,7 +20,7 @@
 // read directly; a warp whose moduli all have at least 34 bits takes its
 // limb form.  Decryption knows the factors: a warp whose factors all lie in
 // (2^30, 2^31) squares their residues instead (ci_crt.cuh), starting from the
-// two square roots, and never forms x_0 (2^18 x 1024: 390 us against 578 in
+// two square roots, and never forms x_0 (2^18 x 1024: 334 us against 578 in
 // the 62-bit form).
 #include <cuda_runtime.h>
 
@@ -41,7 +41,8 @@ using namespace dev;
 
 // Resident blocks per SM asked of the register allocator: 64 registers, no
 // spills (2^18 x 1024: decryption 365 us, 375 with 5 blocks, 379 with 3;
-// encryption 437, 447 and 457).
+// encryption 437, 447 and 457; blocks in order, gen_grid, took another 23 us
+// off each).
 constexpr int kBgMinBlocks = 4;
 
 constexpr int kBgWarps = 8;    // warps per block

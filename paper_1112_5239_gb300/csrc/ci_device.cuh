@@ -332,8 +332,8 @@ struct SrcBbs {
 
 // The same source on the residues of the two factors (ci_crt.cuh), bound by
 // the FMA-heavy pipe as the 62-bit form is, but with 30 instead of 51 cycles
-// of it per squaring of a warp: 2^16 x 4096 outputs in 3.28 instead of 5.38
-// ms, 300 uneven requests in one launch 4.52 instead of 6.88 ms.  Its constants are computed from
+// of it per squaring of a warp: 2^16 x 4096 outputs in 3.10 instead of 5.38
+// ms, 300 uneven requests in one launch 4.46 instead of 6.88 ms.  Its constants are computed from
 // the state's p and q when a warp's work starts, or read from `crt` (kCrtWords
 // fields of P words, written by crt_store) where a call prepares them once for
 // many units.  load() is false in every lane unless all lanes of the warp hold
@@ -600,7 +600,7 @@ __device__ __forceinline__ void store_words(uint32_t *p, const uint4 &v, int lo,
 // tile's 32 steps are unrolled.
 // (50001 x 1001 XORshift outputs: the word-wise form this replaces, a row per
 // warp-wide store, issued 34 instructions per step of a warp, 20 of them for
-// the stores.)
+// the stores, and took 82 us; now 57.)
 constexpr int kTileVec = 32 * 16;  // 16-byte words of a warp's staging tile (the aligned 32 x 32 form: 256)
 template <int kUnroll, int CACHE, class Step>
 __device__ __forceinline__ void written_unaligned(Step step, uint64_t S, uint64_t row0, uint64_t n, uint32_t *out,

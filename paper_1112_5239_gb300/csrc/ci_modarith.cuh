@@ -58,7 +58,8 @@ __host__ __device__ __forceinline__ int clz64(uint64_t x) {
 // x mod m for x < 2^64 and 2 <= m < 2^32, with mu = floor((2^64 - 1) / m).
 // The quotient estimate q = floor(x mu / 2^64) satisfies
 // x/m - 2 < q <= x/m, so x - q m lies in [0, 3m): two conditional
-// subtractions give the residue.
+// subtractions give the residue.  (The kernels go through Mont; the host check
+// holds this form beside it.)
 struct Barrett32 {
     uint64_t m, mu;
     __host__ __device__ __forceinline__ explicit Barrett32(uint64_t mod) : m(mod), mu(~0ull / mod) {}

@@ -14,8 +14,8 @@
 // Steps of one call (all on the caller's stream):
 //   1. k_split_setup: segment states k = 0 .. K-1 are copies of the state
 //      with the own generator jumped ahead by k len iterations (GF(2) matrix
-//      powers for the xor-likes, x <- x^(2^(11 k len) mod lambda(M)) for BBS,
-//      each of the eight 16-bit generators by its own squaring count for
+//      powers for the xor-likes, for BBS x <- x^(2^(11 k len)) modulo each
+//      factor, the exponent mod p - 1, each of the eight 16-bit generators by its own squaring count for
 //      Algorithm 5 as printed) and (s, x) = (0, 0) for k >= 1;
 //   2. written outputs of the BBS sources (62-bit and Algorithm 5 as
 //      printed), where generation is the cost, with many warp groups:
@@ -31,14 +31,16 @@
 //      k_split_fixup runs all fix-ups at once;
 //   4. otherwise (xor-like outputs are cheaper to generate again than to
 //      read back, and consumer sinks have no outputs to fix): pass 1
-//      (k_split_run) runs segments 0 .. K-2 for their end states alone; k_split_carry, one block per warp group,
-//      scans the segments: the true start of segment k is its predecessor's
+//      (k_split_run) runs segments 0 .. K-2 for their end states alone;
+//      k_split_carry, one cluster of blocks per warp group, scans the segments: the true start of segment k is its predecessor's
 //      particular end plus (Q s_a, x_a ^ S s_a) with Q = P^len,
 //      S = P + ... + P^len (a chunked parallel scan over up to 32 warps);
 //      pass 2 (k_split_run) runs every segment from its true start, with the
 //      own words k_split_setup jumped to, into the sink;
 //   5. the last segment's end state becomes the caller's state, and the
 //      per-segment quarter-circle counts or digests are combined.
+// A short call of a narrow xor-like state does all of it in one launch
+// (k_narrow); single_call chooses among the forms.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
