@@ -551,8 +551,9 @@ ci_status ci_naive_generate(void *state_dev, uint64_t n_streams, uint64_t n_per_
  * group per SM in calls of at least 2048 iterations (up to 16384 in one launch
  * of their own), and CI_VAR_BBS16 states of at most one warp group per SM.)
  * Method: each segment's own generator is jumped ahead (xor-likes: GF(2)
- * matrix powers of their step; BBS: x <- x^(2^(11 k len) mod lcm(p-1, q-1))
- * mod M), the segments run from a zero mixing state, a per-warp scan restores
+ * matrix powers of their step; BBS: x <- x^(2^(11 k len)) mod M, the exponent
+ * reduced by the orders of p and q, or by Carmichael's lambda of M where an
+ * imported modulus or state needs it), the segments run from a zero mixing state, a per-warp scan restores
  * their true starts from the linearity of Algorithm 4/5's mixing and Eq.
  * (Oplus) over the lanes, and the segments run again from those starts into
  * the sink (written BBS-source outputs are corrected in place instead: the

@@ -99,7 +99,7 @@ struct CrtModulus {
     }
 };
 
-// 2^e mod (p - 1) for a prime 2 < p < 2^31, through the odd part of p - 1.
+// 2^e mod (p - 1) for 2 < p < 2^31, through the odd part of p - 1.
 __host__ __device__ __forceinline__ uint32_t pow2_mod_order(uint32_t p, uint64_t e) {
     uint32_t m = p - 1, v = 0;
     while (!(m & 1u)) {
@@ -111,8 +111,9 @@ __host__ __device__ __forceinline__ uint32_t pow2_mod_order(uint32_t p, uint64_t
     return M.from(M.pow2_m(e - v)) << v;
 }
 
-// x^(2^e) mod p for a prime p < 2^31, from and to the Montgomery form of x (`one`:
-// that of 1): the exponent reduced mod p - 1.  e >= 1.
+// x^(2^e) mod p for an odd p < 2^31 and an x with x^(p-1) = 1 mod p, from and to
+// the Montgomery form of x (`one`: that of 1): the exponent reduced mod p - 1.
+// e >= 1.
 __host__ __device__ __forceinline__ uint32_t squarings_m(uint32_t p, uint32_t one, uint32_t xm, uint64_t e) {
     return Mont31(p, one).pow_m(xm, pow2_mod_order(p, e));
 }

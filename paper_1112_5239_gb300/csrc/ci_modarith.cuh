@@ -205,5 +205,42 @@ __host__ __device__ __forceinline__ bool is_prime_u32(uint64_t n64) {
     return true;
 }
 
+__host__ __device__ __forceinline__ uint64_t gcd64(uint64_t a, uint64_t b) {
+    while (b) {
+        const uint64_t t = a % b;
+        a = b;
+        b = t;
+    }
+    return a;
+}
+__host__ __device__ __forceinline__ uint64_t lcm64(uint64_t a, uint64_t b) { return a / gcd64(a, b) * b; }
+
+// Carmichael's lambda of M = a b for any odd a, b in [3, 2^32): the least
+// common multiple of r^(k-1) (r - 1) over the prime powers r^k of M, found by
+// trial division.  For every x and every E with 2^E >= 62 (no prime power of M
+// < 2^62 has a larger exponent), x^(2^E) = x^e mod M with
+// e = (2^E mod lambda) + lambda, whether x is a unit or not.
+__host__ __device__ inline uint64_t carmichael(uint32_t a, uint32_t b) {
+    uint64_t lam = 1;
+    while (a > 1 || b > 1) {
+        if (a == 1) {
+            a = b;
+            b = 1;
+        }
+        uint32_t r = a;
+        if (!is_prime_u32(a))
+            for (r = 3; a % r != 0;) r += 2;
+        uint64_t t = r - 1;
+        bool first = true;
+        for (uint32_t *v = &a;; v = &b) {
+            for (; *v % r == 0; *v /= r, first = false)
+                if (!first) t *= r;
+            if (v == &b) break;
+        }
+        lam = lcm64(lam, t);
+    }
+    return lam;
+}
+
 }  // namespace dev
 }  // namespace ci

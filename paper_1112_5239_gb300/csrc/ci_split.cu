@@ -15,7 +15,7 @@
 //   1. k_split_setup: segment states k = 0 .. K-1 are copies of the state
 //      with the own generator jumped ahead by k len iterations (GF(2) matrix
 //      powers for the xor-likes, for BBS x <- x^(2^(11 k len)) modulo each
-//      factor, the exponent mod p - 1, each of the eight 16-bit generators by its own squaring count for
+//      factor, the exponent mod p - 1 (k_split_constants), each of the eight 16-bit generators by its own squaring count for
 //      Algorithm 5 as printed) and (s, x) = (0, 0) for k >= 1;
 //   2. written outputs of the BBS sources (62-bit and Algorithm 5 as
 //      printed), where generation is the cost, with many warp groups:
@@ -212,17 +212,8 @@ cudaError_t ensure_jump_tables(cudaStream_t stream) {
 
 // ------------------------------------------------ BBS jump
 // x <- x^(2^E) mod M with E = 11 * dist squarings, through the exponent
-// 2^E mod lambda(M), lambda = lcm(p - 1, q - 1) (x is a unit mod M);
-// lambda and its Barrett reciprocal come from k_split_constants.
-__device__ __forceinline__ uint64_t gcd64(uint64_t a, uint64_t b) {
-    while (b) {
-        const uint64_t t = a % b;
-        a = b;
-        b = t;
-    }
-    return a;
-}
-
+// (2^E mod lambda) + lambda with lambda from k_split_constants: Carmichael's
+// lambda of M, which holds for every x, or a multiple of the order of x.
 // a^e mod M for a < M, left to right over 2-bit windows of e: two squarings
 // and one product by a^w (by 1 for w = 0) per window, the same work in every
 // lane whatever its exponent bits.
@@ -246,7 +237,7 @@ __device__ __forceinline__ uint64_t bbs_jump(uint64_t y, uint64_t M, uint64_t mu
     Barrett62 L;
     L.set(lam, lam_mu);
     // 2^squarings mod lam by square-and-multiply on the exponent's bits
-    const uint64_t e = pow_mod(L, 2 % lam, squarings);
+    const uint64_t e = pow_mod(L, 2 % lam, squarings) + lam;
     Barrett62 B;
     B.set(M, mu);
     return pow_mod(B, y, e);
@@ -300,28 +291,51 @@ __constant__ uint32_t c_bbs16_squarings[8] = {2, 2, 2, 1, 1, 1, 2, 1};
 
 // Once per lane, for every segment: the constants of the residue form
 // (crt_store) and, in kJumpWords fields behind them, what its jump starts from
-// (the Montgomery forms of y mod p, y mod q, 1 mod p and 1 mod q, p < q).
-// Lanes that do not take the residue form get lambda(M) = lcm(p - 1, q - 1)
-// and its Barrett reciprocal instead: lam[l] = lambda, lam[P + l] =
-// barrett_mu(lambda).
+// (the Montgomery forms of y mod p, y mod q, 1 mod p and 1 mod q, p < q), or
+// lam[l] = lambda and lam[P + l] = barrett_mu(lambda) for bbs_jump.
+// An imported state may have factors that are not prime or not distinct, or a
+// y that is no unit.  The exponents may be reduced modulo p - 1 and q - 1 if
+// y^(p-1) = 1 mod p and y^(q-1) = 1 mod q, which all seeded lanes pass and is
+// tested here.  Lanes that fail jump by Carmichael's lambda of their M, factored
+// by trial division (some tenths of a millisecond).
+// Three threads per lane, in warps of their own: the residue constants, the
+// test of p, the test of q, one power each (one thread after the other: 4 us
+// more for 32 streams).  A failed test leaves its `one` field 0.
 constexpr int kJumpWords = 4;
 __global__ void __launch_bounds__(256) k_split_constants(DevState src, uint64_t *lam, uint32_t *crt) {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, P = src.P;
-    for (uint64_t l = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; l < P; l += stride) {
+    for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < 3 * P; t += stride) {
+        const uint64_t l = t % P;
+        const int role = (int)(t / P);
         const uint32_t a = src.u32[F_P * P + l], b = src.u32[F_Q * P + l];
-        if (crt_store(src, l, crt)) {
-            const uint64_t y = src.u64[G_Y * P + l];
-            const Mont31 Mp(min(a, b)), Mq(max(a, b));
-            uint32_t *jump = crt + kCrtWords * P + l;
-            jump[0] = Mp.to((uint32_t)(y % Mp.m));
-            jump[P] = Mq.to((uint32_t)(y % Mq.m));
-            jump[2 * P] = Mp.one;
-            jump[3 * P] = Mq.one;
+        const bool range = min(a, b) > (1u << 30) && max(a, b) < (1u << 31);
+        const uint64_t y = src.u64[G_Y * P + l];
+        uint64_t v;
+        if (role == 0) {
+            if (crt_store(src, l, crt)) continue;
+            v = 0;
+            if (!range) {
+                Barrett62 B;
+                B.set(src.u64[G_M * P + l], src.u64[G_MU * P + l]);
+                v = lcm64(a - 1, b - 1);
+                if (pow_mod(B, y, v) != 1) v = 0;
+            }
         } else {
-            const uint64_t p = a, q = b, v = (p - 1) / gcd64(p - 1, q - 1) * (q - 1);
-            lam[l] = v;
-            lam[P + l] = barrett_mu(v);
+            uint32_t *jump = crt + (kCrtWords + role - 1) * P + l;
+            jump[2 * P] = 0u;
+            if (!range) continue;
+            const Mont31 Mf(role == 1 ? min(a, b) : max(a, b));
+            const uint32_t yf = Mf.to((uint32_t)(y % Mf.m));
+            if (Mf.pow_m(yf, Mf.m - 1) == Mf.one) {
+                jump[0] = yf;
+                jump[2 * P] = Mf.one;
+                continue;
+            }
+            v = 0;
         }
+        if (!v) v = carmichael(a, b);
+        lam[l] = v;  // of one lane: the same value, whichever of its threads get here
+        lam[P + l] = barrett_mu(v);
     }
 }
 
@@ -330,8 +344,8 @@ __device__ __forceinline__ uint64_t bbs_jump_lane(const DevState &src, uint64_t 
                                                   const uint64_t *lam, const uint32_t *crt) {
     const uint64_t P = src.P;
     CrtModulus C;
-    if (crt_load(src, l, crt, C)) {
-        const uint32_t *jump = crt + kCrtWords * P + l;
+    const uint32_t *jump = crt + kCrtWords * P + l;
+    if (crt_load(src, l, crt, C) && jump[2 * P] && jump[3 * P]) {
         const Mont31 Mp(C.P.p, jump[2 * P]), Mq(C.Q.p, jump[3 * P]);
         return C.value(Mp.from(squarings_m(C.P.p, Mp.one, jump[0], squarings)),
                        Mq.from(squarings_m(C.Q.p, Mq.one, jump[P], squarings)));
@@ -1406,7 +1420,7 @@ ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *ou
 
     ci_status st = CI_OK;
     if (b16) k_split_lambda16<<<split_block_count(8 * h->P), 256, 0, stream>>>(src, lam16);
-    if (bbs) k_split_constants<<<split_block_count(h->P), 256, 0, stream>>>(src, lam64, crt);
+    if (bbs) k_split_constants<<<split_block_count(3 * h->P), 256, 0, stream>>>(src, lam64, crt);
     k_split_setup<<<split_block_count(slots * h->P), 256, 0, stream>>>(src, sp, (uint32_t)K, len, h->variant, h->xl,
                                                                        own, lam16, lam64, crt);
     if ((e = cudaGetLastError()) != cudaSuccess) st = cuda_fail(e, "split setup");
