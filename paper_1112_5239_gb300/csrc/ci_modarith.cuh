@@ -205,21 +205,22 @@ __host__ __device__ __forceinline__ bool is_prime_u32(uint64_t n64) {
     return true;
 }
 
-__host__ __device__ __forceinline__ uint64_t gcd64(uint64_t a, uint64_t b) {
-    while (b) {
-        const uint64_t t = a % b;
-        a = b;
-        b = t;
+template <class T>  // 32- or 64-bit words
+__host__ __device__ __forceinline__ T lcm(T a, T b) {
+    T g = a, r = b;
+    while (r) {
+        const T t = g % r;
+        g = r;
+        r = t;
     }
-    return a;
+    return a / g * b;
 }
-__host__ __device__ __forceinline__ uint64_t lcm64(uint64_t a, uint64_t b) { return a / gcd64(a, b) * b; }
 
 // Carmichael's lambda of M = a b for any odd a, b in [3, 2^32): the least
 // common multiple of r^(k-1) (r - 1) over the prime powers r^k of M, found by
-// trial division.  For every x and every E with 2^E >= 62 (no prime power of M
-// < 2^62 has a larger exponent), x^(2^E) = x^e mod M with
-// e = (2^E mod lambda) + lambda, whether x is a unit or not.
+// trial division.  For every x and every E with 2^E >= 62, x^(2^E) = x^e mod M
+// with e = (2^E mod lambda) + lambda, whether x is a unit or not: both
+// exponents reach the exponent of every prime power of M < 2^62.
 __host__ __device__ inline uint64_t carmichael(uint32_t a, uint32_t b) {
     uint64_t lam = 1;
     while (a > 1 || b > 1) {
@@ -237,7 +238,30 @@ __host__ __device__ inline uint64_t carmichael(uint32_t a, uint32_t b) {
                 if (!first) t *= r;
             if (v == &b) break;
         }
-        lam = lcm64(lam, t);
+        lam = lcm(lam, t);
+    }
+    return lam;
+}
+
+// Carmichael's lambda of any M in [2, 2^16) (even ones and prime powers
+// too); the exponents as above, for 2^E >= 15.  Twice lambda where 8 but not
+// 16 divides M: lambda(8) = 2 is below the exponent of its 2^3, the one case.
+// The product of two primes, all that a seeded state holds, leaves the search
+// at its smaller factor, and the lanes of a warp go on together.
+__host__ __device__ inline uint32_t carmichael16(uint32_t M) {
+    uint32_t r = 3;
+    while (r * r <= M && M % r != 0) r += 2;
+    const uint32_t cofactor = M / r;
+    if ((M & 1u) && M == r * cofactor && r < cofactor && cofactor < r * r) return lcm(r - 1, cofactor - 1);
+    uint32_t rest = M, v = 0;
+    for (; !(rest & 1u); rest >>= 1) ++v;
+    uint32_t lam = 1u << (v < 2 ? 0 : v < 4 ? v - 1 : v - 2);
+    for (r = 3; rest > 1; r += 2) {
+        if (r * r > rest) r = rest;  // a prime
+        if (rest % r) continue;
+        uint32_t t = r - 1;
+        for (rest /= r; rest % r == 0; rest /= r) t *= r;
+        lam = lcm(t, lam);
     }
     return lam;
 }

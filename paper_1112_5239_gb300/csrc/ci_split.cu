@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(256) k_split_constants(DevState src, uint64_t 
             if (!range) {
                 Barrett62 B;
                 B.set(src.u64[G_M * P + l], src.u64[G_MU * P + l]);
-                v = lcm64(a - 1, b - 1);
+                v = lcm<uint64_t>(a - 1, b - 1);
                 if (pow_mod(B, y, v) != 1) v = 0;
             }
         } else {
@@ -353,27 +353,12 @@ __device__ __forceinline__ uint64_t bbs_jump_lane(const DevState &src, uint64_t 
     return bbs_jump(src.u64[G_Y * P + l], src.u64[G_M * P + l], src.u64[G_MU * P + l], lam[l], lam[P + l], squarings);
 }
 
-// lambda(M) = lcm(p - 1, q - 1) of each 16-bit modulus M = p q (p != q primes,
-// as seeded), by trial division; lam[k * P + l] for generator k of lane l.
+// Carmichael's lambda of each 16-bit modulus; lam[k * P + l] for generator k of
+// lane l.
 __global__ void __launch_bounds__(256) k_split_lambda16(DevState src, uint32_t *lam) {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < 8 * src.P; t += stride) {
-        const uint32_t M = src.u32[F_M16 * src.P + t];  // generator t / P of lane t % P
-        uint32_t p = M;  // a prime M (not seeded) gets lambda = M - 1
-        for (uint32_t d = 3; d * d <= M; d += 2)
-            if (M % d == 0) {
-                p = d;
-                break;
-            }
-        const uint32_t q = p == M ? 2u : M / p;
-        uint32_t a = p - 1, b = q - 1;
-        while (b) {
-            const uint32_t t2 = a % b;
-            a = b;
-            b = t2;
-        }
-        lam[t] = (p - 1) / a * (q - 1);
-    }
+    for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < 8 * src.P; t += stride)
+        lam[t] = carmichael16(src.u32[F_M16 * src.P + t]);  // generator t / P of lane t % P
 }
 
 // a^e mod m for m < 2^16 (products fit 32 bits).
@@ -414,9 +399,9 @@ __global__ void __launch_bounds__(256) k_split_setup(DevState src, SegSpace seg,
         d.u32[F_SLOT * src.P + l] = 0;
         const uint64_t dist = k * len;
         if (variant == CI_VAR_BBS16) {
-            for (int g = 0; g < 8; ++g) {  // x <- x^(2^(c_g dist) mod lambda(M)) mod M
+            for (int g = 0; g < 8; ++g) {  // x <- x^(2^(c_g dist)) mod M, for any x and M (carmichael16)
                 const uint32_t M = src.u32[(F_M16 + g) * src.P + l], lam = lam16[(uint64_t)g * src.P + l];
-                const uint32_t e = pow_mod16(2, c_bbs16_squarings[g] * dist, lam);
+                const uint32_t e = pow_mod16(2, c_bbs16_squarings[g] * dist, lam) + lam;
                 d.u32[(F_Y16 + g) * src.P + l] = pow_mod16(src.u32[(F_Y16 + g) * src.P + l], e, M);
             }
         } else if (variant == CI_VAR_BBS) {

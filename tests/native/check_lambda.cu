@@ -46,6 +46,15 @@ int main() {
         bad += differs(m, lam, g() % m, 352), ++n;
     }
     printf("two factors: %ld of %ld differ\n", bad, n);
+    long all = bad;
+    bad = n = 0;
+    for (uint32_t m = 3; m < (1u << 16); ++m) {  // every modulus a 16-bit generator may have
+        const uint64_t lam = carmichael16(m);
+        for (uint64_t x : {(uint64_t)0, (uint64_t)2, (uint64_t)3, (uint64_t)15, (uint64_t)(g() % m), (uint64_t)(g() % m)})
+            for (int E : {4, 5, 32, 64}) bad += differs(m, lam, x, E), ++n;
+    }
+    printf("16-bit moduli: %ld of %ld differ\n", bad, n);
+    bad += all;
     printf("%s\n", bad ? "FAILED" : "ok");
     return bad != 0;
 }

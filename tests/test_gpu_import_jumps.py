@@ -59,3 +59,36 @@ def test_bbs_moduli_equal_the_oracle(kind, L, segments):
         assert np.array_equal(u32v[4 * P:5 * P], lanes["x"])
         assert np.array_equal(u32v[5 * P:6 * P], lanes["tprev"])
         st.free()
+
+
+MODULI16 = [585, 8, 24, 3, 15, 255, 19683, 6561, 65535, 65534, 32768, 4, 65521, 257, 289, 143 * 143, 46341, 51 * 257]
+
+
+@pytest.mark.parametrize("L,segments", [(100, 0), (128, 0), (300, 0), (1500, 0), (100, 2), (1024, 5)])
+def test_bbs16_moduli_equal_the_oracle(L, segments):
+    """Prime powers, even moduli, one prime, more than two; units and not."""
+    torch, ci = cuda_or_skip()
+    st = ci.States(S, variant="bbs16", comb_size=C, seed=SEED)
+    buf = st.export_state().copy()
+    f = buf[512:].view(np.uint32).reshape(25, P)
+    lanes = oracle.init_lanes(oracle.VAR_BBS16, oracle.XL_XOR128, SEED, 0, P)
+    for l in range(32, 64):
+        for g in range(8):
+            M = MODULI16[(3 * l + g) % len(MODULI16)]
+            y = [0, 2 % M, 3 % M, M - 1, 51 % M, (12345 * l + g) % M][(l + g) % 6]
+            f[9 + g, l], f[17 + g, l] = y, M
+            lanes[l]["y16"][g], lanes[l]["m16"][g] = y, M
+    ref, _ = oracle.run(oracle.VAR_BBS16, oracle.XL_XOR128, C, oracle.comb_arrays(oracle.VAR_BBS16, C, 0), lanes, L)
+    for sink in ("written", "digest"):
+        st.import_state(buf)
+        if segments:
+            got = st.generate_split(L, sink=sink, segments=segments)
+        else:
+            got = st.generate(L) if sink == "written" else st.generate_digest(L)
+        if sink == "written":
+            assert np.array_equal(u32(got), ref[:S])
+        else:
+            assert np.array_equal(got.cpu().numpy().view(np.uint64), digest_rows(ref[:S]))
+        f2 = st.export_state()[512:].view(np.uint32).reshape(25, P)
+        assert np.array_equal(f2[9:17].T, lanes["y16"]) and np.array_equal(f2[17:25].T, lanes["m16"])
+        assert np.array_equal(f2[4], lanes["x"]) and np.array_equal(f2[5], lanes["tprev"])
