@@ -458,6 +458,11 @@ __device__ __forceinline__ uint2 mat_vec2(uint32_t m_row, uint32_t n_row, uint32
     return r;
 }
 
+// Row of P for a lane with partners p1 and p2.  The bytes of an imported partner
+// table are lane numbers modulo 32, as the shuffles of the generation loop take
+// them.
+__device__ __forceinline__ uint32_t partner_row(int p1, int p2) { return (1u << (p1 & 31)) ^ (1u << (p2 & 31)); }
+
 // Q = P^len and S = P + ... + P^len, len >= 1, by the bits of len from the
 // top: (Q, S) for k -> 2k: S <- S ^ S Q, Q <- Q Q; k -> k + 1: Q <- Q P,
 // S <- S ^ Q (all are polynomials in P, so they commute).
@@ -512,7 +517,7 @@ __global__ void __cluster_dims__(kCarryBlocks, 1, 1) __launch_bounds__(32 * kCar
     src.load(s0, l);
     int a1, a2;
     src.arrays(s0, l, a1, a2);
-    const uint32_t prow = (1u << s0.table[a1 * 32 + lane]) ^ (1u << s0.table[a2 * 32 + lane]);
+    const uint32_t prow = partner_row(s0.table[a1 * 32 + lane], s0.table[a2 * 32 + lane]);
     uint32_t Q, S;
     power_sums(prow, len, Q, S, sc);
     const uint32_t m = (K - 1 + NW - 1) / NW;
@@ -866,7 +871,7 @@ __global__ void __launch_bounds__(32 * kNarrowWarps)
     const uint2 e = make_uint2(s.slot, s.x);
     ends[bw][lane] = e;
     uint32_t Q, S;
-    power_sums((1u << s.p1) ^ (1u << s.p2), len, Q, S, sc);
+    power_sums(partner_row(s.p1, s.p2), len, Q, S, sc);
     __syncthreads();
     // H(c) ^ e for c = (slot, x)
     auto advance = [&](uint32_t q, uint32_t t, uint2 c, uint2 add) {

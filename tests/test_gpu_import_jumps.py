@@ -92,3 +92,20 @@ def test_bbs16_moduli_equal_the_oracle(L, segments):
         f2 = st.export_state()[512:].view(np.uint32).reshape(25, P)
         assert np.array_equal(f2[9:17].T, lanes["y16"]) and np.array_equal(f2[17:25].T, lanes["m16"])
         assert np.array_equal(f2[4], lanes["x"]) and np.array_equal(f2[5], lanes["tprev"])
+
+
+@pytest.mark.parametrize("variant", ["xor", "bbs", "bbs16"])
+def test_partner_tables_count_modulo_the_warp(variant):
+    """An imported table whose bytes name the same lanes above 31: the plain
+    loop's shuffles take them modulo 32, and so do calls in segments."""
+    torch, ci = cuda_or_skip()
+    st = ci.States(S, variant=variant, comb_size=C, seed=SEED)
+    good = st.export_state().copy()
+    high = good.copy()
+    high[:512] += (np.arange(512) % 8 * 32).astype(np.uint8)
+    for L, segments in ((100, 1), (600, 0), (3000, 0), (20000, 0), (300, 3)):
+        out = []
+        for buf in (good, high):
+            st.import_state(buf)
+            out.append(u32(st.generate_split(L, segments=segments) if segments else st.generate(L)))
+        assert np.array_equal(out[0], out[1]), (L, segments)
