@@ -1168,8 +1168,12 @@ cudaError_t split_prepare(cudaStream_t stream) { return ensure_jump_tables(strea
 
 namespace {
 
-bool jump_tables_ready() {
+// Whether a call of h may jump without building tables first.  Building them
+// waits for the stream once, which a capture forbids: a captured call without
+// them runs whole, in one launch, with the same results.
+bool jumps_at_hand(const ci_states_s &h) {
     int dev = 0;
+    if (h.variant != CI_VAR_XOR) return true;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
     std::lock_guard<std::mutex> lk(g_tables_mu);
     return dev < (int)g_tables_ready.size() && g_tables_ready[dev];
@@ -1306,12 +1310,12 @@ uint64_t split_auto(const ci_states_s &h, uint64_t n, int sink, bool captured) {
 ci_status single_call(const ci_states_s &h, uint64_t n, int sink, uint32_t *out, uint64_t *aux, cudaStream_t stream) {
     const bool captured = stream_capturing(stream);
     cudaError_t e;
-    // building the jump tables waits for the stream once, which a capture forbids
     const int blocks = narrow_blocks(h, n);
-    if (blocks && (!captured || jump_tables_ready())) {
+    const bool whole = captured && !jumps_at_hand(h);
+    if (blocks && !whole) {
         e = launch_narrow(h, blocks, n, sink, out, aux, stream);
     } else {
-        const uint64_t K = split_auto(h, n, sink, captured);
+        const uint64_t K = whole ? 1 : split_auto(h, n, sink, captured);
         if (K > 1) return split_launch(h, n, sink, out, n, 0, aux, K, stream);
         e = sink == CI_SINK_QC       ? launch_fused_qc(h, n, aux, stream)
             : sink == CI_SINK_DIGEST ? launch_digest(h, n, aux, stream)
@@ -1512,8 +1516,8 @@ extern "C" ci_status ci_generate_split(ci_states h, uint64_t n, int32_t sink, vo
     if (sink == CI_SINK_WRITTEN && (n > ~0ull / h->S || out_capacity < h->S * n))
         return fail(CI_E_INVAL, "out_capacity is smaller than n_streams * n");
     if (sink == CI_SINK_QC && (n & 1ull)) return fail(CI_E_INVAL, "quarter-circle sink needs an even length");
-    const uint64_t K = split_segments(*h, n, n_segments);
     const cudaStream_t cs = static_cast<cudaStream_t>(cuda_stream);
+    const uint64_t K = stream_capturing(cs) && !jumps_at_hand(*h) ? 1 : split_segments(*h, n, n_segments);
     if (K <= 1) {  // unsplit: one launch of the tuned single-call kernel
         const cudaError_t e = sink == CI_SINK_QC       ? launch_fused_qc(*h, n, static_cast<uint64_t *>(out_dev), cs)
                               : sink == CI_SINK_DIGEST ? launch_digest(*h, n, static_cast<uint64_t *>(out_dev), cs)
