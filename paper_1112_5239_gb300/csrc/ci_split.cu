@@ -191,23 +191,62 @@ cudaError_t build_jump_tables(const void *columns_symbol, const void *jump_symbo
     return cudaGetLastError();
 }
 
+// The tables of one device: built by the first call that jumps, on its stream,
+// with `done` recorded behind them.  Calls on other streams wait for the event
+// on the device until it has been seen finished; the host never waits.
+struct JumpTables {
+    cudaEvent_t done = nullptr;
+    bool ready = false;
+};
 std::mutex g_tables_mu;
-std::vector<int> g_tables_ready;  // per device ordinal
+std::vector<JumpTables> g_tables;  // per device ordinal
 
-cudaError_t ensure_jump_tables(cudaStream_t stream) {
+// Lets this thread build and query on `stream` while it captures another one
+// (a capture in the global mode refuses such calls otherwise).
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// The current device's entry, with g_tables_mu held; null without a device.
+JumpTables *device_tables() {
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return nullptr;
+    if ((int)g_tables.size() <= dev) g_tables.resize(dev + 1);
+    return &g_tables[dev];
+}
+
+// Whether the tables are finished, with g_tables_mu held.
+bool tables_ready(JumpTables &t) {
+    if (t.ready || !t.done) return t.ready;
+    RelaxedCapture relaxed;
+    t.ready = cudaEventQuery(t.done) == cudaSuccess;
+    if (!t.ready) cudaGetLastError();  // "not ready" is no error of the call
+    return t.ready;
+}
+
+// Work put on `stream` after this finds finished tables.  Not for a capturing
+// stream, unless they are ready.
+cudaError_t ensure_jump_tables(cudaStream_t stream) {
     std::lock_guard<std::mutex> lk(g_tables_mu);
-    if ((int)g_tables_ready.size() <= dev) g_tables_ready.resize(dev + 1, 0);
-    if (g_tables_ready[dev]) return cudaSuccess;
-    if ((e = build_jump_tables<4>(g_columns_xor128, g_jump_xor128, stream)) != cudaSuccess) return e;
-    if ((e = build_jump_tables<2>(g_columns_xor64, g_jump_xor64, stream)) != cudaSuccess) return e;
-    if ((e = build_jump_tables<1>(g_columns_xs32, g_jump_xs32, stream)) != cudaSuccess) return e;
-    // Wait once, so that calls on any stream of this device find finished tables.
-    if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return e;
-    g_tables_ready[dev] = 1;
-    return cudaSuccess;
+    JumpTables *t = device_tables();
+    if (!t) return cudaErrorInvalidDevice;
+    if (tables_ready(*t)) return cudaSuccess;
+    if (t->done) return cudaStreamWaitEvent(stream, t->done, 0);
+    RelaxedCapture relaxed;
+    cudaEvent_t done;
+    cudaError_t e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
+    if (e != cudaSuccess) return e;
+    e = build_jump_tables<4>(g_columns_xor128, g_jump_xor128, stream);
+    if (e == cudaSuccess) e = build_jump_tables<2>(g_columns_xor64, g_jump_xor64, stream);
+    if (e == cudaSuccess) e = build_jump_tables<1>(g_columns_xs32, g_jump_xs32, stream);
+    if (e == cudaSuccess) e = cudaEventRecord(done, stream);
+    if (e == cudaSuccess)
+        t->done = done;
+    else
+        cudaEventDestroy(done);
+    return e;
 }
 
 // ------------------------------------------------ BBS jump
@@ -1168,15 +1207,14 @@ cudaError_t split_prepare(cudaStream_t stream) { return ensure_jump_tables(strea
 
 namespace {
 
-// Whether a call of h may jump without building tables first.  Building them
-// waits for the stream once, which a capture forbids: a captured call without
-// them runs whole, in one launch, with the same results.
+// Whether a captured call of h may jump.  A graph can neither build the tables
+// nor wait for a build outside it: before they are finished such a call runs
+// whole, in one launch, with the same results.
 bool jumps_at_hand(const ci_states_s &h) {
-    int dev = 0;
     if (h.variant != CI_VAR_XOR) return true;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
     std::lock_guard<std::mutex> lk(g_tables_mu);
-    return dev < (int)g_tables_ready.size() && g_tables_ready[dev];
+    JumpTables *t = device_tables();
+    return t && tables_ready(*t);
 }
 
 // Blocks per cluster of the one-launch form for a call of n iterations; 0: it

@@ -31,7 +31,7 @@ ci_status single_call(const ci_states_s &h, uint64_t n, int sink, uint32_t *out,
 ci_status split_launch(const ci_states_s &h, uint64_t n, int sink, uint32_t *out, uint64_t ld, uint64_t col0,
                        uint64_t *aux, uint64_t K, cudaStream_t stream);
 
-// Builds the jump tables for the current device (blocks once on `stream`).
+// Puts the building of the current device's jump tables on `stream`, if no call has.
 cudaError_t split_prepare(cudaStream_t stream);
 
 }  // namespace ci
