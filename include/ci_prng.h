@@ -212,7 +212,8 @@ ci_status ci_generate_bbs(ci_states states, uint64_t n_per_stream, uint32_t *out
  * stream-ordered scratch and are counted from there), otherwise under about
  * two waves of resident warps.  Stream-ordered workspaces come from a memory
  * pool of the library's own, which keeps up to 256 MiB between calls and gives
- * it back when the last state is freed. */
+ * it back when the last state is freed (what calls still running hold: at the
+ * next synchronisation after them). */
 ci_status ci_generate_fused_qc(ci_states states, uint64_t n_per_stream, uint64_t *counts_dev,
                                void *cuda_stream);
 

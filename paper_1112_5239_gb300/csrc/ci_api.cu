@@ -133,14 +133,22 @@ cudaMemPool_t workspace_pool() {
     return g_pools[dev];
 }
 
+// What the pools keep between calls: kWorkspaceKept while handles live.
+void pools_keep(uint64_t bytes) {
+    for (cudaMemPool_t p : g_pools)
+        if (p) cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &bytes);
+}
 void handle_made() {
     std::lock_guard<std::mutex> lock(g_pool_mu);
-    ++g_live_handles;
+    if (++g_live_handles == 1) pools_keep(kWorkspaceKept);
 }
-// Trimming releases unused memory only: workspaces of calls still running stay.
+// The last handle gone, unused memory is released at once, and what calls still
+// running hold (a state in the caller's memory may be freed before its last
+// call ends) at the synchronisation that follows them.  Neither waits.
 void handle_gone() {
     std::lock_guard<std::mutex> lock(g_pool_mu);
     if (--g_live_handles) return;
+    pools_keep(0);
     for (cudaMemPool_t p : g_pools)
         if (p) cudaMemPoolTrimTo(p, 0);
 }

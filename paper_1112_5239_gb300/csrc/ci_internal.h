@@ -107,8 +107,8 @@ int sm_count();
 // the current device (cudaFreeAsync gives them back).  The pool keeps up to
 // kWorkspaceKept bytes between calls: the default pool gives its memory back
 // to the system at every synchronisation, and a call after one then spent
-// 200 us on getting it again.  All of it is released when the last handle is
-// freed.
+// 200 us on getting it again.  When the last handle is freed the unused part is
+// released at once, what running calls hold at the next synchronisation.
 constexpr uint64_t kWorkspaceKept = 256ull << 20;
 cudaError_t workspace_alloc(void **p, size_t bytes, cudaStream_t stream);
 
