@@ -24,8 +24,6 @@
 // the 62-bit form).
 #include <cuda_runtime.h>
 
-#include <algorithm>
-#include <mutex>
 
 #include "ci_crt.cuh"
 #include "ci_device.cuh"
@@ -205,7 +203,7 @@ __global__ void __launch_bounds__(kBgWarps * 32, kBgMinBlocks)
     const uint32_t lane = threadIdx.x & 31u;
     uint8_t *tile = stage[threadIdx.x >> 5];
     uint8_t *row = tile + lane * kBgRowPad;
-    const uint64_t g = warp_group<kBgWarps>(in_order);  // at most one group a warp (gen_grid)
+    const uint64_t g = warp_group(in_order);  // at most one group a warp (gen_grid)
     if (g < (n_msgs + 31) / 32) {
         const uint64_t m0 = g * 32;
         const uint64_t msg = m0 + lane;
@@ -265,17 +263,6 @@ __global__ void __launch_bounds__(kBgWarps * 32, kBgMinBlocks)
     }
 }
 
-template <bool kDecrypt, bool kVec>
-GenGrid bg_grid(uint64_t n_msgs) {
-    static int per_sm = 0;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bg<kDecrypt, kVec>, kBgWarps * 32, 0);
-        if (per_sm <= 0) per_sm = 1;
-    });
-    return gen_grid((n_msgs + 31) / 32, kBgWarps, (uint64_t)sm_count() * per_sm);
-}
-
 ci_status bg_check(uint64_t n_msgs, uint64_t n_chunks, const void *a, const void *b, const void *S0,
                    const void *y, const void *in, const void *out) {
     if (!a || !b || !S0 || !y) return fail(CI_E_INVAL, "bg: key, S0 and y arrays must be non-null");
@@ -295,9 +282,11 @@ cudaError_t bg_launch(uint64_t n_msgs, uint64_t L, const uint64_t *a, const uint
                       const uint64_t *y_in, const uint8_t *in, uint8_t *out, uint64_t *y_out, uint32_t *n_rejected,
                       cudaStream_t stream) {
     const bool vec = bg_vec(L, in, out);
-    const GenGrid gg = vec ? bg_grid<kDecrypt, true>(n_msgs) : bg_grid<kDecrypt, false>(n_msgs);
     auto kern = vec ? k_bg<kDecrypt, true> : k_bg<kDecrypt, false>;
-    kern<<<gg.grid, kBgWarps * 32, 0, stream>>>(n_msgs, L, a, b, S0, y_in, in, out, y_out, n_rejected, gg.in_order);
+    static const int per_sm[2] = {resident_blocks_per_sm(k_bg<kDecrypt, false>, kBgWarps * 32, 0),
+                                  resident_blocks_per_sm(k_bg<kDecrypt, true>, kBgWarps * 32, 0)};
+    const GenGrid gg = gen_grid((n_msgs + 31) / 32, kBgWarps, (uint64_t)sm_count() * per_sm[vec], true);
+    kern<<<gg.grid, gg.warps * 32, 0, stream>>>(n_msgs, L, a, b, S0, y_in, in, out, y_out, n_rejected, gg.in_order);
     return cudaGetLastError();
 }
 

@@ -13,29 +13,45 @@
 
 namespace ci {
 
-// One warp per group of 32 lanes, W warps per block.  A state of more groups
-// than resident warps gets one block per W consecutive groups, handed to the
-// SMs in order as they fall free: the SMs do not run at the same speed (two
+// One warp per group of 32 lanes.  Blocks of consecutive groups are handed to
+// the SMs in order as they fall free: the SMs do not run at the same speed (two
 // dies, one memory each), so a fixed share per SM ends with the slowest, and
 // stores in address order reach 7.6 TB/s where the same stores from a
 // persistent grid reached 6.5 (1 GiB, nothing else in the kernel).  Measured
 // against a persistent grid when it was brought in: 2^20 x 1024 consumed 610
-// instead of 690 us, 2^20 x 256 written 175 instead of 199 us.  A state of fewer groups runs in one
-// wave: one block per group as far as blocks are resident, and warp w of block
-// b takes group w * gridDim.x + b, so that every SM gets its share of the warps.
-// Either way a warp has at most one group.
+// instead of 690 us, 2^20 x 256 written 175 instead of 199 us.  W warps per
+// block; a state of one wave takes smaller blocks as far as the SMs' 32 blocks
+// each hold it, since idle warps of larger ones leave schedulers unused (2^17 x
+// 1024 digested: 82 us, 92 with one or two of a block's four warps at work;
+// 50001 x 1001 XORshift 53, 57).
+// The squaring sources (kHeavy) nearly fill a scheduler with each warp: one-warp
+// blocks up to two warps per scheduler (10^4 x 1024 of Algorithm 5 as printed:
+// 94 us, 139 spread), beyond them a wave is spread over all resident blocks so
+// that every SM gets its share (2^16 x 1024: 261 us, 270 in one-warp blocks).
 struct GenGrid {
-    unsigned grid;
-    uint32_t in_order;
+    unsigned grid, warps;  // blocks; warps per block
+    uint32_t in_order;     // the same if blocks hold consecutive groups, else 0: warp w of block b takes w * grid + b
 };
-inline GenGrid gen_grid(uint64_t groups, int W, uint64_t resident_blocks) {
-    if (groups > resident_blocks * W) return {(unsigned)((groups + W - 1) / W), 1u};
-    return {(unsigned)(groups < resident_blocks ? groups : resident_blocks), 0u};
+inline GenGrid gen_grid(uint64_t groups, int W, uint64_t resident_blocks, bool heavy) {
+    const uint64_t sms = (uint64_t)sm_count();
+    unsigned warps = (unsigned)W;
+    if (groups <= resident_blocks * W) {
+        if (heavy && groups > 8 * sms)
+            return {(unsigned)(groups < resident_blocks ? groups : resident_blocks), warps, 0u};
+        const uint64_t w = (groups + 32 * sms - 1) / (32 * sms);
+        if (w < (uint64_t)W) warps = (unsigned)w;
+    }
+    return {(unsigned)((groups + warps - 1) / warps), warps, warps};
 }
-template <int W>
 __device__ __forceinline__ uint64_t warp_group(uint32_t in_order) {
     const uint64_t w = threadIdx.x >> 5;
-    return in_order ? (uint64_t)blockIdx.x * W + w : w * gridDim.x + blockIdx.x;
+    return in_order ? (uint64_t)blockIdx.x * in_order + w : w * gridDim.x + blockIdx.x;
+}
+template <class Kernel>
+int resident_blocks_per_sm(Kernel kern, int threads, size_t smem) {
+    int n = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem) != cudaSuccess || n <= 0) n = 1;
+    return n;
 }
 
 // Written sinks stage a 32 x KT tile per warp in dynamic shared memory.
@@ -47,7 +63,7 @@ __global__ void __launch_bounds__(W * 32) k_generate(DevState st, uint64_t n, ui
     extern __shared__ uint4 dyn_tiles[];
     const int w = threadIdx.x >> 5;
     uint4 *tile = dyn_tiles + w * kTileVecs<SINK, TC>;
-    const uint64_t g = warp_group<W>(in_order);
+    const uint64_t g = warp_group(in_order);
     if (g < st.P / 32) dev::warp_task<Src, SINK, TC>(st, g, n, out, n, 0, counts, tile);
 }
 
@@ -62,7 +78,7 @@ __global__ void __launch_bounds__(W * 32) k_generate_tma(DevState st, uint64_t n
     uint4 *base = reinterpret_cast<uint4 *>(reinterpret_cast<char *>(tma_tiles) + ((1024u - (sbase & 1023u)) & 1023u));
     const int w = threadIdx.x >> 5;
     uint4 *tiles = base + w * 256 * dev::kTmaTiles;
-    const uint64_t g = warp_group<W>(in_order);
+    const uint64_t g = warp_group(in_order);
     if (g < st.P / 32) dev::warp_task_tma<Src>(st, g, n, &map, tiles);
 }
 
@@ -118,19 +134,14 @@ static cudaError_t launch_gen_tma(const DevState &st, uint64_t n, uint32_t *out,
     CUtensorMap map;
     if (!make_out_tensor_map(&map, out, st.S, n)) return cudaSuccess;
     auto kern = k_generate_tma<Src, W>;
-    const size_t smem = (size_t)W * dev::kTmaTiles * 4096 + 1024;  // + slack for the 1024-byte alignment of the base
+    // + slack for the 1024-byte alignment of the base
+    auto smem = [](unsigned warps) { return (size_t)warps * dev::kTmaTiles * 4096 + 1024; };
     static std::atomic<uint64_t> smem_set{0};
-    allow_smem(kern, smem, smem_set);
-    static std::once_flag once;
-    static int per_sm = 1;
-    std::call_once(once, [&] {
-        int ps = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kern, W * 32, smem) == cudaSuccess && ps > 0)
-            per_sm = ps;
-    });
-    const GenGrid gg = gen_grid(st.P / 32, W, (uint64_t)sm_count() * per_sm);
+    allow_smem(kern, smem(W), smem_set);
+    static const int per_sm = resident_blocks_per_sm(kern, W * 32, smem(W));
+    const GenGrid gg = gen_grid(st.P / 32, W, (uint64_t)sm_count() * per_sm, false);
     *used = true;
-    kern<<<gg.grid, W * 32, smem, stream>>>(st, n, gg.in_order, map);
+    kern<<<gg.grid, gg.warps * 32, smem(gg.warps), stream>>>(st, n, gg.in_order, map);
     return cudaGetLastError();
 }
 
@@ -138,18 +149,12 @@ template <class Src, int SINK, int W, class TC>
 static cudaError_t launch_gen_t(const DevState &st, uint64_t n, uint32_t *out, uint64_t *counts,
                                 cudaStream_t stream) {
     auto kern = k_generate<Src, SINK, W, TC>;
-    const size_t smem = (size_t)W * kTileVecs<SINK, TC> * sizeof(uint4);
+    constexpr size_t tile = kTileVecs<SINK, TC> * sizeof(uint4);
     static std::atomic<uint64_t> smem_set{0};
-    allow_smem(kern, smem, smem_set);
-    static std::once_flag once;
-    static int per_sm = 1;
-    std::call_once(once, [&] {
-        int ps = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kern, W * 32, smem) == cudaSuccess && ps > 0)
-            per_sm = ps;
-    });
-    const GenGrid gg = gen_grid(st.P / 32, W, (uint64_t)sm_count() * per_sm);
-    kern<<<gg.grid, W * 32, smem, stream>>>(st, n, gg.in_order, out, counts);
+    allow_smem(kern, W * tile, smem_set);
+    static const int per_sm = resident_blocks_per_sm(kern, W * 32, W * tile);
+    const GenGrid gg = gen_grid(st.P / 32, W, (uint64_t)sm_count() * per_sm, Src::kHeavy);
+    kern<<<gg.grid, gg.warps * 32, gg.warps * tile, stream>>>(st, n, gg.in_order, out, counts);
     return cudaGetLastError();
 }
 

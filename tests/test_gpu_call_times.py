@@ -1,0 +1,40 @@
+"""Times that two forms of one call must not be apart by: ratios of device times
+on the same GPU, minimum of several runs, with wide margins."""
+import pytest
+
+from gpu_util import cuda_or_skip
+
+pytestmark = pytest.mark.gpu
+
+
+def _us(torch, call, reps=20, runs=7):
+    for _ in range(3):
+        call()
+    best = float("inf")
+    for _ in range(runs):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        for _ in range(reps):
+            call()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) * 1e3 / reps)
+    return best
+
+
+def _written(torch, ci, S, n, offset=0, segments=None, **kw):
+    st = ci.States(S, seed=1, **kw)
+    out = torch.empty(S * n + offset, dtype=torch.int32, device="cuda")[offset:].view(S, n)
+    if segments is None:
+        return _us(torch, lambda: st.generate(n, out=out))
+    return _us(torch, lambda: st.generate_split(n, out=out, segments=segments))
+
+
+def test_a_warp_per_scheduler_costs_as_much_as_a_warp_per_sm():
+    """Algorithm 5 as printed, three and one warp groups per SM: no scheduler has two of
+    them while another has none."""
+    torch, ci = cuda_or_skip()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    one = _written(torch, ci, 32 * sms, 1024, segments=1, variant="bbs16")
+    two = _written(torch, ci, 32 * 3 * sms, 1024, segments=1, variant="bbs16")
+    assert two < 1.25 * one, (one, two)
