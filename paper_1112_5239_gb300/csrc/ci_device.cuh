@@ -588,6 +588,36 @@ __device__ __forceinline__ void store_words(uint32_t *p, const uint4 &v, int lo,
     }
 }
 
+// Rows of up to 64 words with nothing between them (ld == n): the group's rows
+// are one span of the output, staged at a pitch of 65 words (32 banks a step)
+// and stored as that span, 32 consecutive words per warp-wide store.
+constexpr uint64_t kShortRows = 64;
+constexpr int kShortPitch = 65;
+template <class Step>
+__device__ __forceinline__ void written_short(Step step, uint64_t S, uint64_t row0, uint32_t n, uint32_t *out,
+                                              uint4 *tile) {
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t *stage = reinterpret_cast<uint32_t *>(tile);
+#pragma unroll 1
+    for (uint32_t i = 0; i < n; ++i) stage[lane * kShortPitch + i] = step();
+    __syncwarp();
+    const uint32_t rows = S - row0 < 32 ? (uint32_t)(S - row0) : 32u, words = rows * n;
+    const uint32_t dr = 32 / n, dc = 32 % n;
+    uint32_t *dst = out + row0 * n;
+    uint32_t r = lane / n, c = lane % n;
+#pragma unroll 4
+    for (uint32_t i = lane; i < words; i += 32) {
+        dst[i] = stage[r * kShortPitch + c];
+        r += dr;
+        c += dc;
+        if (c >= n) {
+            c -= n;
+            ++r;
+        }
+    }
+    __syncwarp();
+}
+
 // Written rows of any alignment (out 4-byte aligned, any ld, col0 and n).  Row
 // r starts ph_r = 0..31 words after a 128-byte line; its staging row starts at
 // that line, so that everything but a row's first and last words leaves as
@@ -595,24 +625,34 @@ __device__ __forceinline__ void store_words(uint32_t *p, const uint4 &v, int lo,
 // written in two parts 32 steps apart costs its memory write twice: 400 MB in
 // rows of 401 took 132 us by 16-byte, 108 by 32-byte boundaries.)  Output j of
 // the call stands at word (j + ph_r) mod 64 of the row's two lines, of which one
-// is stored after every 32 steps.  The lanes of one step write 32 different
-// banks when ld is odd.  `step` makes the lane's next output; kUnroll of a
-// tile's 32 steps are unrolled.
+// is stored after every 32 steps.  `step` makes the lane's next output; kUnroll
+// of a tile's 32 steps are unrolled.
 // (50001 x 1001 XORshift outputs: the word-wise form this replaces, a row per
 // warp-wide store, issued 34 instructions per step of a warp, 20 of them for
-// the stores, and took 82 us; now 57.)
-constexpr int kTileVec = 32 * 16;  // 16-byte words of a warp's staging tile (the aligned 32 x 32 form: 256)
-template <int kUnroll, int CACHE, class Step>
-__device__ __forceinline__ void written_unaligned(Step step, uint64_t S, uint64_t row0, uint64_t n, uint32_t *out,
-                                                  uint64_t ld, uint64_t col0, uint4 *tile) {
+// the stores, and took 82 us; now 53.)
+// Banks: the lanes of one step write 32 different ones when ld is odd, 16 when
+// it is 2 mod 4.  When ld is a multiple of 4 (in a buffer that is not 16-byte
+// aligned) the rows' phases are equal mod 4: after up to three steps every row
+// stands at a 16-byte word and four steps make one store of it, without
+// conflicts at a pitch of 16 or 17 such words (ld / 4 odd or even).  Word by
+// word, 2^18 x 256 from the second word of a buffer on took 269 us, and the
+// older form 135.
+// kPitch: 16-byte words between staging rows, 0 for 16 or 17 by ld; kQuads: ld
+// is a multiple of 4.
+constexpr int kTileVec = 32 * 17;  // 16-byte words of a warp's staging tile (the aligned 32 x 32 form: 256)
+template <int kUnroll, int CACHE, int kPitch, bool kQuads, class Step>
+__device__ __forceinline__ void written_lines(Step step, uint64_t S, uint64_t row0, uint64_t n, uint32_t *out,
+                                              uint64_t ld, uint64_t col0, uint4 *tile) {
     const int lane = threadIdx.x & 31;
     // words of row r before its first output, up to the line below it
     auto phase = [&](uint64_t r) { return (int)((reinterpret_cast<uintptr_t>(out + r * ld + col0) >> 2) & 31u); };
     const int ph = phase(row0 + lane);  // the row this lane computes
-    uint32_t *w = reinterpret_cast<uint32_t *>(tile + lane * 16) + ph;
+    const int pitch = kPitch ? kPitch : ld % 8 == 0 ? 17 : 16;
+    uint4 *mine = tile + lane * pitch;
+    uint32_t *w = reinterpret_cast<uint32_t *>(mine) + ph;
     // the rows this lane stores: 4 k + lane / 8, 16-byte word c of their lines
     const int c = lane & 7;
-    const uint4 *stored = tile + (lane >> 3) * 16 + c;
+    const uint4 *stored = tile + (lane >> 3) * pitch + c;
     const uint64_t row = row0 + (lane >> 3);
     const bool all_rows = row0 + 32 <= S;
     uint32_t *dst = out + row * ld + col0;  // output `at` of row `row`
@@ -627,20 +667,20 @@ __device__ __forceinline__ void written_unaligned(Step step, uint64_t S, uint64_
         const uint4 *from = stored + half / 4;
         if (at > 0 && at + 32 <= len && all_rows) {  // words of the rows only
 #pragma unroll(kUnroll > 1 ? 8 : 2)
-            for (int k = 0; k < 8; ++k, q += 4 * ld) {
+            for (int k = 0; k < 8; ++k, q += 4 * ld, from += 4 * pitch) {
                 uint32_t *line = reinterpret_cast<uint32_t *>(reinterpret_cast<uintptr_t>(q) & ~(uintptr_t)127);
-                store16<CACHE>(line + 4 * c, from[64 * k]);
+                store16<CACHE>(line + 4 * c, *from);
             }
         } else {
 #pragma unroll 1
-            for (int k = 0; k < 8; ++k, q += 4 * ld) {
+            for (int k = 0; k < 8; ++k, q += 4 * ld, from += 4 * pitch) {
                 const uintptr_t a = reinterpret_cast<uintptr_t>(q);
                 const int p = (int)((a >> 2) & 31u);
                 uint32_t *line = reinterpret_cast<uint32_t *>(a & ~(uintptr_t)127);
                 // words [lo, hi) of this 16-byte word belong to the row
                 const int64_t hi = len - at + p - 4 * c;
                 if (row + 4 * k < S)
-                    store_words<CACHE>(line + 4 * c, from[64 * k], at == 0 ? p - 4 * c : 0, hi > 4 ? 4 : (int)hi);
+                    store_words<CACHE>(line + 4 * c, *from, at == 0 ? p - 4 * c : 0, hi > 4 ? 4 : (int)hi);
             }
         }
         dst += 32;
@@ -650,25 +690,58 @@ __device__ __forceinline__ void written_unaligned(Step step, uint64_t S, uint64_
     };
     // word (ph + j + half) mod 64 of the lane's row, ph + j < 64
     auto place = [&](int j) { return j + ph < 32 ? w + half + j : w - half + j; };
-    while (at + 32 <= len) {
-        if (kUnroll < 32) {
-#pragma unroll(kUnroll)
-            for (int j = 0; j < 32; ++j) *place(j) = step();
-        } else if (half == 0) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) w[j] = step();
-        } else {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) *place(j) = step();
+    int head = 0;  // outputs up to the first 16-byte word, the same in every lane
+    if constexpr (kQuads) {
+        head = -ph & 3;
+        if (head > len) head = (int)len;
+        for (int j = 0; j < head; ++j) w[j] = step();
+        const int first = (ph + head) / 4;
+        while (at + head + 32 <= len) {
+#pragma unroll(kUnroll / 4)
+            for (int q = 0; q < 8; ++q) {
+                uint4 v;
+                v.x = step();
+                v.y = step();
+                v.z = step();
+                v.w = step();
+                mine[(first + half / 4 + q) & 15] = v;
+            }
+            flush();
         }
-        flush();
+    } else {
+        while (at + 32 <= len) {
+            if (kUnroll < 32) {
+#pragma unroll(kUnroll)
+                for (int j = 0; j < 32; ++j) *place(j) = step();
+            } else if (half == 0) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) w[j] = step();
+            } else {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) *place(j) = step();
+            }
+            flush();
+        }
     }
-    // the rest: up to 31 steps behind the words kept from the last tile, at
-    // most 62 words of a row
-    const int rem = (int)(n % 32);
-    for (int j = 0; j < rem; ++j) *place(j) = step();
-    if (__any_sync(kFull, rem + ph > 0)) flush();
-    if (__any_sync(kFull, rem + ph > 32)) flush();
+    // the rest: up to 31 steps behind the words kept from the last tile (and the
+    // head), at most 63 words of a row
+    const int rest = (int)(len - at);
+    for (int j = head; j < rest; ++j) *place(j) = step();
+    if (__any_sync(kFull, rest + ph > 0)) flush();
+    if (__any_sync(kFull, rest + ph > 32)) flush();
+}
+
+template <int kUnroll, int CACHE, class Step>
+__device__ __forceinline__ void written_unaligned(Step step, uint64_t S, uint64_t row0, uint64_t n, uint32_t *out,
+                                                  uint64_t ld, uint64_t col0, uint4 *tile) {
+    if (n <= kShortRows && ld == n)
+        written_short(step, S, row0, (uint32_t)n, out, tile);
+    else if constexpr (kUnroll == 1)  // a step takes far longer than its store
+        written_lines<kUnroll, CACHE, 0, false>(step, S, row0, n, out, ld, col0, tile);
+    else if (ld % 4 == 0)
+        written_lines<kUnroll, CACHE, 0, true>(step, S, row0, n, out, ld, col0, tile);
+    else
+        written_lines<kUnroll, CACHE, 16, false>(step, S, row0, n, out, ld, col0, tile);
 }
 
 // Runs n steps of a loaded lane into the sink; returns the lane's

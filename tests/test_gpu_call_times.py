@@ -38,3 +38,12 @@ def test_a_warp_per_scheduler_costs_as_much_as_a_warp_per_sm():
     one = _written(torch, ci, 32 * sms, 1024, segments=1, variant="bbs16")
     two = _written(torch, ci, 32 * 3 * sms, 1024, segments=1, variant="bbs16")
     assert two < 1.25 * one, (one, two)
+
+
+@pytest.mark.parametrize("S,n", [(1 << 17, 64), (1 << 17, 24), (1 << 15, 1024)])
+def test_rows_off_a_16_byte_boundary(S, n):
+    """Rows of a multiple of eight words from the second word of a buffer on,
+    against rows one word longer: no bank conflicts between the rows of a warp."""
+    torch, ci = cuda_or_skip()
+    even, odd = (_written(torch, ci, S, k, offset=1, segments=1) for k in (n, n + 1))
+    assert even < 1.5 * odd, (even, odd)
