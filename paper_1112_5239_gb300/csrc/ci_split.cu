@@ -1273,11 +1273,30 @@ uint64_t split_segments(const ci_states_s &h, uint64_t n, uint64_t requested) {
 
 namespace {
 
+// Whether a call of n iterations of a BBS state is faster whole than in
+// segments, by the times of both forms (ns).  Whole: a chain of 390 per output
+// up to a warp per scheduler, then by the warps of the fullest one.  In
+// segments: a fixed part and the squarings of all warp groups at the split
+// kernels' rate.  Whole / in segments, us, written: 32 x 128 55 / 59, x 256 105 /
+// 58; 10^4 x 256 105 / 125, x 512 203 / 154; 30000 x 512 266 / 363, x 2048 1041 /
+// 901; 2^16 x 512 463 / 499, x 2048 1829 / 1645; digests (written to scratch and
+// reduced) 30000 x 1024 511 / 575, 2^16 x 1024 919 / 991, 2^18 x 1024 2931 / 3499.
+bool whole_bbs(uint64_t groups, uint64_t n, bool written) {
+    const uint64_t sms = (uint64_t)sm_count();
+    const bool one_launch = groups >= kOneLaunchGroupsPerSm * sms;
+    const uint64_t w = 1 + 51 * groups / (200 * sms);  // the schedulers fill up 2 % before the count says so
+    const uint64_t chain = w == 1 ? 390 : 100 + 210 * w + (!written && !one_launch && w >= 3 ? 150 : 0);
+    const uint64_t rate = (written ? (one_launch ? 53 : 59) : (one_launch ? 62 : 71)) * groups / sms;
+    const uint64_t fixed = (one_launch ? 180000 : 62000 + 110 * groups) + (written ? 0 : 10000);
+    return chain <= rate || n * (chain - rate) < fixed;
+}
+
 // Segment count a single call uses for a CI_VAR_BBS state.  Written sink, and
 // consumer sinks whose outputs fit the scratch (they are written, fixed up and
-// reduced): from the GPU size and the form split_launch takes; larger consumer
+// reduced): whole by the rule above, else from the GPU size and the form
+// split_launch takes; larger consumer
 // calls, which generate twice: > 1 only for states that fill less than about
-// two waves of resident warps.  `captured`: calls too short for segments of
+// two waves.  `captured`: calls too short for segments of
 // kMinSegment stay one plain launch (a split allocates its workspace, which a
 // graph then has to own).
 uint64_t split_auto_bbs(const ci_states_s &h, uint64_t n, int sink, bool captured) {
@@ -1287,6 +1306,7 @@ uint64_t split_auto_bbs(const ci_states_s &h, uint64_t n, int sink, bool capture
     // consumer sinks whose outputs fit the scratch are written, fixed up and
     // reduced (split_launch), so they take the written rule
     if (sink == CI_SINK_WRITTEN || h.S <= kScratchWords / n) {
+        if (whole_bbs(groups, n, sink == CI_SINK_WRITTEN)) return 1;
         // Measured on 2^9 .. 2^13 warp groups of 2^12 .. 2^15 iterations:
         // about ten waves of resident warps (40 per SM) in the one-launch
         // form, four in the three-launch form; segments of at least 256.
@@ -1320,8 +1340,11 @@ uint64_t split_auto(const ci_states_s &h, uint64_t n, int sink, bool captured) {
         // warps (measured, written: 1 group 39x, 32 groups 7x, 128 groups
         // 2.8x faster; 512 groups slower), with about two waves of the split
         // kernels' 16 resident warps per SM and segments of at least 256, or
-        // 64 while they fill less than one wave.
-        if (groups > sms) return 1;
+        // 64 while they fill less than one wave.  Shorter calls run whole, at
+        // 87 ns an output (whole / in segments, us: 32 x 512 49 / 77, x 1024 90 /
+        // 80; 1000 x 1024 90 / 94, x 1500 131 / 111; 4864 x 1500 131 / 160, x 2048
+        // 176 / 169).
+        if (groups > sms || n < 880 + 1140 * groups / sms) return 1;
         uint64_t K = std::min<uint64_t>(sms * 32 / groups, n / kMinSegment);
         if (!captured) K = std::max<uint64_t>(K, std::min<uint64_t>(sms * 16 / groups, n / kMinShortSegment));
         K = std::min<uint64_t>(K, kMaxSegments);

@@ -47,3 +47,12 @@ def test_rows_off_a_16_byte_boundary(S, n):
     torch, ci = cuda_or_skip()
     even, odd = (_written(torch, ci, S, k, offset=1, segments=1) for k in (n, n + 1))
     assert even < 1.5 * odd, (even, odd)
+
+
+@pytest.mark.parametrize("variant,S,n", [("bbs16", 64, 130), ("bbs16", 64, 500), ("bbs16", 4800, 512),
+                                         ("bbs", 30000, 130), ("bbs", 20000, 200), ("bbs", 10000, 130)])
+def test_a_call_is_not_slower_than_whole(variant, S, n):
+    """Calls that choose segments themselves, against one segment."""
+    torch, ci = cuda_or_skip()
+    chosen, whole = (_written(torch, ci, S, n, segments=k, variant=variant) for k in (None, 1))
+    assert chosen < 1.25 * whole, (chosen, whole)
