@@ -475,6 +475,17 @@ enum Sink { SINK_V4 = 0, SINK_SCALAR = 1, SINK_QC = 2, SINK_DIGEST = 3, SINK_NON
 // Multiplier of the per-stream output digest D <- D * K + x (mod 2^64),
 // an odd 64-bit constant.
 constexpr uint64_t kDigestMul = 0xD1342543DE82EF95ull;
+// Its powers, for compile-time exponents.
+__host__ __device__ constexpr uint64_t digest_power(int e) {
+    uint64_t p = 1;
+    for (int i = 0; i < e; ++i) p *= kDigestMul;
+    return p;
+}
+// xor128's outputs join the digest sixteen at a time, each times its own power:
+// in Horner's form a warp alone waited for the product of every step (16000 x
+// 2000: 57 us, 45 so; 2^20 x 1024: 550, 531).  The other xor-likes are faster
+// by Horner (xor64 16000 x 2000: 43 us, 58 in blocks).
+constexpr int kDigestBlock = 16;
 
 // One lane's stream while a warp advances its group: the strategy source, the
 // CI state x, the slot (last strategy) and the two partner lanes.  step() is
@@ -767,8 +778,16 @@ __device__ __forceinline__ uint64_t warp_run(Lane<Src> &s, uint64_t S, uint64_t 
 #pragma unroll(Src::kHeavy ? 1 : 32)
             for (int k = 0; k < 32; ++k) s.step();
         } else if (SINK == SINK_DIGEST) {
+            constexpr int kBlock = std::is_same<Src, SrcXor128>::value ? kDigestBlock : 1;
 #pragma unroll(Src::kHeavy ? 1 : 32)
-            for (int k = 0; k < 32; ++k) hits = hits * kDigestMul + s.step();
+            for (int k = 0; k < 32; k += kBlock) {
+                uint32_t o[kBlock];
+#pragma unroll
+                for (int j = 0; j < kBlock; ++j) o[j] = s.step();
+                hits *= digest_power(kBlock);
+#pragma unroll
+                for (int j = 0; j < kBlock; ++j) hits += o[j] * digest_power(kBlock - 1 - j);
+            }
         } else if (SINK == SINK_QC) {
             uint32_t m = 0, near = ~0u;
             const Lane<Src> before = s;

@@ -56,3 +56,15 @@ def test_a_call_is_not_slower_than_whole(variant, S, n):
     torch, ci = cuda_or_skip()
     chosen, whole = (_written(torch, ci, S, n, segments=k, variant=variant) for k in (None, 1))
     assert chosen < 1.25 * whole, (chosen, whole)
+
+
+def test_digesting_is_not_slower_than_writing():
+    """xor128, one warp per SM: the digest stores nothing."""
+    torch, ci = cuda_or_skip()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    S, n = 32 * sms, 2048
+    st = ci.States(S, seed=1)
+    d = torch.zeros(S, dtype=torch.int64, device="cuda")
+    digest = _us(torch, lambda: st.generate_split(n, sink="digest", out=d, segments=1))
+    written = _written(torch, ci, S, n, segments=1)
+    assert digest < written, (digest, written)
