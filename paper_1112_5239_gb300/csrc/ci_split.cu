@@ -1368,21 +1368,26 @@ uint64_t split_auto(const ci_states_s &h, uint64_t n, int sink, bool captured) {
 
 }  // namespace
 
-ci_status single_call(const ci_states_s &h, uint64_t n, int sink, uint32_t *out, uint64_t *aux, cudaStream_t stream) {
-    const bool captured = stream_capturing(stream);
-    cudaError_t e;
-    const int blocks = narrow_blocks(h, n);
-    const bool whole = captured && !jumps_at_hand(h);
-    if (blocks && !whole) {
-        e = launch_narrow(h, blocks, n, sink, out, aux, stream);
-    } else {
-        const uint64_t K = whole ? 1 : split_auto(h, n, sink, captured);
-        if (K > 1) return split_launch(h, n, sink, out, n, 0, aux, K, stream);
-        e = sink == CI_SINK_QC       ? launch_fused_qc(h, n, aux, stream)
-            : sink == CI_SINK_DIGEST ? launch_digest(h, n, aux, stream)
-                                     : launch_generate(h, n, out, stream);
-    }
+static ci_status launch_status(cudaError_t e) {
     return e == cudaSuccess ? CI_OK : cuda_fail(e, "generation kernel launch");
+}
+
+ci_status single_call(const ci_states_s &h, uint64_t n, int sink, uint32_t *out, uint64_t *aux, cudaStream_t stream) {
+    const int blocks = narrow_blocks(h, n);
+    uint64_t K = blocks ? 1 : split_auto(h, n, sink, false);
+    if (blocks || K > 1) {  // the others run the same captured or not, and are not kept from their launch by the question
+        const bool captured = stream_capturing(stream);
+        if (captured && !jumps_at_hand(h))
+            K = 1;
+        else if (blocks)
+            return launch_status(launch_narrow(h, blocks, n, sink, out, aux, stream));
+        else if (captured)
+            K = split_auto(h, n, sink, true);
+        if (K > 1) return split_launch(h, n, sink, out, n, 0, aux, K, stream);
+    }
+    return launch_status(sink == CI_SINK_QC       ? launch_fused_qc(h, n, aux, stream)
+                         : sink == CI_SINK_DIGEST ? launch_digest(h, n, aux, stream)
+                                                  : launch_generate(h, n, out, stream));
 }
 
 ci_status split_launch(const ci_states_s &hs, uint64_t n, int sink, uint32_t *out, uint64_t ld, uint64_t col0,
