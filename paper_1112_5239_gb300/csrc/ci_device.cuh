@@ -566,8 +566,19 @@ struct TileCfg {
     static constexpr int KT = KT_;
     static constexpr int CH = KT_ / 4;  // 16-byte chunks per tile row
     static constexpr int CACHE = CACHE_;
+    static constexpr bool kBrief = false;
 };
 using TileDefault = TileCfg<32, 0>;
+// For warps that run a few tiles in a launch of some 10 us: the loops with the
+// least code and staging, since their first fetch costs more than conflicts or a
+// longer chain (32 x 8192 digested: 20.5 us, 21.6 with blocks of sixteen; 4096 x
+// 2047 written 24.7, 26.7 with the forms of several strides in one kernel).
+// PITCH: of written_lines.
+template <int PITCH>
+struct TileBrief : TileDefault {
+    static constexpr bool kBrief = true;
+    static constexpr int kPitch = PITCH;
+};
 
 // Index of word `col` of row `row` in a warp's 32 x KT staging tile: 16-byte
 // chunks XOR-swizzled by row so that both the per-lane 16-byte row writes and
@@ -765,8 +776,11 @@ __device__ __forceinline__ uint64_t warp_run(Lane<Src> &s, uint64_t S, uint64_t 
     constexpr int CH = KT / 4;
     const int lane = threadIdx.x & 31;
     if constexpr (SINK == SINK_SCALAR) {
-        written_unaligned<Src::kHeavy ? 1 : 32, TC::CACHE>([&]() { return s.step(); }, S, row0, n, out,
-                                                   ld, col0, tile);
+        auto step = [&]() { return s.step(); };
+        if constexpr (TC::kBrief)
+            written_lines<32, TC::CACHE, TC::kPitch, false>(step, S, row0, n, out, ld, col0, tile);
+        else
+            written_unaligned<Src::kHeavy ? 1 : 32, TC::CACHE>(step, S, row0, n, out, ld, col0, tile);
         return 0;
     }
     const uint64_t nfull = n - n % KT;
@@ -778,7 +792,7 @@ __device__ __forceinline__ uint64_t warp_run(Lane<Src> &s, uint64_t S, uint64_t 
 #pragma unroll(Src::kHeavy ? 1 : 32)
             for (int k = 0; k < 32; ++k) s.step();
         } else if (SINK == SINK_DIGEST) {
-            constexpr int kBlock = std::is_same<Src, SrcXor128>::value ? kDigestBlock : 1;
+            constexpr int kBlock = std::is_same<Src, SrcXor128>::value && !TC::kBrief ? kDigestBlock : 1;
 #pragma unroll(Src::kHeavy ? 1 : 32)
             for (int k = 0; k < 32; k += kBlock) {
                 uint32_t o[kBlock];

@@ -882,10 +882,10 @@ __device__ __forceinline__ void jump_source(SrcXorshift32 &s, uint64_t dist) {
     s.z = v[0];
 }
 
-template <class Src, int SINK>
+template <class Src, int SINK, int PITCH = 16>
 __global__ void __launch_bounds__(32 * kNarrowWarps)
     k_narrow(DevState st, uint64_t n, uint64_t len, uint32_t K, uint32_t *out, uint64_t *aux) {
-    __shared__ uint4 tiles[kNarrowWarps][SINK == SINK_V4 ? 256 : SINK == SINK_SCALAR ? kTileVec : 1];
+    __shared__ uint4 tiles[kNarrowWarps][SINK == SINK_V4 ? 256 : SINK == SINK_SCALAR ? 32 * PITCH : 1];
     __shared__ __align__(16) MatVecScratch scratch[kNarrowWarps];
     __shared__ uint2 ends[kNarrowWarps][32], aggregate[32], all[kNarrowBlocks][32];
     __shared__ uint64_t results[kNarrowWarps][32];
@@ -906,7 +906,7 @@ __global__ void __launch_bounds__(32 * kNarrowWarps)
     if (seg > 0 && seg < K) jump_source(s.src, seg * len);
     const Src start = s.src;
     if (seg > 0) s.slot = s.x = 0;
-    if (seg + 1 < K) warp_run<Src, SINK_NONE, TileDefault>(s, 0, 0, len, nullptr, 0, 0, nullptr);
+    if (seg + 1 < K) warp_run<Src, SINK_NONE, TileBrief<PITCH>>(s, 0, 0, len, nullptr, 0, 0, nullptr);
     const uint2 e = make_uint2(s.slot, s.x);
     ends[bw][lane] = e;
     uint32_t Q, S;
@@ -941,7 +941,7 @@ __global__ void __launch_bounds__(32 * kNarrowWarps)
     uint64_t r = 0;
     if (seg < K) {
         const uint64_t from = seg * len, m = seg + 1 == K ? n - from : len;
-        r = warp_run<Src, SINK, TileDefault>(s, st.S, g * 32, m, out, n, from, tiles[bw]);
+        r = warp_run<Src, SINK, TileBrief<PITCH>>(s, st.S, g * 32, m, out, n, from, tiles[bw]);
         if (SINK == SINK_DIGEST) r *= digest_pow(n - from - m);
         if (seg + 1 == K) s.store(st, l);
     }
@@ -971,7 +971,7 @@ cudaError_t launch_narrow_src(const DevState &st, int sink, int blocks, uint64_t
     cfg.attrs = &cluster;
     cfg.numAttrs = 1;
     auto kern = sink == SINK_V4       ? k_narrow<Src, SINK_V4>
-                : sink == SINK_SCALAR ? k_narrow<Src, SINK_SCALAR>
+                : sink == SINK_SCALAR ? (n % 8 == 0 ? k_narrow<Src, SINK_SCALAR, 17> : k_narrow<Src, SINK_SCALAR>)
                 : sink == SINK_QC     ? k_narrow<Src, SINK_QC>
                                       : k_narrow<Src, SINK_DIGEST>;
     return cudaLaunchKernelEx(&cfg, kern, st, n, len, K, out, aux);
