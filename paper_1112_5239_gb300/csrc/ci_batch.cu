@@ -107,9 +107,12 @@ BatchGeometry batch_geometry(int warps_per_block) {
 }
 
 double kind_cost(uint32_t kind) {
-    // measured ratios of per-output cost (BBS: 11 Barrett squarings per
-    // output; BBS16: 12 32-bit Barrett squarings)
-    return kind == K_BBS ? 40.0 : kind == K_BBS16 ? 8.0 : 1.0;
+    // a unit's time per output in this kernel, 16 warps per SM: xor128 42 ns
+    // digested and 53 written, XORshift 46 and 52, xor64 59 and 69, BBS (residue
+    // form) 852 and 861, Algorithm 5 as printed 336 and 294.  (The order is not
+    // sensitive to them: 40 : 8 and 14 : 3 are within 0.5 % on 300 to 2000
+    // requests.)
+    return kind == K_BBS ? 18.0 : kind == K_BBS16 ? 6.5 : 1.0;
 }
 
 BatchTask make_task(const ci_states_s &h, uint64_t n, int sink_abi, uint32_t *out, uint64_t *aux, uint64_t ld,
