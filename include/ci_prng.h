@@ -189,12 +189,14 @@ ci_status ci_generate(ci_states states, uint64_t n_per_stream, uint32_t *out_dev
  * residues of the two factors of M (62-bit Barrett squares where an imported
  * modulus has a factor outside (2^30, 2^31)).  The stream's two
  * combination arrays are comb[sel1] and comb[8 + sel2] with sel1 = v & 7,
- * sel2 = (v >> 3) & 7 of its BBS seed v.  A CI_VAR_BBS state is run as
- * time segments, as ci_generate_split does, with identical results, unless
- * its streams alone fill about ten waves of resident warps; so is a
- * CI_VAR_BBS16 state of at most one warp group (32 streams) per SM, within
- * the one call.  That form allocates a stream-ordered workspace.  Errors as ci_generate
- * (CI_E_STATE for an xor handle). */
+ * sel2 = (v >> 3) & 7 of its BBS seed v.  A call long enough that it is
+ * faster so is run as time segments, as ci_generate_split does, with identical
+ * results: for CI_VAR_BBS from some 170 iterations of a few streams to some
+ * 1000 of 2^16, unless the streams alone fill about ten waves of resident
+ * warps; for CI_VAR_BBS16 states of at most one warp group (32 streams) per SM
+ * from some 900 to 2000, within the one call.  That form allocates a
+ * stream-ordered workspace.  Errors as ci_generate (CI_E_STATE for an xor
+ * handle). */
 ci_status ci_generate_bbs(ci_states states, uint64_t n_per_stream, uint32_t *out_dev,
                           uint64_t out_capacity_u32, void *cuda_stream);
 
@@ -545,17 +547,18 @@ ci_status ci_naive_generate(void *state_dev, uint64_t n_streams, uint64_t n_per_
  * ci_generate_bbs for CI_SINK_WRITTEN, ci_generate_fused_qc for CI_SINK_QC,
  * ci_generate_digest for CI_SINK_DIGEST).  For states with few streams and
  * long lengths, whose sequential chains leave most of the GPU idle.  (Those
- * single-call entry points split states on their own: written CI_VAR_BBS
- * outputs unless the state fills about ten waves of resident warps, BBS
- * consumer sinks likewise up to 2^29 outputs per call and under about two
- * waves above that, xor-like states of at most one warp
- * group per SM in calls of at least 2048 iterations (up to 16384 in one launch
- * of their own), and CI_VAR_BBS16 states of at most one warp group per SM.)
+ * single-call entry points split states on their own: CI_VAR_BBS and
+ * CI_VAR_BBS16 as ci_generate_bbs describes, their consumer sinks likewise
+ * (CI_VAR_BBS above 2^29 outputs per call only under about two waves), xor-like
+ * states of at most one warp group per SM in calls of more than 16384
+ * iterations, shorter ones in one launch of clusters as ci_generate does.  A
+ * call captured into a graph before the process has jumped on that device runs
+ * unsplit.)
  * Method: each segment's own generator is jumped ahead (xor-likes: GF(2)
  * matrix powers of their step; BBS: x <- x^(2^(11 k len)) mod M, the exponent
  * reduced by the orders of p and q, or by Carmichael's lambda of M where an
- * imported modulus or state needs it), the segments run from a zero mixing state, a per-warp scan restores
- * their true starts from the linearity of Algorithm 4/5's mixing and Eq.
+ * imported modulus or state needs it), the segments run from a zero mixing
+ * state, a per-warp scan restores their true starts from the linearity of Algorithm 4/5's mixing and Eq.
  * (Oplus) over the lanes, and the segments run again from those starts into
  * the sink (written BBS-source outputs are corrected in place instead: the
  * homogeneous part is XORed in, two shuffles per output; their consumer sinks

@@ -651,7 +651,7 @@ __device__ __forceinline__ void written_short(Step step, uint64_t S, uint64_t ro
 // of a tile's 32 steps are unrolled.
 // (50001 x 1001 XORshift outputs: the word-wise form this replaces, a row per
 // warp-wide store, issued 34 instructions per step of a warp, 20 of them for
-// the stores, and took 82 us; now 53.)
+// the stores, and took 82 us; now 52.)
 // Banks: the lanes of one step write 32 different ones when ld is odd, 16 when
 // it is 2 mod 4.  When ld is a multiple of 4 (in a buffer that is not 16-byte
 // aligned) the rows' phases are equal mod 4: after up to three steps every row

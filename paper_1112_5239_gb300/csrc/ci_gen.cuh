@@ -23,7 +23,7 @@ namespace ci {
 // block; a state of one wave takes smaller blocks as far as the SMs' 32 blocks
 // each hold it, since idle warps of larger ones leave schedulers unused (2^17 x
 // 1024 digested: 82 us, 92 with one or two of a block's four warps at work;
-// 50001 x 1001 XORshift 53, 57).
+// 50001 x 1001 XORshift 53, 57 then).
 // The squaring sources (kHeavy) nearly fill a scheduler with each warp: one-warp
 // blocks up to two warps per scheduler (10^4 x 1024 of Algorithm 5 as printed:
 // 94 us, 139 spread), beyond them a wave is spread over all resident blocks so

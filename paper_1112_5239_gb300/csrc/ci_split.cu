@@ -1002,8 +1002,9 @@ constexpr uint64_t kOneLaunchGroupsPerSm = CI_ONE_LAUNCH_GROUPS_PER_SM;
 // Instantiated per source and sink, with at most 64 registers (4 blocks of 8
 // warps per SM): the all-source batched kernel needs 128, which held the
 // BBS segments to 16 resident warps per SM.  BBS segments ask for 3 blocks, 80
-// registers: the residue form's constants fit without spills, and its two
-// independent chains per lane fill the pipes from 24 warps per SM on
+// registers: the residue form's constants fit without spills (k_split_run_fix,
+// with the fix-ups beside them, spills 8 bytes, 24 for unaligned rows), and its
+// two independent chains per lane fill the pipes from 24 warps per SM on
 // (2^16 x 4096: 3.28 ms; 3.50 with 4 blocks, 3.95 with 5, 3.39 with 2;
 // 5.38 in the 62-bit form with 5).  Segments of Algorithm 5 as printed (eight
 // generators per lane, 118 registers in the single-call kernel) ask for 2
