@@ -285,7 +285,8 @@ cudaError_t bg_launch(uint64_t n_msgs, uint64_t L, const uint64_t *a, const uint
     auto kern = vec ? k_bg<kDecrypt, true> : k_bg<kDecrypt, false>;
     static const int per_sm[2] = {resident_blocks_per_sm(k_bg<kDecrypt, false>, kBgWarps * 32, 0),
                                   resident_blocks_per_sm(k_bg<kDecrypt, true>, kBgWarps * 32, 0)};
-    const GenGrid gg = gen_grid((n_msgs + 31) / 32, kBgWarps, (uint64_t)sm_count() * per_sm[vec], true);
+    // a wave is always spread (22704 x 391 encryption: 51.6 us, 53.3 in one-warp blocks)
+    const GenGrid gg = gen_grid((n_msgs + 31) / 32, kBgWarps, (uint64_t)sm_count() * per_sm[vec], 0);
     kern<<<gg.grid, gg.warps * 32, 0, stream>>>(n_msgs, L, a, b, S0, y_in, in, out, y_out, n_rejected, gg.in_order);
     return cudaGetLastError();
 }

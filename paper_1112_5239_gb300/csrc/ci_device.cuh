@@ -610,18 +610,16 @@ __device__ __forceinline__ void store_words(uint32_t *p, const uint4 &v, int lo,
     }
 }
 
-// Rows of up to 64 words with nothing between them (ld == n): the group's rows
-// are one span of the output, staged at a pitch of 65 words (32 banks a step)
-// and stored as that span, 32 consecutive words per warp-wide store.
-constexpr uint64_t kShortRows = 64;
-constexpr int kShortPitch = 65;
-template <class Step>
+// Rows of up to kPitch words with nothing between them (ld == n): the group's
+// rows are one span of the output, staged at an odd pitch (32 banks a step) and
+// stored as that span, 32 consecutive words per warp-wide store.
+template <int kPitch, class Step>
 __device__ __forceinline__ void written_short(Step step, uint64_t S, uint64_t row0, uint32_t n, uint32_t *out,
                                               uint4 *tile) {
     const uint32_t lane = threadIdx.x & 31;
     uint32_t *stage = reinterpret_cast<uint32_t *>(tile);
 #pragma unroll 1
-    for (uint32_t i = 0; i < n; ++i) stage[lane * kShortPitch + i] = step();
+    for (uint32_t i = 0; i < n; ++i) stage[lane * kPitch + i] = step();
     __syncwarp();
     const uint32_t rows = S - row0 < 32 ? (uint32_t)(S - row0) : 32u, words = rows * n;
     const uint32_t dr = 32 / n, dc = 32 % n;
@@ -629,7 +627,7 @@ __device__ __forceinline__ void written_short(Step step, uint64_t S, uint64_t ro
     uint32_t r = lane / n, c = lane % n;
 #pragma unroll 4
     for (uint32_t i = lane; i < words; i += 32) {
-        dst[i] = stage[r * kShortPitch + c];
+        dst[i] = stage[r * kPitch + c];
         r += dr;
         c += dc;
         if (c >= n) {
@@ -756,15 +754,21 @@ __device__ __forceinline__ void written_lines(Step step, uint64_t S, uint64_t ro
 template <int kUnroll, int CACHE, class Step>
 __device__ __forceinline__ void written_unaligned(Step step, uint64_t S, uint64_t row0, uint64_t n, uint32_t *out,
                                                   uint64_t ld, uint64_t col0, uint4 *tile) {
-    if (n <= kShortRows && ld == n)
-        written_short(step, S, row0, (uint32_t)n, out, tile);
-    else if constexpr (kUnroll == 1)  // a step takes far longer than its store
-        written_lines<kUnroll, CACHE, 0, false>(step, S, row0, n, out, ld, col0, tile);
-    else if (ld % 4 == 0)
-        written_lines<kUnroll, CACHE, 0, true>(step, S, row0, n, out, ld, col0, tile);
-    else
+    constexpr bool kLong = kUnroll == 1;  // a step takes far longer than its store: the least code and staging
+    constexpr int kShort = kLong ? 63 : 65;
+    if (n <= kShort && ld == n) {
+        written_short<kShort>(step, S, row0, (uint32_t)n, out, tile);
+    } else if constexpr (kLong) {
         written_lines<kUnroll, CACHE, 16, false>(step, S, row0, n, out, ld, col0, tile);
+    } else {
+        if (ld % 4 == 0)
+            written_lines<kUnroll, CACHE, 0, true>(step, S, row0, n, out, ld, col0, tile);
+        else
+            written_lines<kUnroll, CACHE, 16, false>(step, S, row0, n, out, ld, col0, tile);
+    }
 }
+template <class Src>  // of a source's unaligned rows
+constexpr int kScalarTile = Src::kHeavy ? 32 * 16 : kTileVec;
 
 // Runs n steps of a loaded lane into the sink; returns the lane's
 // quarter-circle hits or the Horner digest of these outputs (0 for the others).

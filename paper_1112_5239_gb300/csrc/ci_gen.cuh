@@ -28,15 +28,17 @@ namespace ci {
 // blocks up to two warps per scheduler (10^4 x 1024 of Algorithm 5 as printed:
 // 94 us, 139 spread), beyond them a wave is spread over all resident blocks so
 // that every SM gets its share (2^16 x 1024: 261 us, 270 in one-warp blocks).
+constexpr uint64_t kNeverSpread = 1ull << 32;
 struct GenGrid {
     unsigned grid, warps;  // blocks; warps per block
     uint32_t in_order;     // the same if blocks hold consecutive groups, else 0: warp w of block b takes w * grid + b
 };
-inline GenGrid gen_grid(uint64_t groups, int W, uint64_t resident_blocks, bool heavy) {
+// `spread_from`: one-wave states of more groups per SM are spread.
+inline GenGrid gen_grid(uint64_t groups, int W, uint64_t resident_blocks, uint64_t spread_from) {
     const uint64_t sms = (uint64_t)sm_count();
     unsigned warps = (unsigned)W;
     if (groups <= resident_blocks * W) {
-        if (heavy && groups > 8 * sms)
+        if (groups > spread_from * sms)
             return {(unsigned)(groups < resident_blocks ? groups : resident_blocks), warps, 0u};
         const uint64_t w = (groups + 32 * sms - 1) / (32 * sms);
         if (w < (uint64_t)W) warps = (unsigned)w;
@@ -55,14 +57,14 @@ int resident_blocks_per_sm(Kernel kern, int threads, size_t smem) {
 }
 
 // Written sinks stage a 32 x KT tile per warp in dynamic shared memory.
-template <int SINK, class TC>
-constexpr int kTileVecs = SINK >= dev::SINK_QC ? 0 : SINK == dev::SINK_SCALAR ? dev::kTileVec : TC::KT * 8;
+template <class Src, int SINK, class TC>
+constexpr int kTileVecs = SINK >= dev::SINK_QC ? 0 : SINK == dev::SINK_SCALAR ? dev::kScalarTile<Src> : TC::KT * 8;
 template <class Src, int SINK, int W, class TC>
 __global__ void __launch_bounds__(W * 32) k_generate(DevState st, uint64_t n, uint32_t in_order, uint32_t *out,
                                                      uint64_t *counts) {
     extern __shared__ uint4 dyn_tiles[];
     const int w = threadIdx.x >> 5;
-    uint4 *tile = dyn_tiles + w * kTileVecs<SINK, TC>;
+    uint4 *tile = dyn_tiles + w * kTileVecs<Src, SINK, TC>;
     const uint64_t g = warp_group(in_order);
     if (g < st.P / 32) dev::warp_task<Src, SINK, TC>(st, g, n, out, n, 0, counts, tile);
 }
@@ -139,7 +141,7 @@ static cudaError_t launch_gen_tma(const DevState &st, uint64_t n, uint32_t *out,
     static std::atomic<uint64_t> smem_set{0};
     allow_smem(kern, smem(W), smem_set);
     static const int per_sm = resident_blocks_per_sm(kern, W * 32, smem(W));
-    const GenGrid gg = gen_grid(st.P / 32, W, (uint64_t)sm_count() * per_sm, false);
+    const GenGrid gg = gen_grid(st.P / 32, W, (uint64_t)sm_count() * per_sm, kNeverSpread);
     *used = true;
     kern<<<gg.grid, gg.warps * 32, smem(gg.warps), stream>>>(st, n, gg.in_order, map);
     return cudaGetLastError();
@@ -149,11 +151,11 @@ template <class Src, int SINK, int W, class TC>
 static cudaError_t launch_gen_t(const DevState &st, uint64_t n, uint32_t *out, uint64_t *counts,
                                 cudaStream_t stream) {
     auto kern = k_generate<Src, SINK, W, TC>;
-    constexpr size_t tile = kTileVecs<SINK, TC> * sizeof(uint4);
+    constexpr size_t tile = kTileVecs<Src, SINK, TC> * sizeof(uint4);
     static std::atomic<uint64_t> smem_set{0};
     allow_smem(kern, W * tile, smem_set);
     static const int per_sm = resident_blocks_per_sm(kern, W * 32, W * tile);
-    const GenGrid gg = gen_grid(st.P / 32, W, (uint64_t)sm_count() * per_sm, Src::kHeavy);
+    const GenGrid gg = gen_grid(st.P / 32, W, (uint64_t)sm_count() * per_sm, Src::kHeavy ? 8 : kNeverSpread);
     kern<<<gg.grid, gg.warps * 32, gg.warps * tile, stream>>>(st, n, gg.in_order, out, counts);
     return cudaGetLastError();
 }

@@ -219,8 +219,8 @@ __host__ __device__ __forceinline__ T lcm(T a, T b) {
 // Carmichael's lambda of M = a b for any odd a, b in [3, 2^32): the least
 // common multiple of r^(k-1) (r - 1) over the prime powers r^k of M, found by
 // trial division.  For every x and every E with 2^E >= 62, x^(2^E) = x^e mod M
-// with e = (2^E mod lambda) + lambda, whether x is a unit or not: both
-// exponents reach the exponent of every prime power of M < 2^62.
+// with e = 2^E mod lambda, plus lambda where that is below 62, whether x is a
+// unit or not: both exponents reach that of every prime power of M < 2^62.
 __host__ __device__ inline uint64_t carmichael(uint32_t a, uint32_t b) {
     uint64_t lam = 1;
     while (a > 1 || b > 1) {
@@ -244,7 +244,7 @@ __host__ __device__ inline uint64_t carmichael(uint32_t a, uint32_t b) {
 }
 
 // Carmichael's lambda of any M in [2, 2^16) (even ones and prime powers
-// too); the exponents as above, for 2^E >= 15.  Twice lambda where 8 but not
+// too); the exponents as above, with 15 for 62.  Twice lambda where 8 but not
 // 16 divides M: lambda(8) = 2 is below the exponent of its 2^3, the one case.
 // The product of two primes, all that a seeded state holds, leaves the search
 // at its smaller factor, and the lanes of a warp go on together.

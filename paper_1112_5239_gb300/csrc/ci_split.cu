@@ -251,8 +251,9 @@ cudaError_t ensure_jump_tables(cudaStream_t stream) {
 
 // ------------------------------------------------ BBS jump
 // x <- x^(2^E) mod M with E = 11 * dist squarings, through the exponent
-// (2^E mod lambda) + lambda with lambda from k_split_constants: Carmichael's
-// lambda of M, which holds for every x, or a multiple of the order of x.
+// 2^E mod lambda, plus lambda where that is below 62, with lambda from
+// k_split_constants: Carmichael's lambda of M, which holds for every x, or a
+// multiple of the order of x.
 // a^e mod M for a < M, left to right over 2-bit windows of e: two squarings
 // and one product by a^w (by 1 for w = 0) per window, the same work in every
 // lane whatever its exponent bits.
@@ -276,7 +277,8 @@ __device__ __forceinline__ uint64_t bbs_jump(uint64_t y, uint64_t M, uint64_t mu
     Barrett62 L;
     L.set(lam, lam_mu);
     // 2^squarings mod lam by square-and-multiply on the exponent's bits
-    const uint64_t e = pow_mod(L, 2 % lam, squarings) + lam;
+    uint64_t e = pow_mod(L, 2 % lam, squarings);
+    if (e < 62) e += lam;
     Barrett62 B;
     B.set(M, mu);
     return pow_mod(B, y, e);
@@ -384,10 +386,12 @@ __device__ __forceinline__ uint64_t bbs_jump_lane(const DevState &src, uint64_t 
     const uint64_t P = src.P;
     CrtModulus C;
     const uint32_t *jump = crt + kCrtWords * P + l;
-    if (crt_load(src, l, crt, C) && jump[2 * P] && jump[3 * P]) {
-        const Mont31 Mp(C.P.p, jump[2 * P]), Mq(C.Q.p, jump[3 * P]);
-        return C.value(Mp.from(squarings_m(C.P.p, Mp.one, jump[0], squarings)),
-                       Mq.from(squarings_m(C.Q.p, Mq.one, jump[P], squarings)));
+    // all loaded before the test: one round trip
+    const uint32_t yp = jump[0], yq = jump[P], one_p = jump[2 * P], one_q = jump[3 * P];
+    if (crt_load(src, l, crt, C) & (one_p != 0u) & (one_q != 0u)) {
+        const Mont31 Mp(C.P.p, one_p), Mq(C.Q.p, one_q);
+        return C.value(Mp.from(squarings_m(C.P.p, one_p, yp, squarings)),
+                       Mq.from(squarings_m(C.Q.p, one_q, yq, squarings)));
     }
     return bbs_jump(src.u64[G_Y * P + l], src.u64[G_M * P + l], src.u64[G_MU * P + l], lam[l], lam[P + l], squarings);
 }
@@ -440,7 +444,8 @@ __global__ void __launch_bounds__(256) k_split_setup(DevState src, SegSpace seg,
         if (variant == CI_VAR_BBS16) {
             for (int g = 0; g < 8; ++g) {  // x <- x^(2^(c_g dist)) mod M, for any x and M (carmichael16)
                 const uint32_t M = src.u32[(F_M16 + g) * src.P + l], lam = lam16[(uint64_t)g * src.P + l];
-                const uint32_t e = pow_mod16(2, c_bbs16_squarings[g] * dist, lam) + lam;
+                uint32_t e = pow_mod16(2, c_bbs16_squarings[g] * dist, lam);
+                if (e < 15) e += lam;
                 d.u32[(F_Y16 + g) * src.P + l] = pow_mod16(src.u32[(F_Y16 + g) * src.P + l], e, M);
             }
         } else if (variant == CI_VAR_BBS) {
@@ -1019,7 +1024,7 @@ __global__ void __launch_bounds__(256, split_min_blocks<Src>()) k_split_run(SegS
                                                    uint32_t k_end, uint32_t K, uint64_t len, uint64_t len_last,
                                                    uint64_t groups, uint32_t *out, uint64_t ld, uint64_t col0,
                                                    uint64_t *aux, const uint32_t *crt) {
-    __shared__ uint4 tiles[8][SINK == SINK_SCALAR ? kTileVec : 256];
+    __shared__ uint4 tiles[8][SINK == SINK_SCALAR ? kScalarTile<Src> : 256];
     uint4 *tile = tiles[threadIdx.x >> 5];
     const uint64_t units = (uint64_t)(k_end - k_begin) * groups;
     // warp w of block b starts at unit w * gridDim.x + b: a partial last
@@ -1086,7 +1091,7 @@ __global__ void __launch_bounds__(256, split_min_blocks<Src>()) k_split_run_fix(
                                                        uint64_t len_last, uint64_t groups, uint32_t *out, uint64_t ld,
                                                        uint64_t col0, uint2 *starts, uint32_t *events,
                                                        unsigned long long *next_unit, const uint32_t *crt) {
-    __shared__ uint4 tiles[8][SINK == SINK_SCALAR ? kTileVec : 256];
+    __shared__ uint4 tiles[8][SINK == SINK_SCALAR ? kScalarTile<Src> : 256];
     uint4 *tile = tiles[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const DevState s0 = seg.at(0);
