@@ -442,6 +442,7 @@ __global__ void __launch_bounds__(256) k_split_setup(DevState src, SegSpace seg,
         d.u32[F_SLOT * src.P + l] = 0;
         const uint64_t dist = k * len;
         if (variant == CI_VAR_BBS16) {
+#pragma unroll  // (rolled: 1000 x 65536 74 us instead of 56, and 2^16 BBS streams 95 instead of 84)
             for (int g = 0; g < 8; ++g) {  // x <- x^(2^(c_g dist)) mod M, for any x and M (carmichael16)
                 const uint32_t M = src.u32[(F_M16 + g) * src.P + l], lam = lam16[(uint64_t)g * src.P + l];
                 uint32_t e = pow_mod16(2, c_bbs16_squarings[g] * dist, lam);
