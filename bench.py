@@ -57,7 +57,7 @@ def parse_args():
     ap.add_argument("--requests", type=int, default=10_000, help="batched suite: number of requests")
     ap.add_argument("--serving-requests", type=int, default=20_000, help="serving suite: requests per rate")
     ap.add_argument("--profile", choices=["written", "fused", "fused_xor64", "bbs", "bbs_split", "bbs_split_1g", "bbs16",
-                                          "batched",
+                                          "batched", "written_4", "written_8", "short", "unaligned", "narrow",
                                           "bg", "bg_dec", "naive"],
                     default=None,
                     help="small case for ncu: autotune, 2 warm-up launches, then 1 launch of one kernel inside "
@@ -67,7 +67,9 @@ def parse_args():
 
 def run_profile_case(kind: str) -> None:
     """Small case for profiler captures: 2^19 streams x 256 written (512 MiB,
-    larger than L2), 2^19 x 4096 fused (xor128 or xor64), 2^16 x 1024 BBS
+    larger than L2; written_4 and written_8: TMA tiles with that many warps per
+    block), short rows (10^6 x 100), unaligned rows (XORshift 50001 x 1001), a
+    narrow call (4096 x 1024), 2^19 x 4096 fused (xor128 or xor64), 2^16 x 1024 BBS
     written (256 MiB; one unsplit launch), the benchmark's BBS call (2^16 x
     16384 written, 4 GiB, run as time segments) or the same on 2^16 x 4096
     (1 GiB), Algorithm 5 as printed or
@@ -84,10 +86,20 @@ def run_profile_case(kind: str) -> None:
 
     torch.cuda.set_device(0)
     ci.autotune()  # the launch shapes the benchmark uses
-    if kind == "written":
+    if kind.startswith("written"):
+        if kind != "written":
+            table = ci.tune_table()
+            table["xor128/written"].update(warps_per_block=int(kind[-1]), tile_depth=32, cache_policy=2)
+            ci.set_tune_table(table)
         st = ci.States(1 << 19, seed=SEED_MAIN)
         out = torch.empty((1 << 19, CHUNK), dtype=torch.int32, device="cuda")
         run = lambda: st.generate(CHUNK, out=out)  # noqa: E731
+    elif kind in ("short", "unaligned", "narrow"):
+        S, n, xl = {"short": (10**6, 100, "xor128"), "unaligned": (50001, 1001, "xorshift32"),
+                    "narrow": (4096, 1024, "xor128")}[kind]
+        st = ci.States(S, seed=SEED_MAIN, xl=xl)
+        out = torch.empty((S, n), dtype=torch.int32, device="cuda")
+        run = lambda: st.generate(n, out=out)  # noqa: E731
     elif kind in ("fused", "fused_xor64"):
         st = ci.States(1 << 19, seed=SEED_MAIN, xl="xor64" if kind == "fused_xor64" else "xor128")
         counts = torch.zeros(1 << 19, dtype=torch.int64, device="cuda")
